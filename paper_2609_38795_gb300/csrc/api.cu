@@ -229,9 +229,9 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, bool two_rows = 
 // fp32 inputs run tf32 products, which take K-major operands only: the head is then read from
 // a transposed copy W^T [V, d] placed in the workspace.
 // Forward-type workspace: `fields` partial statistics per row and part, one fp64 pair per
-// anchor, and W^T for fp32 inputs.
+// anchor and the merge kernel's ticket, and W^T for fp32 inputs.
 struct FwdLayout {
-  size_t part_off, anchor_off, wt_off, total;
+  size_t part_off, anchor_off, ticket_off, wt_off, total;
 };
 
 FwdLayout fwd_layout(const alr_params* p, int sms, int fields = alr::kPFields,
@@ -240,7 +240,8 @@ FwdLayout fwd_layout(const alr_params* p, int sms, int fields = alr::kPFields,
   FwdLayout L{};
   L.part_off = 0;
   L.anchor_off = round_up(size_t(fields) * P.n_parts * size_t(P.N) * sizeof(float), 1024);
-  L.wt_off = L.anchor_off + round_up(2 * sizeof(double) * size_t(P.N / P.B), 1024);
+  L.ticket_off = L.anchor_off + 2 * sizeof(double) * size_t(P.N / P.B);
+  L.wt_off = round_up(L.ticket_off + 16, 1024);
   L.total = L.wt_off;
   if (p->dtype == ALR_F32) L.total += round_up(size_t(p->V) * p->d * sizeof(float), 1024);
   return L;
@@ -427,6 +428,7 @@ int fwd_impl(const alr_params* p, const void* Hd, const void* Ht, const void* W,
   alr::LossArgs args{};
   args.plan = loss_plan(p, info.sms, false);
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
+  args.ticket = reinterpret_cast<unsigned*>(ws + lay.ticket_off);
   args.corpus_tok = p->mode != ALR_MODE_ALR ? corpus_tok : nullptr;
   args.lam = p->lambda;
   args.withhold_first_stage = g_withhold_next.exchange(0);
@@ -453,11 +455,8 @@ int fwd_impl(const alr_params* p, const void* Hd, const void* Ht, const void* W,
   e = alr::launch_combine(args.plan, args.part, p->mode, p->gamma, row_mask, args.corpus_tok,
                           out->loss_row, out->ent_row, out->lse_d, out->lse_t, out->argmax_d,
                           out->argmax_t, out->gap_d, out->gap_t, out->logp_x, out->weight, anchor,
-                          s);
+                          args.ticket, p->lambda, out->loss_total, out->weight_sum, out->wl_sum, s);
   if (e != cudaSuccess) return cuda_fail(e, "combine launch");
-  e = alr::launch_finalize(anchor, int(p->N / p->B), p->lambda, out->loss_total, out->weight_sum,
-                          out->wl_sum, s);
-  if (e != cudaSuccess) return cuda_fail(e, "finalize launch");
   return ALR_OK;
 }
 
@@ -896,6 +895,7 @@ int topk_fwd_impl(const alr_params* p, const void* Hd, const void* W, const int3
   alr::LossArgs args{};
   args.plan = loss_plan(p, info.sms, false, true);
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
+  args.ticket = reinterpret_cast<unsigned*>(ws + lay.ticket_off);
   args.top_idx = top_idx;
   args.zd_out = Zd;
   args.zd_ref = Zd_ref;
@@ -912,11 +912,9 @@ int topk_fwd_impl(const alr_params* p, const void* Hd, const void* W, const int3
   double* anchor = reinterpret_cast<double*>(ws + lay.anchor_off);
   e = alr::launch_topk_combine(args.plan, args.part, top_prob, tail, row_mask, weight_in, p->gamma,
                                out->loss_row, out->lse_d, out->tail_q, out->argmax_d, out->gap_d,
-                               out->weight, anchor, s);
+                               out->weight, anchor, args.ticket, p->lambda, out->loss_total,
+                               out->weight_sum, out->wl_sum, s);
   if (e != cudaSuccess) return cuda_fail(e, "top-k combine launch");
-  e = alr::launch_finalize(anchor, int(p->N / p->B), p->lambda, out->loss_total, out->weight_sum,
-                          out->wl_sum, s);
-  if (e != cudaSuccess) return cuda_fail(e, "finalize launch");
   return ALR_OK;
 }
 

@@ -30,16 +30,14 @@ struct LossPlan {
 // Partial statistics of one row over the columns of one vocabulary split seen by one
 // epilogue thread (structure of arrays, field-major: part[f * n_parts * N + part * N + row]).
 enum PartField {
-  kPMd = 0,   // running max of z_d
+  kPMd = 0,   // max of z_d
   kPSd,       // sum exp(z_d - m_d)
-  kPMt,       // running max of z_t
+  kPMt,       // max of z_t
   kPSt,       // sum exp(z_t - m_t)
   kPU,        // sum exp(z_t - m_t) * (z_d - m_d)
   kPW,        // sum exp(z_t - m_t) * (z_t - m_t)
-  kPBd,       // best z_d
-  kPId,       // its index (int bits)
+  kPId,       // index of the maximum of z_d (int bits)
   kPSecd,     // second-best z_d (any other index)
-  kPBt,
   kPIt,
   kPSect,
   kPZx,       // z_t at the corpus token if it lies in the split, else NaN
@@ -53,18 +51,17 @@ constexpr int kTopK = 8;
 
 // Partial record of the label readout: log-sum-exp state, the k best target logits with their
 // token ids, z_t at the corpus token.
-// kRSLo: the rounding error of the sum kRS (the sum is kRS + kRSLo); kRR: the exponent
-// residual r of the reference kRM (every summed exponential carries the factor 2^r).
+// kRSLo: the rounding error of the sum kRS (the sum is kRS + kRSLo).
 enum ReadoutField {
-  kRM = 0, kRS, kRTop, kRIdx = kRTop + kTopK, kRZx = kRIdx + kTopK, kRSLo, kRR, kRFields
+  kRM = 0, kRS, kRTop, kRIdx = kRTop + kTopK, kRZx = kRIdx + kTopK, kRSLo, kRFields
 };
 
 // Partial record of the top-k loss forward: log-sum-exp state and greedy top-2 of z_d, and
 // z_d at the row's k label tokens (NaN where the token is outside the part's columns).
-// kKSLo: the rounding error of the sum kKS; kKSIn: the part of kKS that the row's label
-// tokens contributed (the same rounded terms); kKR: the exponent residual of kKM.
+// kKM: the maximum; kKSLo: the rounding error of the sum kKS; kKSIn: the part of kKS that the
+// row's label tokens contributed (the same rounded terms).
 enum TopkField {
-  kKM = 0, kKS, kKBest, kKIdx, kKSec, kKZ, kKSLo = kKZ + kTopK, kKSIn, kKR, kKFields
+  kKM = 0, kKS, kKIdx, kKSec, kKZ, kKSLo = kKZ + kTopK, kKSIn, kKFields
 };
 
 // What one launch of the fused loss kernel computes.
@@ -81,6 +78,7 @@ enum LossMode {
 struct LossArgs {
   LossPlan plan;
   float* part;                // forward: partial statistics
+  unsigned* ticket;           // forward: cleared for the merge kernel after this one (nullable)
   const int32_t* corpus_tok;  // forward: nullable
   void* G;                    // backward: logit gradient [N, V] (element type of the inputs)
   const float* lse_d;         // backward
@@ -143,13 +141,15 @@ size_t plain_gemm_smem_bytes(int dtype);
 cudaError_t launch_gather(const void* feat, int S, int L, int d, int elem_bytes,
                           const int32_t* seq, const int32_t* pos, const int32_t* valid_len,
                           int A, int B, void* out, float* row_valid, cudaStream_t s);
+// Merge of the partial records (combine_kernels.cu).  block_part: two doubles per anchor at most;
+// ticket: cleared by the fused kernel before.  loss_total, weight_sum and wl_sum (nullable) are
+// the batch sums of Eq. 1.
 cudaError_t launch_combine(const LossPlan& plan, const float* part, int mode, float gamma,
                            const float* row_mask, const int32_t* corpus_tok, float* loss_row,
                            float* ent_row, float* lse_d, float* lse_t, int32_t* argmax_d,
                            int32_t* argmax_t, float* gap_d, float* gap_t, float* logp_x,
-                           float* weight, double* anchor_part, cudaStream_t s);
-cudaError_t launch_finalize(const double* anchor_part, int A, float lam, float* loss_total,
-                            float* weight_sum, float* wl_sum, cudaStream_t s);
+                           float* weight, double* block_part, unsigned* ticket, float lam,
+                           float* loss_total, float* weight_sum, float* wl_sum, cudaStream_t s);
 // loss_total = lambda * wl_sum / weight_sum (0 when weight_sum = 0), from reduced sums.
 cudaError_t launch_loss_from_sums(const float* wl_sum, const float* weight_sum, float lam,
                                   float* loss_total, cudaStream_t s);
@@ -161,7 +161,9 @@ cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const f
                                 const float* tail, const float* row_mask, const float* weight_in,
                                 float gamma, float* loss_row, float* lse_d, float* tail_q,
                                 int32_t* argmax_d, float* gap_d, float* weight,
-                                double* anchor_part, cudaStream_t s);
+                                double* block_part, unsigned* ticket, float lam,
+                                float* loss_total, float* weight_sum, float* wl_sum,
+                                cudaStream_t s);
 // G = lambda omega_r / sum omega (exp(z_d - lse_d) - exp(z_t - lse_t)) from kept logits
 // (dtype 0: fp16 values plus the group references zd_ref / zt_ref [ceil(V / 16), N];
 // dtype 1: fp32, references unused) into G [N, V] (bf16 / fp32); G may be zd itself.

@@ -169,12 +169,6 @@ ALR_DEV void sum2_scaled(float& s, float& c, float sc, float x) {
   c = fmaf(c, sc, e);
 }
 
-// The exponent every column gets relative to the reference m is fma(z, log2 e, -m log2 e),
-// which at z = m is not 0 but the rounding residual of m log2 e (exactly representable, up to
-// ~4e-6 at |m| ~ 40): every exponential summed against m carries the factor 2^r.  The merge
-// divides it out, so that log S and the log-probabilities taken from it keep their precision.
-ALR_DEV float exp_residual(float m) { return fmaf(m, kLog2e, -m * kLog2e); }
-
 // Online log-sum-exp: move the reference from m to max(m, cm) and add the sub-chunk's
 // exp(z - ref) (masked -inf columns add 0) to the compensated sum (s, c).  Even and odd
 // columns are summed in the two lanes of packed registers; each lane's exponential equals the
@@ -511,6 +505,7 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
     }
     mbar_init(drain_bar, 1);
     *abort_word = 0;
+    if (blockIdx.x == 0 && args.ticket != nullptr) *args.ticket = 0u;
     fence_mbar_init();
   }
   if (threadIdx.x == 32) {
@@ -897,10 +892,8 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
           o[kPStLo * fs] = st.c_t;
           o[kPU * fs] = st.u;
           o[kPW * fs] = st.w;
-          o[kPBd * fs] = st.best_d;
           o[kPId * fs] = __int_as_float(st.i_d);
           o[kPSecd * fs] = st.sec_d;
-          o[kPBt * fs] = st.best_t;
           o[kPIt * fs] = __int_as_float(st.i_t);
           o[kPSect * fs] = st.sec_t;
           o[kPZx * fs] = st.zx;
@@ -908,7 +901,6 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
           o[kRM * fs] = m;
           o[kRS * fs] = s;
           o[kRSLo * fs] = sc;
-          o[kRR * fs] = exp_residual(m);
 #pragma unroll
           for (int i = 0; i < kTopK; ++i) {
             o[(kRTop + i) * fs] = tk[i];
@@ -920,8 +912,6 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
           o[kKS * fs] = s;
           o[kKSLo * fs] = sc;
           o[kKSIn * fs] = s_in;
-          o[kKR * fs] = exp_residual(m);
-          o[kKBest * fs] = best;
           o[kKIdx * fs] = __int_as_float(bidx);
           o[kKSec * fs] = sec;
 #pragma unroll

@@ -1,17 +1,13 @@
-// Row-level kernels of the slot-loss path: the IRA gather, block plan, draws and context, the
-// merge of per-split forward statistics into the per-row loss terms and slot weights, the
-// batch reduction of Eq. 1, the accepted-length statistic and the erase-gate weights.  (The
-// logit gradient from kept logits is in grad_kernels.cu.)
-#include <cfloat>
-#include <cuda_fp16.h>
+// Row-level kernels of the slot-loss path: the IRA gather, block plan, draws and context, L from
+// reduced sums, the accepted-length statistic and the erase-gate weights.  (The merge of the
+// forward's partial records is in combine_kernels.cu, the logit gradient from kept logits in
+// grad_kernels.cu.)
 
 #include "kernels.h"
 #include "tc_common.cuh"
 
 namespace alr {
 namespace {
-
-__device__ __forceinline__ float quiet_nan() { return __int_as_float(0x7fc00000); }
 
 // ------------------------------------------------------------------ IRA gather ---
 // One warp per output row; each lane moves 16-byte vectors, issuing a batch of loads before
@@ -103,157 +99,6 @@ __device__ __forceinline__ float gate_for_lane(bool active, int lane, bool hard,
   return expf(incl - v);
 }
 
-// --------------------------------------------------------------- combine ---
-// One warp per anchor.  Merges the per-split statistics of each row into the log-sum-exps,
-// l_r = LSE_d - (sum_v e^{z_t - m_t} z_d) / (sum_v e^{z_t - m_t}), the label entropy,
-// the greedy tokens with their top-1/top-2 gaps, log p_t(x), and the slot weight omega_r of
-// Eq. 1 (envelope w_k, mask, optional gate of Eq. 2).  Writes the anchor's sum omega l and
-// sum omega for the batch reduction.
-__global__ void __launch_bounds__(256) combine_kernel(
-    LossPlan P, const float* __restrict__ part, int mode, float gamma,
-    const float* __restrict__ row_mask, const int32_t* __restrict__ corpus_tok,
-    float* __restrict__ loss_row, float* __restrict__ ent_row, float* __restrict__ lse_d_out,
-    float* __restrict__ lse_t_out, int32_t* __restrict__ argmax_d, int32_t* __restrict__ argmax_t,
-    float* __restrict__ gap_d, float* __restrict__ gap_t, float* __restrict__ logp_x_out,
-    float* __restrict__ weight, double* __restrict__ anchor_part) {
-  const int A = P.N / P.B;
-  const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (a >= A) return;
-  const bool active = lane < P.B;
-  const int r = a * P.B + (active ? lane : 0);
-  const size_t fs = size_t(P.n_parts) * P.N;
-
-  // the sums of exponentials are merged in fp64: their logarithms are the near-zero parts of
-  // the loss and the entropy when the softmax is sharp
-  float Md = -INFINITY, Mt = -INFINITY, U = 0.f, Wt = 0.f;
-  double Sd = 0.0, St = 0.0;
-  float bd = -INFINITY, secd = -INFINITY, bt = -INFINITY, sect = -INFINITY, zx = quiet_nan();
-  int id = 0x7fffffff, it = 0x7fffffff;
-  if (active) {
-    for (int k = 0; k < P.n_parts; ++k) {
-      const float* p = part + size_t(k) * P.N + r;
-      // a part's sums of exponentials, from their two-float parts
-      const float md = p[kPMd * fs], mt = p[kPMt * fs];
-      const double sd = double(p[kPSd * fs]) + double(p[kPSdLo * fs]);
-      const double st = double(p[kPSt * fs]) + double(p[kPStLo * fs]);
-      const float nmd = fmaxf(Md, md), nmt = fmaxf(Mt, mt);
-      const float so = ex2((Mt - nmt) * kLog2e), sn = ex2((mt - nmt) * kLog2e);
-      // U, Wt and the parts' u, w are measured from their own maxima (z_d - M_d, z_t - M_t):
-      // move both to the merged references before adding.  A side with no columns yet (its
-      // maximum still -inf: the merge's start, or a part past the vocabulary) adds nothing.
-      const bool have = Mt > -INFINITY, part_has = mt > -INFINITY;
-      const float Uo = have ? fmaf(Md - nmd, float(St), U) : 0.f;
-      const float Wo = have ? fmaf(Mt - nmt, float(St), Wt) : 0.f;
-      const float un = part_has ? fmaf(md - nmd, float(st), p[kPU * fs]) : 0.f;
-      const float wn = part_has ? fmaf(mt - nmt, float(st), p[kPW * fs]) : 0.f;
-      U = Uo * so + un * sn;
-      Wt = Wo * so + wn * sn;
-      Sd = (have ? Sd * double(ex2((Md - nmd) * kLog2e)) : 0.0) +
-           (part_has ? sd * double(ex2((md - nmd) * kLog2e)) : 0.0);
-      St = (have ? St * double(so) : 0.0) + (part_has ? st * double(sn) : 0.0);
-      Md = nmd;
-      Mt = nmt;
-      // top-2 merge; equal leaders go to the lower token id
-      const float b2 = p[kPBd * fs], s2 = p[kPSecd * fs];
-      const int i2 = __float_as_int(p[kPId * fs]);
-      if (b2 > bd || (b2 == bd && i2 < id)) {
-        secd = fmaxf(bd, s2);
-        bd = b2;
-        id = i2;
-      } else {
-        secd = fmaxf(secd, b2);
-      }
-      const float b3 = p[kPBt * fs], s3 = p[kPSect * fs];
-      const int i3 = __float_as_int(p[kPIt * fs]);
-      if (b3 > bt || (b3 == bt && i3 < it)) {
-        sect = fmaxf(bt, s3);
-        bt = b3;
-        it = i3;
-      } else {
-        sect = fmaxf(sect, b3);
-      }
-      const float z = p[kPZx * fs];
-      if (z == z) zx = z;
-    }
-  }
-  const double lsd = log(Sd), lst = log(St);
-  const float lse_d = Md + float(lsd);
-  const float lse_t = Mt + float(lst);
-  // l = lse_d - E_p[z_d] = log S_d - E_p[z_d - M_d]: two non-negative terms, no cancellation
-  const float loss = float(lsd - double(U) / St);
-  const float logp = zx - lse_t;
-  const bool erase = mode != 0;
-  const int x = (erase && active) ? corpus_tok[r] : -1;
-  const float gate = erase ? gate_for_lane(active, lane, mode == 2, logp, x == it) : 1.f;
-  float w = 0.f;
-  if (active) {
-    w = expf(-float(lane) / gamma) * gate;
-    if (row_mask != nullptr) w *= row_mask[r];
-    loss_row[r] = loss;
-    if (ent_row) ent_row[r] = float(lst - double(Wt) / St);
-    lse_d_out[r] = lse_d;
-    lse_t_out[r] = lse_t;
-    argmax_d[r] = id;
-    argmax_t[r] = it;
-    if (gap_d) gap_d[r] = bd - secd;
-    if (gap_t) gap_t[r] = bt - sect;
-    if (erase && logp_x_out) logp_x_out[r] = logp;
-    weight[r] = w;
-  }
-  double wl = active ? double(w) * double(loss) : 0.0;
-  double ws = active ? double(w) : 0.0;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    wl += __shfl_xor_sync(0xffffffffu, wl, off);
-    ws += __shfl_xor_sync(0xffffffffu, ws, off);
-  }
-  if (lane == 0) {
-    anchor_part[2 * a] = wl;
-    anchor_part[2 * a + 1] = ws;
-  }
-}
-
-// Batch reduction of Eq. 1 in a fixed order (one block, deterministic).  wl_sum (nullable)
-// receives the numerator sum omega l itself, for a sum across the shards of a batch.
-__global__ void __launch_bounds__(1024) finalize_kernel(const double* __restrict__ anchor_part,
-                                                        int A, float lam,
-                                                        float* __restrict__ loss_total,
-                                                        float* __restrict__ weight_sum,
-                                                        float* __restrict__ wl_sum) {
-  __shared__ double s_wl[32], s_ws[32];
-  double wl = 0.0, ws = 0.0;
-  for (int a = threadIdx.x; a < A; a += blockDim.x) {
-    wl += anchor_part[2 * a];
-    ws += anchor_part[2 * a + 1];
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    wl += __shfl_xor_sync(0xffffffffu, wl, off);
-    ws += __shfl_xor_sync(0xffffffffu, ws, off);
-  }
-  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    s_wl[warp] = wl;
-    s_ws[warp] = ws;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    wl = lane < int(blockDim.x / 32) ? s_wl[lane] : 0.0;
-    ws = lane < int(blockDim.x / 32) ? s_ws[lane] : 0.0;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      wl += __shfl_xor_sync(0xffffffffu, wl, off);
-      ws += __shfl_xor_sync(0xffffffffu, ws, off);
-    }
-    if (lane == 0) {
-      *loss_total = ws > 0.0 ? float(double(lam) * wl / ws) : 0.f;
-      *weight_sum = float(ws);
-      if (wl_sum != nullptr) *wl_sum = float(wl);
-    }
-  }
-}
-
 // Eq. 1 from sums that the caller reduced over the shards of a batch: L = lambda * wl / ws,
 // 0 when ws = 0 (no supervised slot anywhere in the batch).
 __global__ void loss_from_sums_kernel(const float* __restrict__ wl_sum,
@@ -309,177 +154,6 @@ __global__ void __launch_bounds__(256) erase_weights_kernel(
     float w = expf(-float(lane) / gamma) * g;
     if (row_mask != nullptr) w *= row_mask[r];
     weight[r] = w;
-  }
-}
-
-// ---------------------------------------------------------- compact labels ---
-// Insert (v, id) into a list sorted by value descending, equal values by id ascending.
-__device__ __forceinline__ void insert_ranked(float (&t)[kTopK], int (&ti)[kTopK], float v,
-                                              int id) {
-  if (!(v > t[kTopK - 1] || (v == t[kTopK - 1] && id < ti[kTopK - 1]))) return;
-  t[kTopK - 1] = v;
-  ti[kTopK - 1] = id;
-#pragma unroll
-  for (int k = kTopK - 1; k > 0; --k) {
-    const bool up = t[k] > t[k - 1] || (t[k] == t[k - 1] && ti[k] < ti[k - 1]);
-    const float a = t[k], b = t[k - 1];
-    const int ia = ti[k], ib = ti[k - 1];
-    t[k - 1] = up ? a : b;
-    t[k] = up ? b : a;
-    ti[k - 1] = up ? ia : ib;
-    ti[k] = up ? ib : ia;
-  }
-}
-
-// 2^-r for the exponent residual r of a reference (|r| <= 4e-3 over the fp16 range of logits):
-// 1 - x + x^2 / 2 with x = r ln 2, within 5e-9 relative (1e-15 for |r| <= 3e-5, |logit| < 1000).
-__device__ __forceinline__ double inv_exp2_small(float r) {
-  const double x = double(r) * 0.6931471805599453;
-  return 1.0 - x + 0.5 * x * x;
-}
-
-// Label readout merge, one thread per row: log-sum-exp over all parts, the k best target
-// logits (ties to the lower id), their probabilities and the tail mass
-//   tail = (S - sum_k exp(t_k - M)) / S,
-// the greedy token with its top-1 minus top-2 gap, and log p at the corpus token.
-__global__ void __launch_bounds__(256) readout_combine_kernel(
-    LossPlan P, const float* __restrict__ part, int has_corpus, int32_t* __restrict__ top_idx,
-    float* __restrict__ top_prob, float* __restrict__ tail, float* __restrict__ lse_t,
-    int32_t* __restrict__ argmax_t, float* __restrict__ gap_t, float* __restrict__ logp_x) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= P.N) return;
-  const size_t fs = size_t(P.n_parts) * P.N;
-  float M = -INFINITY, zx = quiet_nan();
-  double S = 0.0;   // merged in fp64 from the parts' two-float sums
-  float t[kTopK];
-  int ti[kTopK];
-#pragma unroll
-  for (int i = 0; i < kTopK; ++i) {
-    t[i] = -INFINITY;
-    ti[i] = 0x7fffffff;
-  }
-  for (int k = 0; k < P.n_parts; ++k) {
-    const float* p = part + size_t(k) * P.N + r;
-    const float m = p[kRM * fs];
-    const float nm = fmaxf(M, m);
-    const double sp = (double(p[kRS * fs]) + double(p[kRSLo * fs])) * inv_exp2_small(p[kRR * fs]);
-    S = (M > -INFINITY ? S * double(ex2((M - nm) * kLog2e)) : 0.0) +
-        (m > -INFINITY ? sp * double(ex2((m - nm) * kLog2e)) : 0.0);
-    M = nm;
-#pragma unroll
-    for (int i = 0; i < kTopK; ++i) {
-      const float v = p[(kRTop + i) * fs];
-      if (v > -INFINITY) insert_ranked(t, ti, v, __float_as_int(p[(kRIdx + i) * fs]));
-    }
-    const float z = p[kRZx * fs];
-    if (z == z) zx = z;
-  }
-  const double ls = log(S);
-  const float lse = M + float(ls);
-  double inside = 0.0;
-#pragma unroll
-  for (int i = 0; i < kTopK; ++i) {
-    const double e = exp(double(t[i]) - double(M));
-    top_idx[size_t(r) * kTopK + i] = ti[i];
-    top_prob[size_t(r) * kTopK + i] = float(e / S);
-    inside += e;
-  }
-  // with V <= k every token is in the list and the tail is empty by definition
-  tail[r] = P.V <= kTopK ? 0.f : float(fmax(0.0, (S - inside) / S));
-  if (lse_t) lse_t[r] = lse;
-  if (argmax_t) argmax_t[r] = ti[0];
-  if (gap_t) gap_t[r] = t[0] - t[1];
-  if (has_corpus && logp_x) logp_x[r] = float((double(zx) - double(M)) - ls);
-}
-
-// Top-k loss merge, one warp per anchor: log-sum-exp and greedy top-2 of z_d, the label
-// tokens' z_d, the drafter's mass outside them
-//   tail_q = (S_d - sum_i exp(z_i - M_d)) / S_d,
-// the loss l = -sum_i prob_i (z_i - LSE_d) - tail log tail_q (no tail term when tail = 0),
-// the slot weight (given, or envelope times mask) and the anchor's sums for Eq. 1.
-__global__ void __launch_bounds__(256) topk_combine_kernel(
-    LossPlan P, const float* __restrict__ part, const float* __restrict__ top_prob,
-    const float* __restrict__ tail, const float* __restrict__ row_mask,
-    const float* __restrict__ weight_in, float gamma, float* __restrict__ loss_row,
-    float* __restrict__ lse_d_out, float* __restrict__ tail_q_out, int32_t* __restrict__ argmax_d,
-    float* __restrict__ gap_d, float* __restrict__ weight, double* __restrict__ anchor_part) {
-  const int A = P.N / P.B;
-  const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (a >= A) return;
-  const bool active = lane < P.B;
-  const int r = a * P.B + (active ? lane : 0);
-  const size_t fs = size_t(P.n_parts) * P.N;
-  // the sum of exponentials is merged in fp64 from its two-float parts: with a sharp drafter
-  // its logarithm is the near-zero part of every log q
-  float M = -INFINITY, bd = -INFINITY, secd = -INFINITY;
-  double S = 0.0, Sout = 0.0;   // all columns; the columns outside the row's label tokens
-  int id = 0x7fffffff;
-  float zk[kTopK];
-#pragma unroll
-  for (int i = 0; i < kTopK; ++i) zk[i] = quiet_nan();
-  if (active) {
-    for (int k = 0; k < P.n_parts; ++k) {
-      const float* p = part + size_t(k) * P.N + r;
-      const float m = p[kKM * fs];
-      const float nm = fmaxf(M, m);
-      // the part's sums without the factor 2^r its exponentials carry
-      const double unr = inv_exp2_small(p[kKR * fs]);
-      const double sp = (double(p[kKS * fs]) + double(p[kKSLo * fs])) * unr;
-      const double so =
-          ((double(p[kKS * fs]) - double(p[kKSIn * fs])) + double(p[kKSLo * fs])) * unr;
-      const double f_old = M > -INFINITY ? double(ex2((M - nm) * kLog2e)) : 0.0;
-      const double f_new = m > -INFINITY ? double(ex2((m - nm) * kLog2e)) : 0.0;
-      S = S * f_old + sp * f_new;
-      Sout = Sout * f_old + so * f_new;
-      M = nm;
-      const float b2 = p[kKBest * fs], s2 = p[kKSec * fs];
-      const int i2 = __float_as_int(p[kKIdx * fs]);
-      if (b2 > bd || (b2 == bd && i2 < id)) {
-        secd = fmaxf(bd, s2);
-        bd = b2;
-        id = i2;
-      } else {
-        secd = fmaxf(secd, b2);
-      }
-#pragma unroll
-      for (int i = 0; i < kTopK; ++i) {
-        const float z = p[(kKZ + i) * fs];
-        if (z == z) zk[i] = z;
-      }
-    }
-  }
-  float loss = 0.f, w = 0.f;
-  if (active) {
-    const double ls = log(S);
-    const float lse = M + float(ls);
-    // log q_i = (z_i - M) - log S: the difference z_i - M is exact in fp64
-    double ce = 0.0;
-    for (int i = 0; i < kTopK; ++i)
-      ce -= double(top_prob[size_t(r) * kTopK + i]) * ((double(zk[i]) - double(M)) - ls);
-    const double tq = fmax(Sout / S, 1e-30);
-    const float tl = tail[r];
-    if (tl > 0.f) ce -= double(tl) * log(tq);
-    loss = float(ce);
-    w = weight_in != nullptr ? weight_in[r]
-                             : expf(-float(lane) / gamma) * (row_mask ? row_mask[r] : 1.f);
-    loss_row[r] = loss;
-    lse_d_out[r] = lse;
-    tail_q_out[r] = float(tq);
-    argmax_d[r] = id;
-    if (gap_d) gap_d[r] = bd - secd;
-    weight[r] = w;
-  }
-  double wl = active ? double(w) * double(loss) : 0.0;
-  double ws = active ? double(w) : 0.0;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    wl += __shfl_xor_sync(0xffffffffu, wl, off);
-    ws += __shfl_xor_sync(0xffffffffu, ws, off);
-  }
-  if (lane == 0) {
-    anchor_part[2 * a] = wl;
-    anchor_part[2 * a + 1] = ws;
   }
 }
 
@@ -698,46 +372,6 @@ cudaError_t launch_gather(const void* feat, int S, int L, int d, int elem_bytes,
   if (blocks == 0) return cudaSuccess;
   return launch_pdl(gather_kernel, unsigned(blocks), 256, s, static_cast<const uint4*>(feat), S,
                     L, vec, seq, pos, valid_len, A, B, static_cast<uint4*>(out), row_valid);
-}
-
-cudaError_t launch_combine(const LossPlan& plan, const float* part, int mode, float gamma,
-                           const float* row_mask, const int32_t* corpus_tok, float* loss_row,
-                           float* ent_row, float* lse_d, float* lse_t, int32_t* argmax_d,
-                           int32_t* argmax_t, float* gap_d, float* gap_t, float* logp_x,
-                           float* weight, double* anchor_part, cudaStream_t s) {
-  const int A = plan.N / plan.B;
-  combine_kernel<<<(A + 7) / 8, 256, 0, s>>>(plan, part, mode, gamma, row_mask, corpus_tok,
-                                             loss_row, ent_row, lse_d, lse_t, argmax_d, argmax_t,
-                                             gap_d, gap_t, logp_x, weight, anchor_part);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool has_corpus,
-                                   int32_t* top_idx, float* top_prob, float* tail, float* lse_t,
-                                   int32_t* argmax_t, float* gap_t, float* logp_x,
-                                   cudaStream_t s) {
-  readout_combine_kernel<<<(plan.N + 255) / 256, 256, 0, s>>>(plan, part, has_corpus ? 1 : 0,
-                                                              top_idx, top_prob, tail, lse_t,
-                                                              argmax_t, gap_t, logp_x);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const float* top_prob,
-                                const float* tail, const float* row_mask, const float* weight_in,
-                                float gamma, float* loss_row, float* lse_d, float* tail_q,
-                                int32_t* argmax_d, float* gap_d, float* weight,
-                                double* anchor_part, cudaStream_t s) {
-  const int A = plan.N / plan.B;
-  topk_combine_kernel<<<(A + 7) / 8, 256, 0, s>>>(plan, part, top_prob, tail, row_mask, weight_in,
-                                                  gamma, loss_row, lse_d, tail_q, argmax_d, gap_d,
-                                                  weight, anchor_part);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_finalize(const double* anchor_part, int A, float lam, float* loss_total,
-                            float* weight_sum, float* wl_sum, cudaStream_t s) {
-  finalize_kernel<<<1, 1024, 0, s>>>(anchor_part, A, lam, loss_total, weight_sum, wl_sum);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_loss_from_sums(const float* wl_sum, const float* weight_sum, float lam,

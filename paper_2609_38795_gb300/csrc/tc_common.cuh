@@ -38,6 +38,12 @@ ALR_DEV float ex2(float x) {
   return y;
 }
 
+// The exponent every column gets relative to the reference m is fma(z, log2 e, -m log2 e),
+// which at z = m is not 0 but the rounding residual of m log2 e (exactly representable, up to
+// ~4e-6 at |m| ~ 40): every exponential summed against m carries the factor 2^r.  The merge
+// divides it out, so that log S and the log-probabilities taken from it keep their precision.
+ALR_DEV float exp_residual(float m) { return fmaf(m, kLog2e, -m * kLog2e); }
+
 // ------------------------------------------------------ paired fp32 arithmetic ---
 // Two fp32 lanes in one 64-bit register, combined by the sm_100-family packed instructions:
 // each lane is computed exactly as the scalar instruction would, in one issue slot for both.

@@ -1,0 +1,92 @@
+"""The merge of the forward's partial records (combine_kernels.cu) at the edges of its block
+shapes: 8, 16 or 32 rows per block by the anchor size, whole anchors per block, the last block
+partly filled, and the large-batch shape (at least 304 blocks of 32 rows), for the
+full-vocabulary forward, the label readout and the top-k forward, against the oracle."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import alr_oracle as orc
+from paper_2609_38795_gb300 import alr, build_lib, synthetic
+from tests import parity as P
+from tests import test_gpu_topk as T
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    build_lib.build()
+    alr.lib()
+    assert alr.alr_device_supported() == alr.ALR_OK, alr.alr_last_error()
+
+
+# (A, B): one row; a partial 8-row block; anchors of 3 and 8 in 8 rows; 9 and 16 in 16; 17 and
+# 32 in 32; the last shape of the small form (303 blocks of 30 rows) and the first of the large
+SHAPES = [(1, 1), (13, 1), (5, 3), (3, 8), (3, 9), (7, 16), (4, 17), (3, 32), (606, 15),
+          (607, 15), (9729, 1)]
+
+
+@pytest.mark.parametrize("mode", [alr.ALR_MODE_ERASE_SOFT, alr.ALR_MODE_ERASE_HARD])
+@pytest.mark.parametrize("A,B", SHAPES)
+def test_forward_merge(A, B, mode):
+    """V = 520 fills two vocabulary tiles and 8 columns of a third, so some records are empty."""
+    d, V = 64, 520
+    b = synthetic.slot_batch(d, V, A, B, 0.5, dtype=torch.bfloat16, device="cuda", seed=A + B)
+    b = synthetic.sharpen(b)
+    N = A * B
+    g = torch.Generator(device="cuda").manual_seed(A)
+    mask = (torch.rand(N, generator=g, device="cuda") < 0.9).float()
+    mask[0] = 1.0
+    greedy = (b["Ht"].float() @ b["W"].float()).argmax(1).to(torch.int32)
+    rep, rnd = synthetic.corpus_replacement(N, V, 0.2, device="cuda", seed=A)
+    tok = synthetic.corpus_tokens(greedy, rep, rnd)
+    sl = P.gpu_forward(b["Hd"], b["Ht"], b["W"], B, mode=mode, row_mask=mask, corpus_tok=tok)
+    r = orc.slot_loss_forward(P.np64(b["Hd"]), P.np64(b["Ht"]), P.np64(b["W"]), B, mode=mode,
+                              row_mask=P.np64(mask), corpus_tok=P.npi(tok))
+    got = P.fwd_to_numpy(sl)
+    if mode == alr.ALR_MODE_ERASE_HARD:
+        # a hard gate hangs on the greedy token: anchors with a near-tied target row may differ
+        near = (r["gap_t"] < P.NEAR_TIE).reshape(A, B).any(1)
+        keep = np.repeat(~near, B)
+        np.testing.assert_allclose(got["weight"][keep], r["weight"][keep], rtol=1e-5, atol=0)
+        assert np.all(P.rel_err(got["loss_row"], r["loss_row"]) <= P.LOSS_RTOL)
+    else:
+        P.compare_forward(got, r, mode=mode)
+    # the batch sums are the fp32 values of fp64 sums of the row results themselves: 2^-24
+    # relative for the final rounding, and as much again for the weights' own rounding
+    w, l = got["weight"], got["loss_row"]
+    np.testing.assert_allclose(got["weight_sum"], w.sum(), rtol=2.0 ** -23)
+    np.testing.assert_allclose(got["loss_total"], (w * l).sum() / w.sum(), rtol=2.0 ** -22)
+    assert alr.alr_device_status() == alr.ALR_OK
+
+
+@pytest.mark.parametrize("A,B", SHAPES)
+def test_readout_and_topk_merge(A, B):
+    d, V = 64, 520
+    b = synthetic.sharpen(synthetic.slot_batch(d, V, A, B, 0.5, dtype=torch.bfloat16,
+                                               device="cuda", seed=31 * A + B))
+    z = orc.label_readout(P.np64(b["Ht"]), P.np64(b["W"]), k=T.K)
+    g = T.gpu_readout(b["Ht"], b["W"], B)
+    T.compare_readout(g, z)
+    lab = dict(idx=g["top_idx"], prob=g["top_prob"], tail=g["tail"])
+    labels = T.host_labels(lab)
+    _, out = T.gpu_topk_forward(b["Hd"], b["W"], B, lab)
+    zd = P.np64(b["Hd"]) @ P.np64(b["W"])
+    lse = np.log(np.exp(zd - zd.max(1, keepdims=True)).sum(1)) + zd.max(1)
+    rows = np.arange(A * B)[:, None]
+    q = np.exp(zd[rows, labels[0]] - lse[:, None])
+    rest = np.exp(zd - lse[:, None])
+    rest[rows, labels[0]] = 0.0
+    loss = -(labels[1] * np.log(q)).sum(1) - labels[2] * np.log(rest.sum(1))
+    np.testing.assert_allclose(P.np64(out["lse_d"]), lse, rtol=2e-4)
+    np.testing.assert_allclose(P.np64(out["tail_q"]), rest.sum(1), rtol=1e-3)
+    assert P.rel_err(P.np64(out["loss_row"]), loss).max() <= P.LOSS_RTOL
+    w, l = P.np64(out["weight"]), P.np64(out["loss_row"])
+    np.testing.assert_allclose(float(out["weight_sum"].item()), w.sum(), rtol=2.0 ** -23)
+    np.testing.assert_allclose(float(out["loss_total"].item()), (w * l).sum() / w.sum(),
+                               rtol=2.0 ** -22)
+    assert alr.alr_device_status() == alr.ALR_OK
