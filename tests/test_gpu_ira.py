@@ -93,3 +93,29 @@ def test_ira_plan_and_context_bit_exact():
     assert sec.sum() == (pe_ref >= 0).sum()
     assert (cl_ref > 0).sum() > 100 and (rlen.numpy() < K).any()
     assert alr.alr_device_status() == alr.ALR_OK
+
+
+# key patterns of the draw's radix select: the bits that tell keys apart sit in the digit that
+# decides (32 - bits low bits vary), 0: all keys equal, so positions decide
+@pytest.mark.parametrize("bits", [0, 3, 8, 14, 20, 32])
+@pytest.mark.parametrize("L,max_b", [(40, 64), (1025, 1), (4096, 128), (16384, 7),
+                                     (16384, 4000)])
+def test_ira_draw_select_digits(L, max_b, bits):
+    """Draws whose m-th smallest key shares 0 to 4 leading digits with the others, at 1 to 16
+    positions per thread and with every valid position drawn, against the oracle bit for bit."""
+    S, K = 3, 15
+    g = torch.Generator().manual_seed(L + bits)
+    ok = (torch.rand(S, L, generator=g) < torch.tensor([0.3, 0.9, 1.0])[:, None]).to(torch.uint8)
+    low = torch.randint(0, 1 << bits, (S, L), generator=g, dtype=torch.int64)
+    keys = (low - (1 << 31 if bits == 32 else 0)).to(torch.int32)
+    if bits < 32:
+        keys[1] ^= 0x5A5A5A5A                             # the same spread over other digit values
+    off_u = torch.zeros(S, max(max_b // 2, 1), dtype=torch.int32)[:, :max_b // 2].contiguous()
+    out = dict(n_valid=torch.empty(S, dtype=torch.int32, device="cuda"),
+               anchor_pos=torch.full((S, max_b), -7, dtype=torch.int32, device="cuda"),
+               offsets=torch.empty(S, max_b // 2, dtype=torch.int32, device="cuda"))
+    alr.alr_ira_draw(K, max_b, ok.cuda(), keys.cuda(), off_u.cuda(), out)
+    torch.cuda.synchronize()
+    n_valid, anchor_pos, _ = orc.ira_draw(ok.numpy(), _u32(keys), _u32(off_u), K, max_b)
+    assert np.array_equal(P.npi(out["n_valid"]), n_valid)
+    assert np.array_equal(P.npi(out["anchor_pos"]), anchor_pos)
