@@ -15,6 +15,7 @@
 // barrier).  Cl = NoCluster: one CTA per tile.
 #pragma once
 
+#include "gemm_epilogue.cuh"
 #include "kernels.h"
 #include "tc_common.cuh"
 
@@ -33,7 +34,8 @@ constexpr int kABytes = kBM * 128;                // 16 KB
 constexpr int kBBytes = kBN * 128;                // 32 KB
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kCtrlBytes = 256;
-constexpr size_t kSmemBytes = 1024 + size_t(kStages) * kStageBytes + kCtrlBytes;
+constexpr int kEpiBytes = kEpiWarps * kEpiStageBytes;   // the epilogue warps' staging
+constexpr size_t kSmemBytes = 1024 + size_t(kStages) * kStageBytes + kEpiBytes + kCtrlBytes;
 
 template <typename Elem>
 struct Geo {
@@ -111,7 +113,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   using G = Geo<Elem>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_1024(smem_raw);
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint8_t* epi_stage = smem + kStages * kStageBytes;
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(epi_stage + kEpiBytes);
   uint64_t* empty_bar = full_bar + kStages;
   uint64_t* tfull_bar = empty_bar + kStages;
   uint64_t* tempty_bar = tfull_bar + 2;
@@ -242,6 +245,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       int mb, nb;
       decode_tile(args, t, mb, nb);
       if (kMc) mb = kMc * mb + rank;
+      const int m0 = mb * kBM + q * 32, n0 = nb * kBN;
+      CStrip<kAcc, kBN> strip;
+      strip.begin(args, m0, n0, lane);
       // The first epilogue warp waits for the accumulator and posts the outcome in the
       // buffer's word; the others wait, descheduled, in a named barrier.  Every epilogue warp
       // passes the same barriers and follows the one outcome, so they leave together; a word
@@ -254,40 +260,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       named_bar_sync(kEpiBarrier, kEpiWarps * 32);
       if (tile_ready[abuf] == 0) break;
       tc_fence_after();
-      const int m = mb * kBM + q * 32 + lane;
-      const bool m_ok = m < args.M;
-      float* crow = args.C + size_t(m_ok ? m : 0) * size_t(args.ldc);
-      const uint32_t tb = lane_addr + uint32_t(abuf * kBN);
-#pragma unroll 1
-      for (int c = 0; c < kBN / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld32(tb + c * 32, r);
-        tmem_ld_wait();
-        reg_fence(r);
-        const int n0 = nb * kBN + c * 32;
-        if (m_ok) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const int n = n0 + j;
-            if (n < args.Nc) {
-              float4 v = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                     __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
-              float4* dst = reinterpret_cast<float4*>(crow + n);
-              if (kAcc) {
-                const float4 o = *dst;
-                v.x += o.x;
-                v.y += o.y;
-                v.z += o.z;
-                v.w += o.w;
-              }
-              *dst = v;
-            }
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty_bar[abuf]);
+      strip.finish(args, m0, n0, lane_addr + uint32_t(abuf * kBN),
+                   epi_stage + q * kEpiStageBytes, lane, [&] {
+                     tc_fence_before();
+                     __syncwarp();
+                     if (lane == 0) mbar_arrive(&tempty_bar[abuf]);
+                   });
       if (++abuf == 2) {
         abuf = 0;
         aphase ^= 1;

@@ -18,6 +18,7 @@
 
 #include "cluster_forms.h"
 #include "cluster_ptx.cuh"
+#include "gemm_epilogue.cuh"
 #include "kernels.h"
 
 namespace alr {
@@ -41,8 +42,9 @@ constexpr uint32_t kChunkBytes = kKE * 128;
 // CTA's allocation.
 constexpr int kGuardBytes = 16 * 1024;
 constexpr int kCtrlBytes = 256;
+constexpr int kEpiBytes = kEpiWarps * kEpiStageBytes;   // the epilogue warps' staging
 constexpr size_t kSmemBytes =
-    1024 + size_t(kStages) * kStageBytes + kGuardBytes + kCtrlBytes;
+    1024 + size_t(kStages) * kStageBytes + kGuardBytes + kEpiBytes + kCtrlBytes;
 static_assert((2 * kStages + 2 * 2 + 1) * 8 + 8 <= kCtrlBytes, "control block");
 
 ALR_DEV void decode_tile(const GemmArgs& a, int t, int& mb, int& nb) {
@@ -85,7 +87,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                      const __grid_constant__ CUtensorMap tm_b, const GemmArgs args) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_1024(smem_raw);
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes + kGuardBytes);
+  uint8_t* epi_stage = smem + kStages * kStageBytes + kGuardBytes;
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(epi_stage + kEpiBytes);
   uint64_t* empty_bar = full_bar + kStages;
   uint64_t* tfull_bar = empty_bar + kStages;
   uint64_t* tempty_bar = tfull_bar + 2;
@@ -213,42 +216,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int t = pair; t < args.n_tiles; t += n_pairs) {
       int mb, nb;
       decode_tile(args, t, mb, nb);
+      const int m0 = mb * 2 * kRows + int(rank) * kRows + q * 32, n0 = nb * kCols;
+      CStrip<kAcc, kCols> strip;
+      strip.begin(args, m0, n0, lane);
       if (!warp_wait_cl(&tfull_bar[abuf], aphase, ab)) break;
       tc_fence_after();
-      const int m = mb * 2 * kRows + int(rank) * kRows + q * 32 + lane;
-      const bool m_ok = m < args.M;
-      float* crow = args.C + size_t(m_ok ? m : 0) * size_t(args.ldc);
-      const uint32_t tb = lane_addr + uint32_t(abuf * kCols);
-#pragma unroll 1
-      for (int c = 0; c < kCols / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld32(tb + c * 32, r);
-        tmem_ld_wait();
-        reg_fence(r);
-        const int n0 = nb * kCols + c * 32;
-        if (m_ok) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const int n = n0 + j;
-            if (n < args.Nc) {
-              float4 v = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                     __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
-              float4* dst = reinterpret_cast<float4*>(crow + n);
-              if (kAcc) {
-                const float4 o = *dst;
-                v.x += o.x;
-                v.y += o.y;
-                v.z += o.z;
-                v.w += o.w;
-              }
-              *dst = v;
-            }
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(abuf ? tempty_cl1 : tempty_cl0);
+      strip.finish(args, m0, n0, lane_addr + uint32_t(abuf * kCols),
+                   epi_stage + q * kEpiStageBytes, lane, [&] {
+                     tc_fence_before();
+                     __syncwarp();
+                     if (lane == 0) mbar_arrive_cluster(abuf ? tempty_cl1 : tempty_cl0);
+                   });
       if (++abuf == 2) {
         abuf = 0;
         aphase ^= 1;
