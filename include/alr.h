@@ -29,8 +29,11 @@
  *              floating-point rounding of the GEMMs, and the loss kernels' outputs not at all):
  *              ALR_GEMM_FORM = mcast (default: clusters of two CTAs share each B tile by TMA
  *              multicast) | single | mcast4 | pair (CTA pairs with M = 256 tcgen05 products)
- *              selects the bf16 GEMM kernel; ALR_LOSS_FORM = single (default) | mcast selects
- *              the fused loss kernels' form.  fp32 (tf32) products always run on single CTAs.
+ *              selects the GEMM form of every bf16 product; unset, a product with too few output
+ *              tiles to fill the device splits each tile's K over a cluster of CTAs instead (any
+ *              element type, in any process; partial sums added in a fixed order).
+ *              ALR_LOSS_FORM = single (default) | mcast selects the fused loss kernels' form.
+ *              fp32 (tf32) products share no tiles: they run on single CTAs or split K.
  *              The cluster forms (mcast, mcast4, pair, and the loss kernels' mcast) are built
  *              into a second library, libalr_cluster.so, which this library loads from its own
  *              directory on first use.  A process launched as one rank of several (environment

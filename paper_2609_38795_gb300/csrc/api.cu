@@ -296,9 +296,49 @@ GemmForm gemm_form(int dtype) {
   return kGemmMcast;
 }
 
+// How one product runs: its form, and the CTAs per tile of the split form (then `form` is
+// kGemmSingle).
+struct GemmChoice {
+  GemmForm form;
+  int split;
+};
+
+// Split-K rule.  A product with fewer tiles than SMs leaves SMs idle for the whole of its K loop;
+// a cluster of `split` CTAs per tile, each on a share of K, fills them.  Cost in K blocks (64
+// bf16, 0.36 us each on a busy chip): waves of clusters times the share of K plus a fixed 8 + 2
+// split for the start-up and the reduction through distributed shared memory.  Taken only where it
+// promises 15 % over the plain form, which shares B tiles by multicast: measured (us, plain
+// -> split) 128 x 4096 x 151936: 815 -> 216 (6 CTAs); 512 x 4096 x 151936: 817 -> 452 (2); 2000 x
+// 1000 x 60000: 314 -> 175 (2); 16 x 2048 x 32000: 174 -> 37 (12); 768 x 4096 x 60000: 339 -> 300
+// (4); 300 x 512 x 4000: 24.6 -> 14.9 (5); no gain: 1024 x 4096 x 32000 (128 tiles) 182 against
+// 193, 192 x 320 x 1400 (22 K blocks) 13.9 against 13.8, 1920 x 4096 x 151936 (240 tiles) 1663
+// against 1762.  A form asked for by name is never replaced.
+GemmChoice choose_gemm(int dtype, int M, int Nc, int K, int sms) {
+  const GemmChoice plain{gemm_form(dtype), 1};
+  const char* v = getenv("ALR_GEMM_FORM");
+  if (v != nullptr && *v != '\0') return plain;
+  const int64_t tiles = int64_t((M + 127) / 128) * ((Nc + 255) / 256);
+  const int64_t n_kb = (int64_t(K) + k_per_row(dtype) - 1) / k_per_row(dtype);
+  if (tiles >= sms) return plain;
+  int best = 1;
+  int64_t best_cost = n_kb * 85 / 100;
+  for (int split : {2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
+    if (split > n_kb) break;
+    const int clusters = alr::plain_gemm_split_clusters(split);
+    if (clusters < 1) continue;
+    const int64_t cost =
+        (tiles + clusters - 1) / clusters * ((n_kb + split - 1) / split + 8 + 2 * split);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = split;
+    }
+  }
+  return best > 1 ? GemmChoice{kGemmSingle, best} : plain;
+}
+
 // Rows of a K-major B box (B columns loaded by one copy).
-uint32_t gemm_b_rows(int dtype) {
-  switch (gemm_form(dtype)) {
+uint32_t gemm_b_rows(const GemmChoice& c) {
+  switch (c.form) {
     case kGemmSingle: return 256;
     case kGemmMcast4: return 64;
     default: return 128;
@@ -336,12 +376,12 @@ alr::GemmArgs pair_gemm_plan(int M, int Nc, int K, float* C, int64_t ldc, int pa
   return g;
 }
 
-// C (+)= A B with the operand maps already encoded (B boxes of gemm_b_rows(dt) rows).
-int launch_gemm(int dt, bool a_mn, bool b_mn, bool acc, const CUtensorMap& ma,
+// C (+)= A B with the operand maps already encoded (B boxes of gemm_b_rows(c) rows).
+int launch_gemm(const GemmChoice& c, int dt, bool a_mn, bool b_mn, bool acc, const CUtensorMap& ma,
                 const CUtensorMap& mb, int M, int Nc, int K, float* C, int64_t ldc, int sms,
                 cudaStream_t s, const char* what) {
   cudaError_t e;
-  const GemmForm form = gemm_form(dt);
+  const GemmForm form = c.form;
   const alr::ClusterForms* cf = alr::cluster_forms();   // non-NULL for every cluster form
   if (form == kGemmPair) {
     const int pairs = cf->pair_gemm_max_pairs();
@@ -368,6 +408,7 @@ int launch_gemm(int dt, bool a_mn, bool b_mn, bool acc, const CUtensorMap& ma,
     e = cf->launch_gemm(cl, a_mn, b_mn, acc, &ma, &mb, &g, s);
   } else {
     alr::GemmArgs g = gemm_plan(M, Nc, K, C, ldc, sms);
+    g.split = c.split;
     g.status = alr::device_status_ptr();
     if (g.status == nullptr) return fail(ALR_ERR_CUDA, "status word lookup failed");
     g.withhold_first_stage = g_withhold_next.exchange(0);
@@ -650,19 +691,21 @@ int head_grads_impl(const alr_params* p, const void* Hd, const void* W, const vo
   cudaError_t e;
   // dH_d = G W^T: A = G [N, V] K-major, B = W [d, V] K-major.
   CUtensorMap m_ga, m_wk;
+  const GemmChoice dh = choose_gemm(dt, int(p->N), p->d, p->V, info.sms);
   if ((rc = make_map(&m_ga, G, dt, p->V, p->N, p->V * es, kke, 128)) != ALR_OK) return rc;
-  if ((rc = make_map(&m_wk, W, dt, p->V, p->d, p->V * es, kke, gemm_b_rows(dt))) != ALR_OK)
+  if ((rc = make_map(&m_wk, W, dt, p->V, p->d, p->V * es, kke, gemm_b_rows(dh))) != ALR_OK)
     return rc;
-  if ((rc = launch_gemm(dt, false, false, false, m_ga, m_wk, int(p->N), p->d, p->V, dHd, p->d,
+  if ((rc = launch_gemm(dh, dt, false, false, false, m_ga, m_wk, int(p->N), p->d, p->V, dHd, p->d,
                         info.sms, s, "dH GEMM launch")) != ALR_OK)
     return rc;
   if (dW == nullptr) return ALR_OK;
   CUtensorMap m_ha, m_gb;
+  const GemmChoice dw = choose_gemm(dt, p->d, p->V, int(p->N), info.sms);
   if (dt == ALR_BF16) {
     // dW += H_d^T G: A = H_d read as [K = N, M = d] (MN-major), B = G [K = N, V] (MN-major).
     if ((rc = make_map(&m_ha, Hd, dt, p->d, p->N, p->d * es, kke, kke)) != ALR_OK) return rc;
     if ((rc = make_map(&m_gb, G, dt, p->V, p->N, p->V * es, kke, kke)) != ALR_OK) return rc;
-    return launch_gemm(dt, true, true, true, m_ha, m_gb, p->d, p->V, int(p->N), dW, p->V,
+    return launch_gemm(dw, dt, true, true, true, m_ha, m_gb, p->d, p->V, int(p->N), dW, p->V,
                        info.sms, s, "dW GEMM launch");
   } else {
     // K-major operands from transposed copies H_d^T [d, N'] and G^T [V, N'].
@@ -675,9 +718,9 @@ int head_grads_impl(const alr_params* p, const void* Hd, const void* W, const vo
                                      int(lay.ld_n), s)) != cudaSuccess)
       return cuda_fail(e, "G transpose launch");
     if ((rc = make_map(&m_ha, hdt, dt, p->N, p->d, lay.ld_n * 4, kke, 128)) != ALR_OK) return rc;
-    if ((rc = make_map(&m_gb, gt, dt, p->N, p->V, lay.ld_n * 4, kke, gemm_b_rows(dt))) != ALR_OK)
+    if ((rc = make_map(&m_gb, gt, dt, p->N, p->V, lay.ld_n * 4, kke, gemm_b_rows(dw))) != ALR_OK)
       return rc;
-    return launch_gemm(dt, false, false, true, m_ha, m_gb, p->d, p->V, int(p->N), dW, p->V,
+    return launch_gemm(dw, dt, false, false, true, m_ha, m_gb, p->d, p->V, int(p->N), dW, p->V,
                        info.sms, s, "dW GEMM launch");
   }
 }
@@ -1185,14 +1228,15 @@ int alr_gemm(int32_t dtype, int32_t a_mn, int32_t b_mn, int32_t accumulate, cons
   int rc = require_sm103(&info);
   if (rc != ALR_OK) return rc;
   const uint32_t kke = k_per_row(dtype);
+  const GemmChoice choice = choose_gemm(dtype, M, Nc, K, info.sms);
   CUtensorMap ma, mb;
   if (a_mn) rc = make_map(&ma, A, dtype, M, K, M * es, kke, kke);
   else rc = make_map(&ma, A, dtype, K, M, K * es, kke, 128);
   if (rc != ALR_OK) return rc;
   if (b_mn) rc = make_map(&mb, B, dtype, Nc, K, Nc * es, kke, kke);
-  else rc = make_map(&mb, B, dtype, K, Nc, K * es, kke, gemm_b_rows(dtype));
+  else rc = make_map(&mb, B, dtype, K, Nc, K * es, kke, gemm_b_rows(choice));
   if (rc != ALR_OK) return rc;
-  return launch_gemm(dtype, a_mn != 0, b_mn != 0, accumulate != 0, ma, mb, M, Nc, K, C, Nc,
+  return launch_gemm(choice, dtype, a_mn != 0, b_mn != 0, accumulate != 0, ma, mb, M, Nc, K, C, Nc,
                      info.sms, static_cast<cudaStream_t>(stream), "gemm launch");
 }
 

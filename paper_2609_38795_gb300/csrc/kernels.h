@@ -125,6 +125,7 @@ struct GemmArgs {
   int group_m;      // m-blocks per raster group
   int n_tiles;
   int grid;
+  int split;        // CTAs that share one tile's K blocks (split form; 0 or 1: not split)
   int* status;
   int withhold_first_stage;   // test hook: the producer never fills its first stage
 };
@@ -133,7 +134,10 @@ struct GemmArgs {
 cudaError_t launch_plain_gemm(int dtype, bool a_mn, bool b_mn, bool accumulate,
                               const CUtensorMap& a, const CUtensorMap& b, const GemmArgs& args,
                               cudaStream_t s);
-size_t plain_gemm_smem_bytes(int dtype);
+// Split form (args.split CTAs per tile, a cluster): how many such clusters the current device holds
+// at once (0: none).
+constexpr int kMaxSplit = 16;
+int plain_gemm_split_clusters(int n_cta);
 // The cluster forms of the same kernel (multicast clusters, CTA pairs) are in
 // libalr_cluster.so (cluster_forms.h).
 

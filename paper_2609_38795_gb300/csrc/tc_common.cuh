@@ -319,6 +319,28 @@ ALR_DEV uint32_t n_clusters_x() {
   return r;
 }
 
+ALR_DEV uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
+// Shared::cluster address of the object at the same offset as `p` in CTA `rank`'s shared memory.
+ALR_DEV uint32_t cluster_smem_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+  return r;
+}
+
+ALR_DEV float4 ld_cluster_v4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+
 // All threads of every CTA of the cluster: arrive (release) and wait (acquire).
 ALR_DEV void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" :::
@@ -327,6 +349,12 @@ ALR_DEV void cluster_sync() {
 
 // The form of a kernel that runs without clusters: no CTA shares its operand tiles.
 struct NoCluster {
+  static constexpr int kCtas = 1;
+};
+
+// The form of the plain GEMM whose clusters split the contraction of one tile: the CTAs share no
+// operand tile, only their partial sums, through distributed shared memory.
+struct SplitCluster {
   static constexpr int kCtas = 1;
 };
 

@@ -10,13 +10,6 @@
 
 namespace alr {
 
-// Shared::cluster address of the object at the same offset as `p` in CTA `rank`'s smem.
-ALR_DEV uint32_t cluster_addr(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-  return r;
-}
-
 // Arrive on an mbarrier in any CTA of the cluster (release at cluster scope).
 ALR_DEV void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar)

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           uint8_t* sb = smem + stage * kStageBytes;
-          const uint32_t fb = cluster_addr(&full_bar[stage], 0);
+          const uint32_t fb = cluster_smem_addr(&full_bar[stage], 0);
           if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2 * kStageBytes);
           load_operand<kAMN, kRows>(sb, &tm_a, fb, m0, kb);
           load_operand<kBMN, kHalf>(sb + kABytes, &tm_b, fb, n0, kb);
@@ -209,8 +209,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // -------------------------------------------------------------------- epilogue ---
     const int q = warp & 3;
     const uint32_t lane_addr = tmem_base + (uint32_t(q * 32) << 16);
-    const uint32_t tempty_cl0 = cluster_addr(&tempty_bar[0], 0);
-    const uint32_t tempty_cl1 = cluster_addr(&tempty_bar[1], 0);
+    const uint32_t tempty_cl0 = cluster_smem_addr(&tempty_bar[0], 0);
+    const uint32_t tempty_cl1 = cluster_smem_addr(&tempty_bar[1], 0);
     int abuf = 0;
     uint32_t aphase = 0;
     for (int t = pair; t < args.n_tiles; t += n_pairs) {

@@ -64,3 +64,31 @@ def test_gemm_layouts(form, dtype, a_mn, b_mn, shape, monkeypatch):
     err2 = (C.double() - 2 * ref).abs().max().item() / (2 * ref.abs().max().item())
     assert err2 <= tol, err2
     assert alr.alr_device_status() == alr.ALR_OK
+
+
+@pytest.mark.parametrize("dtype,a_mn,b_mn", [(torch.float32, False, False)] + [
+    (torch.bfloat16, a, b) for a, b in itertools.product([False, True], repeat=2)])
+@pytest.mark.parametrize("shape", [(128, 64, 8200), (16, 2048, 4104), (304, 512, 4000),
+                                   (136, 1000, 30008), (2000, 264, 2000), (8, 8, 1024)])
+def test_gemm_split_k(dtype, a_mn, b_mn, shape, monkeypatch):
+    """Few-tile products with a long K, which split each tile's K over a cluster (1 to 32 tiles:
+    clusters of 16 down to 4 CTAs, K shares of unequal length, a K tail, partial tiles):
+    against fp64, bit-identical from run to run, and adding to C exactly what the overwriting
+    form writes."""
+    monkeypatch.delenv("ALR_GEMM_FORM", raising=False)
+    M, Nc, K = shape
+    A_st, B_st, ref = _operands(M, Nc, K, dtype, a_mn, b_mn, seed=M + Nc + K)
+    C = torch.full((M, Nc), float("nan"), device="cuda")
+    C2 = C.clone()
+    alr.alr_gemm(A_st, B_st, C, M, Nc, K, a_mn=a_mn, b_mn=b_mn)
+    alr.alr_gemm(A_st, B_st, C2, M, Nc, K, a_mn=a_mn, b_mn=b_mn)
+    torch.cuda.synchronize()
+    tol = 1e-4 if dtype == torch.bfloat16 else 5e-3      # as in test_gemm_layouts
+    assert (C.double() - ref).abs().max().item() <= tol * ref.abs().max().item()
+    assert torch.equal(C, C2)
+    base = torch.randn(M, Nc, device="cuda")
+    acc = base.clone()
+    alr.alr_gemm(A_st, B_st, acc, M, Nc, K, a_mn=a_mn, b_mn=b_mn, accumulate=True)
+    torch.cuda.synchronize()
+    assert torch.equal(acc, base + C)
+    assert alr.alr_device_status() == alr.ALR_OK
