@@ -27,11 +27,12 @@
  *   Inputs.    Outputs are unspecified when the inputs contain NaN or Inf.
  *   Kernel forms (environment, read at every call; results do not depend on them except for
  *              floating-point rounding of the GEMMs, and the loss kernels' outputs not at all):
- *              ALR_GEMM_FORM = mcast (default: clusters of two CTAs share each B tile by TMA
- *              multicast) | single | mcast4 | pair (CTA pairs with M = 256 tcgen05 products)
- *              selects the GEMM form of every bf16 product; unset, a product with too few output
- *              tiles to fill the device splits each tile's K over a cluster of CTAs instead (any
- *              element type, in any process; partial sums added in a fixed order).
+ *              ALR_GEMM_FORM = mcast (clusters of two CTAs share each B tile by TMA multicast) |
+ *              single | mcast4 | pair (CTA pairs with M = 256 tcgen05 products) selects the form of
+ *              every bf16 GEMM; unset, each product takes single, mcast or pair by its sizes, or
+ *              splits each tile's K over a cluster of CTAs when it has too few output tiles to
+ *              fill the device (any element type, in any process; partial sums added in a fixed
+ *              order).
  *              ALR_LOSS_FORM = single (default) | mcast selects the fused loss kernels' form.
  *              fp32 (tf32) products share no tiles: they run on single CTAs or split K.
  *              The cluster forms (mcast, mcast4, pair, and the loss kernels' mcast) are built
@@ -114,7 +115,8 @@ int alr_device_supported(void);
 int alr_device_status(void* stream, int clear);
 
 /*
- * The kernel forms the next bf16 call will use in this process (no device needed):
+ * The kernel forms of this process (no device needed): the one ALR_GEMM_FORM names, or, with it
+ * unset, the one the largest bf16 products take, and the loss kernels':
  *   *gemm: 0 single CTAs, 1 clusters of two sharing B tiles by TMA multicast, 2 CTA pairs
  *          (cta_group::2), 3 clusters of four with multicast;
  *   *loss: 0 single CTAs, 1 clusters of two sharing head tiles by TMA multicast.

@@ -271,19 +271,17 @@ BwdLayout bwd_layout(const alr_params* p, bool with_g = true) {
   return L;
 }
 
-// Form of the bf16 products, chosen by the environment variable ALR_GEMM_FORM:
+// Forms of the products.  The environment variable ALR_GEMM_FORM names one for every bf16 product:
 //   "mcast"   clusters of two CTAs, each on a 128 x 256 tile, sharing every B tile by TMA
-//             multicast, the default;
+//             multicast;
+//   "mcast4"  as "mcast" with clusters of four CTAs, each loading a quarter of the B tile;
 //   "single"  one CTA per 128 x 256 tile, each loading its own B tiles (plain_gemm.cu);
 //   "pair"    CTA pairs with M = 256 products.
-// The cluster forms ("mcast", "mcast4", "pair") live in libalr_cluster.so (csrc_cluster/),
-// which only a single-process run loads: in a process that is one rank of several, or where
-// that library cannot be loaded, every form runs as "single" (alr_kernel_forms reports it).
-// The step runs at the GB300's power cap, so the form that moves fewest bytes per product
-// wins: multicast halves the B traffic out of L2 and runs 6 % faster than single CTAs at the
-// same clock and power.  The pair form issues more products per clock but draws more power
-// per product and settles at a clock ~20 % lower.  tf32 products always run on single CTAs.
-//   "mcast4"  as "mcast" with clusters of four CTAs, each loading a quarter of the B tile.
+// Unset, choose_gemm() picks single, mcast or pair, or the split of a tile's K over a cluster, by
+// the sizes.  The cluster forms ("mcast", "mcast4", "pair") live in libalr_cluster.so
+// (csrc_cluster/), which only a single-process run loads: in a process that is one rank of
+// several, or where that library cannot be loaded, every named form runs as "single"
+// (alr_kernel_forms reports it).  tf32 products run on single CTAs or split K.
 enum GemmForm { kGemmSingle = 0, kGemmMcast = 1, kGemmPair = 2, kGemmMcast4 = 3 };
 
 GemmForm gemm_form(int dtype) {
@@ -303,37 +301,70 @@ struct GemmChoice {
   int split;
 };
 
-// Split-K rule.  A product with fewer tiles than SMs leaves SMs idle for the whole of its K loop;
-// a cluster of `split` CTAs per tile, each on a share of K, fills them.  Cost in K blocks (64
-// bf16, 0.36 us each on a busy chip): waves of clusters times the share of K plus a fixed 8 + 2
-// split for the start-up and the reduction through distributed shared memory.  Taken only where it
-// promises 15 % over the plain form, which shares B tiles by multicast: measured (us, plain
-// -> split) 128 x 4096 x 151936: 815 -> 216 (6 CTAs); 512 x 4096 x 151936: 817 -> 452 (2); 2000 x
-// 1000 x 60000: 314 -> 175 (2); 16 x 2048 x 32000: 174 -> 37 (12); 768 x 4096 x 60000: 339 -> 300
-// (4); 300 x 512 x 4000: 24.6 -> 14.9 (5); no gain: 1024 x 4096 x 32000 (128 tiles) 182 against
-// 193, 192 x 320 x 1400 (22 K blocks) 13.9 against 13.8, 1920 x 4096 x 151936 (240 tiles) 1663
-// against 1762.  A form asked for by name is never replaced.
+// The form of a product when none is asked for by name: the cheapest by a cost in 0.01 us, from
+// the rounds a form needs over the SMs and a fixed time per K block (64 bf16) and per launch,
+// fitted to the measurements below (us, random operands, timed alone).
+//   pair    27 per K block: six 32 KB stages per CTA ride out the load latency that four 48 KB
+//           stages do not (500-520 against 600-690 cycles per K block, 512 being the tensor
+//           pipe's time), and B is read once per pair.  It draws more power per product, though: at
+//           the text8b size (4.1e13 flop per product, the step at the power cap throughout) dH
+//           and dW gain 2.6 ms and the forward behind them loses 5, 102.5 -> 106.1 ms per step;
+//           at 1.0e13 the step gains 1 %, at 2.4e12 4 %, at 5.4e11 5 %.  So: up to kPairFlops.
+//   mcast   35.5 per K block; single 42, but no cluster has to be placed and an odd row block
+//           leaves no CTA idle (128 x 32000 x 512: 9.4 against 15.4 us).
+//   split   few tiles, long K: `split` CTAs per tile fill SMs that would idle.  128 x 4096 x
+//           151936: 823 (mcast) -> 208 us (6 CTAs); 512 x 4096 x 151936: 632 (pair) -> 460 (2);
+//           2000 x 1000 x 60000: 255 (pair) -> 178 (2); 16 x 2048 x 32000: 174 -> 37 (12); 300 x
+//           512 x 4000: 23 -> 15 (5).  No gain past one tile per SM (1920 x 4096 x 151936: 1663
+//           against 1762).  Taken where it promises 10 %.
+constexpr double kPairFlops = 1.5e13;
+constexpr int64_t kPairMinBlocks = 32;   // below, the start of a pair's tile costs what it saves
+
 GemmChoice choose_gemm(int dtype, int M, int Nc, int K, int sms) {
-  const GemmChoice plain{gemm_form(dtype), 1};
+  GemmChoice best{gemm_form(dtype), 1};
   const char* v = getenv("ALR_GEMM_FORM");
-  if (v != nullptr && *v != '\0') return plain;
-  const int64_t tiles = int64_t((M + 127) / 128) * ((Nc + 255) / 256);
+  if (v != nullptr && *v != '\0') return best;
+  const int64_t n_mb = (M + 127) / 128, n_nb = (Nc + 255) / 256, tiles = n_mb * n_nb;
   const int64_t n_kb = (int64_t(K) + k_per_row(dtype) - 1) / k_per_row(dtype);
-  if (tiles >= sms) return plain;
-  int best = 1;
-  int64_t best_cost = n_kb * 85 / 100;
+  auto rounds = [](int64_t units, int64_t at_once) { return (units + at_once - 1) / at_once; };
+
+  best = GemmChoice{kGemmSingle, 1};
+  int64_t best_cost = rounds(tiles, sms) * n_kb * 42;
+  const alr::ClusterForms* cf = dtype == ALR_BF16 ? alr::cluster_forms() : nullptr;
+  if (cf != nullptr) {
+    const int64_t units = (n_mb + 1) / 2 * n_nb;   // both cluster forms take two row blocks
+    const int clusters = cf->gemm_max_clusters(2);
+    if (clusters > 0) {
+      const int64_t cost = rounds(units, clusters) * n_kb * 71 / 2 + 60;
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = GemmChoice{kGemmMcast, 1};
+      }
+    }
+    // (the withheld-stage hook is not in the pair form)
+    if (n_kb >= kPairMinBlocks && 2.0 * M * Nc * K <= kPairFlops && g_withhold_next.load() == 0) {
+      const int pairs = cf->pair_gemm_max_pairs();
+      const int64_t cost = pairs > 0 ? rounds(units, pairs) * n_kb * 27 + 150 : best_cost;
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = GemmChoice{kGemmPair, 1};
+      }
+    }
+  }
+  if (tiles >= sms) return best;
+  best_cost = best_cost * 9 / 10;
   for (int split : {2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
     if (split > n_kb) break;
     const int clusters = alr::plain_gemm_split_clusters(split);
     if (clusters < 1) continue;
     const int64_t cost =
-        (tiles + clusters - 1) / clusters * ((n_kb + split - 1) / split + 8 + 2 * split);
+        rounds(tiles, clusters) * ((n_kb + split - 1) / split * 36 + 290 + 70 * split);
     if (cost < best_cost) {
       best_cost = cost;
-      best = split;
+      best = GemmChoice{kGemmSingle, split};
     }
   }
-  return best > 1 ? GemmChoice{kGemmSingle, best} : plain;
+  return best;
 }
 
 // Rows of a K-major B box (B columns loaded by one copy).

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256) ira_blocks_kernel(
 // candidate.  Positions live in registers (L <= 16 per thread).  Counting each valid pair's rank
 // among all L instead took 380 us for 6 samples of L = 4096; this takes 8.5 us.
 // Offsets: j = 2 + floor(u (K - 2) / 2^32).
-constexpr int kDrawThreads = 1024;
+constexpr int kDrawThreads = 1024;         // most; 256 and 512 for short samples
 constexpr int kDrawPer = 16;               // positions per thread: L <= 16384
 constexpr int kDrawSlack = 64;
 using Pair = unsigned long long;           // key << 32 | position
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kDrawThreads)
   int mine = 0;
 #pragma unroll
   for (int j = 0; j < kDrawPer; ++j) {
-    const int a = tid + j * kDrawThreads;
+    const int a = tid + j * int(blockDim.x);
     c[j] = kNoPair;
     if (a < L && anchor_ok[row + a] != 0) {
       c[j] = (Pair(keys[row + a]) << 32) | unsigned(a);
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kDrawThreads)
   __syncthreads();
   const int v = s_valid, m = min(v, max_blocks);
   int32_t* out = anchor_pos + size_t(s) * size_t(max_blocks);
-  for (int i = m + tid; i < max_blocks; i += kDrawThreads) out[i] = -1;
+  for (int i = m + tid; i < max_blocks; i += blockDim.x) out[i] = -1;
 
   // candidates: pairs whose bits from `shift` up are at most `prefix` (all valid ones when m = v)
   Pair prefix = kNoPair;
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kDrawThreads)
     if (c[j] != kNoPair && (c[j] >> shift) <= prefix) cand[atomicAdd(&s_cand, 1)] = c[j];
   __syncthreads();
   const int n = s_cand;
-  for (int i = warp; i < n; i += kDrawThreads / 32) {
+  for (int i = warp; i < n; i += int(blockDim.x >> 5)) {
     const Pair mypair = cand[i];
     int rank = 0;
     for (int q = lane; q < n; q += 32) rank += cand[q] < mypair ? 1 : 0;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kDrawThreads)
     if (lane == 0 && rank < m) out[rank] = int(unsigned(mypair));
   }
   const int H = max_blocks / 2;
-  for (int i = tid; i < H; i += kDrawThreads) {
+  for (int i = tid; i < H; i += blockDim.x) {
     const unsigned long long u = offset_u[size_t(s) * H + i];
     offsets[size_t(s) * H + i] = 2 + int((u * unsigned(K - 2)) >> 32);
   }
@@ -407,7 +407,8 @@ cudaError_t launch_ira_draw(int S, int L, int K, int max_blocks, const uint8_t* 
   cudaError_t e = cudaFuncSetAttribute(ira_draw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        int(smem));
   if (e != cudaSuccess) return e;
-  ira_draw_kernel<<<S, kDrawThreads, smem, s>>>(L, K, max_blocks, anchor_ok, keys, offset_u, n_valid,
+  const int threads = L <= 256 ? 256 : L <= 512 ? 512 : kDrawThreads;
+  ira_draw_kernel<<<S, threads, smem, s>>>(L, K, max_blocks, anchor_ok, keys, offset_u, n_valid,
                                         anchor_pos, offsets);
   return cudaGetLastError();
 }

@@ -30,6 +30,7 @@ constexpr int kHalf = kCols / 2;            // columns of B loaded by each CTA
 constexpr int kThreads = 256;
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiWarps = 4;
+constexpr int kEpiBarrier = 1;              // named barrier of the epilogue warps
 constexpr int kStages = 6;
 constexpr int kABytes = kRows * 128;        // 16 KB: 128 rows x 64 bf16 of K
 constexpr int kBBytes = kHalf * 128;        // 16 KB
@@ -45,7 +46,7 @@ constexpr int kCtrlBytes = 256;
 constexpr int kEpiBytes = kEpiWarps * kEpiStageBytes;   // the epilogue warps' staging
 constexpr size_t kSmemBytes =
     1024 + size_t(kStages) * kStageBytes + kGuardBytes + kEpiBytes + kCtrlBytes;
-static_assert((2 * kStages + 2 * 2 + 1) * 8 + 8 <= kCtrlBytes, "control block");
+static_assert((2 * kStages + 2 * 2 + 1) * 8 + 16 <= kCtrlBytes, "control block");
 
 ALR_DEV void decode_tile(const GemmArgs& a, int t, int& mb, int& nb) {
   const int per_group = a.group_m * a.n_nb;
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* drain_bar = tempty_bar + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
   volatile int* abort_word = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* tile_ready = abort_word + 1;   // [2], one per accumulator buffer
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -219,7 +221,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int m0 = mb * 2 * kRows + int(rank) * kRows + q * 32, n0 = nb * kCols;
       CStrip<kAcc, kCols> strip;
       strip.begin(args, m0, n0, lane);
-      if (!warp_wait_cl(&tfull_bar[abuf], aphase, ab)) break;
+      // one epilogue warp polls the accumulator barrier, the others sleep in a named barrier and
+      // follow the outcome it posts (as in plain_gemm_kernel.cuh)
+      if (warp == kEpiWarp0) {
+        const bool w = warp_wait_cl(&tfull_bar[abuf], aphase, ab);
+        if (lane == 0) tile_ready[abuf] = w ? 1 : 0;
+        __syncwarp();
+      }
+      named_bar_sync(kEpiBarrier, kEpiWarps * 32);
+      if (tile_ready[abuf] == 0) break;
       tc_fence_after();
       strip.finish(args, m0, n0, lane_addr + uint32_t(abuf * kCols),
                    epi_stage + q * kEpiStageBytes, lane, [&] {

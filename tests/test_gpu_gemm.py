@@ -69,12 +69,14 @@ def test_gemm_layouts(form, dtype, a_mn, b_mn, shape, monkeypatch):
 @pytest.mark.parametrize("dtype,a_mn,b_mn", [(torch.float32, False, False)] + [
     (torch.bfloat16, a, b) for a, b in itertools.product([False, True], repeat=2)])
 @pytest.mark.parametrize("shape", [(128, 64, 8200), (16, 2048, 4104), (304, 512, 4000),
-                                   (136, 1000, 30008), (2000, 264, 2000), (8, 8, 1024)])
-def test_gemm_split_k(dtype, a_mn, b_mn, shape, monkeypatch):
-    """Few-tile products with a long K, which split each tile's K over a cluster (1 to 32 tiles:
-    clusters of 16 down to 4 CTAs, K shares of unequal length, a K tail, partial tiles):
-    against fp64, bit-identical from run to run, and adding to C exactly what the overwriting
-    form writes."""
+                                   (136, 1000, 30008), (2000, 264, 2000), (8, 8, 1024),
+                                   (2200, 2056, 2056), (2200, 2056, 520), (104, 8200, 72)])
+def test_gemm_form_chosen_by_size(dtype, a_mn, b_mn, shape, monkeypatch):
+    """The form each size takes when none is named.  Few tiles and a long K split each tile's K
+    over a cluster (1 to 32 tiles: clusters of 16 down to 4 CTAs, K shares of unequal length, a
+    K tail, partial tiles); 2200 x 2056 takes CTA pairs at K = 2056 and multicast clusters at
+    520 (bf16); one row block and K = 72 single CTAs.  Against fp64, bit-identical from run to
+    run, and adding to C exactly what the overwriting form writes."""
     monkeypatch.delenv("ALR_GEMM_FORM", raising=False)
     M, Nc, K = shape
     A_st, B_st, ref = _operands(M, Nc, K, dtype, a_mn, b_mn, seed=M + Nc + K)
