@@ -2,6 +2,7 @@
 // work planning and kernel launches.  No entry point allocates device memory.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -183,8 +184,52 @@ bool loss_multicast(const alr_params* p) {
   return v != nullptr && strcmp(v, "mcast") == 0 && alr::cluster_forms() != nullptr;
 }
 
-// two_rows: the single-operand modes (readout, top-k), whose units hold two row blocks.
-alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, bool two_rows = false) {
+// Vocabulary splits of a forward over `rb` row blocks (row-block pairs in the two-row modes).
+// CTAs take units (row block x split) in turn, so a round that is not full costs a whole unit:
+// with 19 splits throughout, 9 row blocks are 171 units on 152 CTAs, two rounds for the work of
+// one.  The split count is the one whose rounds times unit length (in vocabulary tiles, plus
+// the fixed cost of a unit) is smallest; `base` (one round over `group` row blocks, 19 splits
+// for 8) stays unless another promises 2 %.  More splits are more partial records: they take
+// at most kPartBytes beyond base's, so every problem the no-workspace forward took still fits.
+// Measured (us, 19 splits -> chosen): forward of 1152 x 1024 x 60000 358 -> 223, 2176 x 2048 x
+// 100000 1443 -> 1150, 8320 x 1024 x 32000 857 -> 760, 1920 x 4096 x 151936 2770 -> 2677; label
+// readout of 4096 x 2048 x 32000 533 -> 431.
+constexpr int64_t kPartBytes = 48ll << 20;
+constexpr int64_t kMaxRecordBytes = 4 * int64_t(sizeof(float)) * alr::kPFields;   // per row and split
+
+enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
+
+int forward_splits(const alr_params* p, int sms, int rb, int n_vt, int group, PlanKind kind) {
+  const int base = std::min(n_vt, std::max(1, sms / std::min(rb, group)));
+  const int64_t fit = p->dtype == ALR_BF16 ? kPartBytes / (p->N * kMaxRecordBytes) : 0;
+  const int most = int(std::min<int64_t>(n_vt, std::max<int64_t>(base, fit)));
+  // cycles of one tile: two 128 x 256 products over d (about 1090 per 64 of d) and an epilogue of
+  // about 7000; a unit adds its first loads and its record, about 2500, and in the readout the
+  // filling of its top-8 lists, about 25000; a split adds its records' trip through memory (at
+  // about 2800 bytes a cycle)
+  const double tile = 1090.0 * ((p->d + 63) / 64) * (p->dtype == ALR_BF16 ? 1 : 2) + 7000.0;
+  const double per_unit = (kind == kPlanReadout ? 27500.0 : 2500.0) / tile;
+  const double per_split = 2.0 * double(p->N) * kMaxRecordBytes / 2800.0 / tile;
+  auto cost = [&](int vs) {
+    const int rounds = int((int64_t(rb) * vs + sms - 1) / sms);
+    const double mean = double(n_vt) / vs, longest = (n_vt + vs - 1) / vs;
+    // splits differ by one tile at most, and successive groups rotate them over the CTAs
+    return std::min(rounds * longest, rounds * mean + 1.0) + rounds * per_unit + vs * per_split;
+  };
+  int best = base;
+  double best_cost = 0.98 * cost(base);
+  for (int vs = 1; vs <= most; ++vs)
+    if (cost(vs) < best_cost) {
+      best_cost = cost(vs);
+      best = vs;
+    }
+  return best;
+}
+
+// kind: the readout and the top-k modes are the single-operand ones, whose units hold two row
+// blocks.
+alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = kPlanFwd) {
+  const bool two_rows = kind != kPlanFwd;
   alr::LossPlan P{};
   P.N = int(p->N);
   P.d = p->d;
@@ -193,31 +238,27 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, bool two_rows = 
   P.bn = ALR_LOSS_BN;
   P.mc = (!two_rows && loss_multicast(p)) ? 1 : 0;
   // row blocks; row-block pairs for the two-row modes and for the multicast form (which
-  // places sms / 2 clusters).  Forward: the vocabulary splits are sized so that one round of
-  // the grid covers 8 row blocks (152 CTAs / 8 = 19 splits: 32 units per CTA at 256 row
-  // blocks) and a raster group spans two rounds (16 row blocks).  Recomputing backward: one
-  // vocabulary tile per unit, raster groups of 16 row blocks as well.
+  // places sms / 2 clusters).  Forward: the splits of forward_splits (the same for both
+  // forms), in raster groups of up to two rounds of the grid at its base split (16 row blocks).
+  // Recomputing backward: one vocabulary tile per unit, raster groups of 16 row blocks as well.
   const int rb = int((p->N + 127) / 128);
   const bool pairs = P.mc || two_rows;
   P.n_rb = pairs ? (rb + 1) / 2 : rb;
-  const int slots = P.mc ? sms / 2 : sms;
   const int group = pairs ? 4 : 8;
   P.n_vt = (p->V + P.bn - 1) / P.bn;
-  P.group_rows = P.n_rb < group ? P.n_rb : group;
+  // two rounds per raster group: twice the row blocks share each W split, so W leaves DRAM
+  // about half as often, with the same number of units per CTA (forward 49.8 against 50.0 ms at
+  // the text8b size, recomputed logit gradient 46.2 against 46.4 ms with 8, three alternating
+  // A/B rounds)
+  P.group_rows = P.n_rb < 2 * group ? P.n_rb : 2 * group;
   if (bwd) {
     P.n_vs = P.n_vt;  // one tile per unit
-    // 16 row blocks share each W tile (the recomputed logit gradient 46.2 against 46.4 ms
-    // with 8, three alternating A/B rounds)
-    P.group_rows = P.n_rb < 2 * group ? P.n_rb : 2 * group;
   } else {
-    int vs = slots / P.group_rows;
-    if (vs < 1) vs = 1;
-    P.n_vs = vs < P.n_vt ? vs : P.n_vt;
-    // two rounds per raster group: twice the row blocks share each W split, so W leaves
-    // DRAM about half as often, with the same number of units per CTA (forward 49.8 against
-    // 50.0 ms at the text8b size, three alternating A/B rounds)
-    const int wide = 2 * group;
-    P.group_rows = P.n_rb < wide ? P.n_rb : wide;
+    P.n_vs = forward_splits(p, sms, two_rows ? P.n_rb : rb, P.n_vt, two_rows ? 4 : 8, kind);
+    // groups of equal size: 17 row blocks are 9 + 8, not 16 + 1 (in the backward's short units
+    // the smaller groups only cost sharing: 2176 x 2048 x 100000 1071 -> 1105 us)
+    const int n_groups = (P.n_rb + P.group_rows - 1) / P.group_rows;
+    P.group_rows = (P.n_rb + n_groups - 1) / n_groups;
   }
   // partial records per row and split: one per epilogue column group
   P.n_parts = P.n_vs * (P.bn / (two_rows ? 128 : 64));
@@ -234,9 +275,11 @@ struct FwdLayout {
   size_t part_off, anchor_off, ticket_off, wt_off, total;
 };
 
-FwdLayout fwd_layout(const alr_params* p, int sms, int fields = alr::kPFields,
-                     bool two_rows = false) {
-  const alr::LossPlan P = loss_plan(p, sms, false, two_rows);
+FwdLayout fwd_layout(const alr_params* p, int sms, PlanKind kind = kPlanFwd) {
+  const int fields = kind == kPlanFwd       ? alr::kPFields
+                     : kind == kPlanReadout ? alr::kRFields
+                                            : alr::kKFields;
+  const alr::LossPlan P = loss_plan(p, sms, false, kind);
   FwdLayout L{};
   L.part_off = 0;
   L.anchor_off = round_up(size_t(fields) * P.n_parts * size_t(P.N) * sizeof(float), 1024);
@@ -692,7 +735,7 @@ int logit_grad_impl(const alr_params* p, const void* Hd, const void* Ht, const v
       (rc = make_map(&m_gs, G, dt, p->V, p->N, p->V * es, 16, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) != ALR_OK)
     return rc;
   alr::LossArgs args{};
-  args.plan = loss_plan(p, info.sms, true, topk);
+  args.plan = loss_plan(p, info.sms, true, topk ? kPlanTopk : kPlanFwd);
   args.G = G;
   args.lse_d = lse_d;
   args.lse_t = lse_t;
@@ -888,7 +931,7 @@ size_t alr_readout_workspace_size(const alr_params* p) {
   if (check_params(p) != ALR_OK) return 0;
   DevInfo info;
   if (device_info(&info) != ALR_OK) return 0;
-  return fwd_layout(p, info.sms, alr::kRFields, true).total;
+  return fwd_layout(p, info.sms, kPlanReadout).total;
 }
 
 int alr_label_readout(const alr_params* p, const void* Ht, const void* W,
@@ -906,7 +949,7 @@ int alr_label_readout(const alr_params* p, const void* Ht, const void* W,
     return fail(ALR_ERR_INVALID_ARG, "Ht and W must be 16-byte aligned");
   DevInfo info;
   if ((rc = require_sm103(&info)) != ALR_OK) return rc;
-  const FwdLayout lay = fwd_layout(p, info.sms, alr::kRFields, true);
+  const FwdLayout lay = fwd_layout(p, info.sms, kPlanReadout);
   if ((rc = check_workspace(workspace, ws_bytes, lay.total)) != ALR_OK) return rc;
   const int dt = p->dtype;
   const size_t es = elem_size(dt);
@@ -916,7 +959,7 @@ int alr_label_readout(const alr_params* p, const void* Ht, const void* W,
   if ((rc = make_map(&m_h, Ht, dt, p->d, p->N, p->d * es, k_per_row(dt), 128)) != ALR_OK) return rc;
   if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, s)) != ALR_OK) return rc;
   alr::LossArgs args{};
-  args.plan = loss_plan(p, info.sms, false, true);
+  args.plan = loss_plan(p, info.sms, false, kPlanReadout);
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
   args.corpus_tok = corpus_tok;
   args.status = alr::device_status_ptr();
@@ -933,7 +976,7 @@ size_t alr_topk_fwd_workspace_size(const alr_params* p) {
   if (check_params(p) != ALR_OK) return 0;
   DevInfo info;
   if (device_info(&info) != ALR_OK) return 0;
-  return fwd_layout(p, info.sms, alr::kKFields, true).total;
+  return fwd_layout(p, info.sms, kPlanTopk).total;
 }
 
 }  // extern "C"
@@ -957,7 +1000,7 @@ int topk_fwd_impl(const alr_params* p, const void* Hd, const void* W, const int3
     return fail(ALR_ERR_INVALID_ARG, "Hd and W must be 16-byte aligned");
   DevInfo info;
   if ((rc = require_sm103(&info)) != ALR_OK) return rc;
-  const FwdLayout lay = fwd_layout(p, info.sms, alr::kKFields, true);
+  const FwdLayout lay = fwd_layout(p, info.sms, kPlanTopk);
   if ((rc = check_workspace(workspace, ws_bytes, lay.total)) != ALR_OK) return rc;
   const int dt = p->dtype;
   const size_t es = elem_size(dt);
@@ -967,7 +1010,7 @@ int topk_fwd_impl(const alr_params* p, const void* Hd, const void* W, const int3
   if ((rc = make_map(&m_h, Hd, dt, p->d, p->N, p->d * es, k_per_row(dt), 128)) != ALR_OK) return rc;
   if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, s)) != ALR_OK) return rc;
   alr::LossArgs args{};
-  args.plan = loss_plan(p, info.sms, false, true);
+  args.plan = loss_plan(p, info.sms, false, kPlanTopk);
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
   args.ticket = reinterpret_cast<unsigned*>(ws + lay.ticket_off);
   args.top_idx = top_idx;

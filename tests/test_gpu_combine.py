@@ -90,3 +90,32 @@ def test_readout_and_topk_merge(A, B):
     np.testing.assert_allclose(float(out["loss_total"].item()), (w * l).sum() / w.sum(),
                                rtol=2.0 ** -22)
     assert alr.alr_device_status() == alr.ALR_OK
+
+
+@pytest.mark.parametrize("N", [1104, 2080])
+def test_forward_at_uneven_row_blocks(N):
+    """9 and 17 row blocks: the split count and the raster groups (9 + 8) that fill the SMs."""
+    B, d, V = 16, 64, 20000
+    b = synthetic.sharpen(synthetic.slot_batch(d, V, N // B, B, 0.5, dtype=torch.bfloat16,
+                                               device="cuda", seed=N))
+    r = orc.slot_loss_forward(P.np64(b["Hd"]), P.np64(b["Ht"]), P.np64(b["W"]), B)
+    P.compare_forward(P.fwd_to_numpy(P.gpu_forward(b["Hd"], b["Ht"], b["W"], B)), r)
+    z = orc.label_readout(P.np64(b["Ht"]), P.np64(b["W"]), k=T.K)
+    T.compare_readout(T.gpu_readout(b["Ht"], b["W"], B), z)
+    assert alr.alr_device_status() == alr.ALR_OK
+
+
+def test_forward_workspace_stays_within_the_fixed_scratch():
+    """Every bf16 problem whose records at 19 splits (15 fp32 fields per row, split and
+    64-column group: what the no-workspace forward's limit was set for) fit the fixed 64 MiB
+    still fits, whatever split count its row blocks take."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    limit = 64 << 20
+    up = lambda x: (x + 1023) // 1024 * 1024  # noqa: E731
+    for N in list(range(16, 4096, 112)) + list(range(4096, 16000, 592)):
+        for d, V in ((64, 1000), (1000, 60000), (4096, 151936)):
+            n_vt, rb = (V + 255) // 256, (N + 127) // 128
+            vs = min(n_vt, max(1, sms // min(rb, 8)))
+            start = up(15 * 4 * vs * 4 * N) + up(16 * (N // 16))
+            need = alr.alr_fwd_workspace_size(alr.make_params(N, d, V, 16))
+            assert 0 < need <= max(limit, start), (N, d, V, need, start)
