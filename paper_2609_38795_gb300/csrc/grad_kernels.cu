@@ -20,10 +20,19 @@ namespace {
 // before the thread that read it overwrites it, and no other thread touches it.  Masked rows
 // (c_r = 0) read nothing.
 constexpr int kLogitsUnroll = 4;
-constexpr int kGradRows = 32;
+constexpr int kGradRows = 32;              // most rows of a block
 constexpr int kGradCols = 2048;
-constexpr int kGradGroups = kGradCols / kKeepGroup;
 constexpr int kGradThreads = kGradCols / 8;
+
+// Rows per block: 32 where that gives eight blocks to each of 152 SMs, else halved down to one
+// pass of kLogitsUnroll rows, since the passes of a block follow one another, each a memory
+// round trip (192 rows of V = 1400: 6 blocks of 8 passes took 11.9 us, now 3.7).
+inline int grad_rows(int N, int V) {
+  const long long cols = (V + kGradCols - 1) / kGradCols;
+  int rows = kGradRows;
+  while (rows > kLogitsUnroll && (N + rows - 1) / rows * cols < 8 * 152) rows /= 2;
+  return rows;
+}
 
 // 8 kept logits as loaded: fp16 (bf16 inputs) or fp32 (fp32 inputs).
 template <typename Z>
@@ -103,10 +112,10 @@ __global__ void __launch_bounds__(kGradThreads) logits_grad_kernel(
     const Z* zd, const Z* zt, const uint16_t* __restrict__ zd_ref,
     const uint16_t* __restrict__ zt_ref, const float* __restrict__ lse_d,
     const float* __restrict__ lse_t, const float* __restrict__ weight,
-    const float* __restrict__ weight_sum, float lam, int N, int V, Gt* G) {
+    const float* __restrict__ weight_sum, float lam, int N, int V, int rows, Gt* G) {
   __shared__ float s_c[kGradRows], s_ad[kGradRows], s_at[kGradRows];
-  const int r0 = blockIdx.x * kGradRows, c0 = blockIdx.y * kGradCols;
-  const int nr = min(kGradRows, N - r0), nc = min(kGradCols, V - c0);
+  const int r0 = blockIdx.x * rows, c0 = blockIdx.y * kGradCols;
+  const int nr = min(rows, N - r0), nc = min(kGradCols, V - c0);
   if (threadIdx.x < nr) {
     const int r = r0 + threadIdx.x;
     s_c[threadIdx.x] = row_factor(weight, weight_sum, lam, r);
@@ -162,13 +171,13 @@ __global__ void __launch_bounds__(kGradThreads) topk_logits_grad_kernel(
     const float* __restrict__ top_prob, const float* __restrict__ tail,
     const float* __restrict__ tail_q, const float* __restrict__ lse_d,
     const float* __restrict__ weight, const float* __restrict__ weight_sum, float lam, int N,
-    int V, Gt* G) {
+    int V, int rows, Gt* G) {
   static_assert(kGradRows * kTopK <= kGradThreads, "one thread per label of the block's rows");
   __shared__ float s_c[kGradRows], s_cb[kGradRows], s_ad[kGradRows];
   __shared__ float lab_g[kGradRows * kTopK];
   __shared__ int lab_v[kGradRows * kTopK];
-  const int r0 = blockIdx.x * kGradRows, c0 = blockIdx.y * kGradCols;
-  const int nr = min(kGradRows, N - r0), nc = min(kGradCols, V - c0);
+  const int r0 = blockIdx.x * rows, c0 = blockIdx.y * kGradCols;
+  const int nr = min(rows, N - r0), nc = min(kGradCols, V - c0);
   if (threadIdx.x < nr) {
     const int r = r0 + threadIdx.x;
     const float c = row_factor(weight, weight_sum, lam, r);
@@ -239,15 +248,16 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
                                     const float* tail, const float* tail_q, const float* lse_d,
                                     const float* weight, const float* weight_sum, float lam, int N,
                                     int V, void* G, cudaStream_t s) {
-  const dim3 grid(unsigned((N + kGradRows - 1) / kGradRows), unsigned((V + kGradCols - 1) / kGradCols));
+  const int rows = grad_rows(N, V);
+  const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
     topk_logits_grad_kernel<__half, __nv_bfloat16><<<grid, kGradThreads, 0, s>>>(
         static_cast<const __half*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
-        weight_sum, lam, N, V, static_cast<__nv_bfloat16*>(G));
+        weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
   else
     topk_logits_grad_kernel<float, float><<<grid, kGradThreads, 0, s>>>(
         static_cast<const float*>(zd), nullptr, top_idx, top_prob, tail, tail_q, lse_d, weight,
-        weight_sum, lam, N, V, static_cast<float*>(G));
+        weight_sum, lam, N, V, rows, static_cast<float*>(G));
   return cudaGetLastError();
 }
 
@@ -255,15 +265,16 @@ cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const 
                                const uint16_t* zt_ref, const float* lse_d, const float* lse_t,
                                const float* weight, const float* weight_sum, float lam, int N,
                                int V, void* G, cudaStream_t s) {
-  const dim3 grid(unsigned((N + kGradRows - 1) / kGradRows), unsigned((V + kGradCols - 1) / kGradCols));
+  const int rows = grad_rows(N, V);
+  const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
     logits_grad_kernel<__half, __nv_bfloat16><<<grid, kGradThreads, 0, s>>>(
         static_cast<const __half*>(zd), static_cast<const __half*>(zt), zd_ref, zt_ref, lse_d,
-        lse_t, weight, weight_sum, lam, N, V, static_cast<__nv_bfloat16*>(G));
+        lse_t, weight, weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
   else
     logits_grad_kernel<float, float><<<grid, kGradThreads, 0, s>>>(
         static_cast<const float*>(zd), static_cast<const float*>(zt), nullptr, nullptr, lse_d,
-        lse_t, weight, weight_sum, lam, N, V, static_cast<float*>(G));
+        lse_t, weight, weight_sum, lam, N, V, rows, static_cast<float*>(G));
   return cudaGetLastError();
 }
 

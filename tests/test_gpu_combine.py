@@ -119,3 +119,23 @@ def test_forward_workspace_stays_within_the_fixed_scratch():
             start = up(15 * 4 * vs * 4 * N) + up(16 * (N // 16))
             need = alr.alr_fwd_workspace_size(alr.make_params(N, d, V, 16))
             assert 0 < need <= max(limit, start), (N, d, V, need, start)
+
+
+@pytest.mark.parametrize("B", [1, 15, 32])
+@pytest.mark.parametrize("A", [1, 2, 31, 256, 257])
+def test_accept_len_block_edges(A, B):
+    """One block up to 256 anchors (1, 2, 31 and 32 warps), one warp per anchor of many past it."""
+    g = torch.Generator(device="cuda").manual_seed(A + B)
+    t = torch.randint(0, 50, (A * B,), generator=g, device="cuda", dtype=torch.int32)
+    same = torch.rand(A * B, generator=g, device="cuda") < 0.8
+    d = torch.where(same, t, t + 1)
+    active = (torch.rand(A * B, generator=g, device="cuda") < 0.95).float()
+    acc = torch.full((A,), -1, dtype=torch.int32, device="cuda")
+    hist = torch.full((B + 1,), -1, dtype=torch.int64, device="cuda")
+    for w in (active, None):
+        alr.alr_accept_len(d, t, B, acc, hist, active=w)
+        torch.cuda.synchronize()
+        ok = same if w is None else same & (w > 0)
+        want = ok.view(A, B).int().cumprod(1).sum(1)
+        assert torch.equal(acc, want.to(torch.int32))
+        assert torch.equal(hist, torch.bincount(want, minlength=B + 1))
