@@ -12,6 +12,7 @@
 #include <cfloat>
 
 #include "kernels.h"
+#include "launch.h"
 #include "tc_common.cuh"
 
 namespace alr {
@@ -276,8 +277,9 @@ struct MergeSmem {
 // Merge all partial records of this block's rows [row0, row0 + n_rows), n_rows <= kRows, into
 // sm.get(0, row - row0).  Every thread of the block calls it; it ends with a block barrier.
 template <class St, int kRows, int kWarps>
-ALR_DEV void merge_rows(const LossPlan& P, const float* __restrict__ part, int row0, int n_rows,
+ALR_DEV void merge_rows(const LossPlan& P, const float* part, int row0, int n_rows,
                         MergeSmem<St, kRows, kWarps>& sm) {
+  pdl_wait_and_release();
   constexpr int kSlots = 32 / kRows;       // records of a row read by one warp at a time
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rr = lane % kRows, slot = lane / kRows;
@@ -398,9 +400,9 @@ struct FullOut {
 
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps)
-    combine_kernel(LossPlan P, const float* __restrict__ part, int rows_per_block, int mode,
-                   float gamma, const float* __restrict__ row_mask,
-                   const int32_t* __restrict__ corpus_tok, FullOut o, BatchOut bo) {
+    combine_kernel(LossPlan P, const float* part, int rows_per_block, int mode,
+                   float gamma, const float* row_mask,
+                   const int32_t* corpus_tok, FullOut o, BatchOut bo) {
   __shared__ MergeSmem<FullState, kRows, kWarps> sm;
   __shared__ float s_loss[kRows], s_logp[kRows];
   const int row0 = blockIdx.x * rows_per_block;
@@ -460,11 +462,11 @@ __global__ void __launch_bounds__(32 * kWarps)
 // gap, and log p at the corpus token.  Rows are independent.
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps)
-    readout_combine_kernel(LossPlan P, const float* __restrict__ part, int has_corpus,
-                           int32_t* __restrict__ top_idx, float* __restrict__ top_prob,
-                           float* __restrict__ tail, float* __restrict__ lse_t,
-                           int32_t* __restrict__ argmax_t, float* __restrict__ gap_t,
-                           float* __restrict__ logp_x) {
+    readout_combine_kernel(LossPlan P, const float* part, int has_corpus,
+                           int32_t* top_idx, float* top_prob,
+                           float* tail, float* lse_t,
+                           int32_t* argmax_t, float* gap_t,
+                           float* logp_x) {
   static_assert(kRows * kTopK <= 32 * kWarps, "one thread per label");
   __shared__ MergeSmem<ReadoutState, kRows, kWarps> sm;
   __shared__ double s_e[kTopK][kRows];
@@ -518,9 +520,9 @@ struct TopkOut {
 
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps)
-    topk_combine_kernel(LossPlan P, const float* __restrict__ part, int rows_per_block,
-                        const float* __restrict__ top_prob, const float* __restrict__ tail,
-                        const float* __restrict__ row_mask, const float* __restrict__ weight_in,
+    topk_combine_kernel(LossPlan P, const float* part, int rows_per_block,
+                        const float* top_prob, const float* tail,
+                        const float* row_mask, const float* weight_in,
                         float gamma, TopkOut o, BatchOut bo) {
   __shared__ MergeSmem<TopkState, kRows, kWarps> sm;
   const int row0 = blockIdx.x * rows_per_block;
@@ -592,9 +594,8 @@ cudaError_t launch_combine(const LossPlan& plan, const float* part, int mode, fl
               : m.rows == 8  ? combine_kernel<8, 16>
               : m.rows == 16 ? combine_kernel<16, 16>
                              : combine_kernel<32, 16>;
-  kern<<<m.blocks, 32 * m.warps, 0, s>>>(plan, part, m.rows_per_block, mode, gamma, row_mask,
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, mode, gamma, row_mask,
                                        corpus_tok, o, b);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool has_corpus,
@@ -603,9 +604,8 @@ cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool
                                    cudaStream_t s) {
   const MergeShape m = merge_shape(plan.N, 1);
   auto kern = m.warps == 8 ? readout_combine_kernel<32, 8> : readout_combine_kernel<8, 16>;
-  kern<<<m.blocks, 32 * m.warps, 0, s>>>(plan, part, has_corpus ? 1 : 0, top_idx, top_prob, tail,
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, has_corpus ? 1 : 0, top_idx, top_prob, tail,
                                          lse_t, argmax_t, gap_t, logp_x);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const float* top_prob,
@@ -622,9 +622,8 @@ cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const f
               : m.rows == 8  ? topk_combine_kernel<8, 16>
               : m.rows == 16 ? topk_combine_kernel<16, 16>
                              : topk_combine_kernel<32, 16>;
-  kern<<<m.blocks, 32 * m.warps, 0, s>>>(plan, part, m.rows_per_block, top_prob, tail, row_mask,
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, top_prob, tail, row_mask,
                                        weight_in, gamma, o, b);
-  return cudaGetLastError();
 }
 
 }  // namespace alr

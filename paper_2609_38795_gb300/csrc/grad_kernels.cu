@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 
 #include "kernels.h"
+#include "launch.h"
 #include "tc_common.cuh"
 
 namespace alr {
@@ -109,11 +110,12 @@ __device__ __forceinline__ float row_factor(const float* weight, const float* we
 
 template <typename Z, typename Gt>
 __global__ void __launch_bounds__(kGradThreads) logits_grad_kernel(
-    const Z* zd, const Z* zt, const uint16_t* __restrict__ zd_ref,
-    const uint16_t* __restrict__ zt_ref, const float* __restrict__ lse_d,
-    const float* __restrict__ lse_t, const float* __restrict__ weight,
-    const float* __restrict__ weight_sum, float lam, int N, int V, int rows, Gt* G) {
+    const Z* zd, const Z* zt, const uint16_t* zd_ref,
+    const uint16_t* zt_ref, const float* lse_d,
+    const float* lse_t, const float* weight,
+    const float* weight_sum, float lam, int N, int V, int rows, Gt* G) {
   __shared__ float s_c[kGradRows], s_ad[kGradRows], s_at[kGradRows];
+  pdl_wait_and_release();
   const int r0 = blockIdx.x * rows, c0 = blockIdx.y * kGradCols;
   const int nr = min(rows, N - r0), nc = min(kGradCols, V - c0);
   if (threadIdx.x < nr) {
@@ -167,15 +169,16 @@ __global__ void __launch_bounds__(kGradThreads) logits_grad_kernel(
 // buffer).  The label tokens of a row are distinct.
 template <typename Z, typename Gt>
 __global__ void __launch_bounds__(kGradThreads) topk_logits_grad_kernel(
-    const Z* zd, const uint16_t* __restrict__ zd_ref, const int32_t* __restrict__ top_idx,
-    const float* __restrict__ top_prob, const float* __restrict__ tail,
-    const float* __restrict__ tail_q, const float* __restrict__ lse_d,
-    const float* __restrict__ weight, const float* __restrict__ weight_sum, float lam, int N,
+    const Z* zd, const uint16_t* zd_ref, const int32_t* top_idx,
+    const float* top_prob, const float* tail,
+    const float* tail_q, const float* lse_d,
+    const float* weight, const float* weight_sum, float lam, int N,
     int V, int rows, Gt* G) {
   static_assert(kGradRows * kTopK <= kGradThreads, "one thread per label of the block's rows");
   __shared__ float s_c[kGradRows], s_cb[kGradRows], s_ad[kGradRows];
   __shared__ float lab_g[kGradRows * kTopK];
   __shared__ int lab_v[kGradRows * kTopK];
+  pdl_wait_and_release();
   const int r0 = blockIdx.x * rows, c0 = blockIdx.y * kGradCols;
   const int nr = min(rows, N - r0), nc = min(kGradCols, V - c0);
   if (threadIdx.x < nr) {
@@ -251,14 +254,12 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
   const int rows = grad_rows(N, V);
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
-    topk_logits_grad_kernel<__half, __nv_bfloat16><<<grid, kGradThreads, 0, s>>>(
+    return launch_pdl(topk_logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
         static_cast<const __half*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
         weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
-  else
-    topk_logits_grad_kernel<float, float><<<grid, kGradThreads, 0, s>>>(
-        static_cast<const float*>(zd), nullptr, top_idx, top_prob, tail, tail_q, lse_d, weight,
+  return launch_pdl(topk_logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+        static_cast<const float*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
         weight_sum, lam, N, V, rows, static_cast<float*>(G));
-  return cudaGetLastError();
 }
 
 cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const uint16_t* zd_ref,
@@ -268,14 +269,12 @@ cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const 
   const int rows = grad_rows(N, V);
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
-    logits_grad_kernel<__half, __nv_bfloat16><<<grid, kGradThreads, 0, s>>>(
+    return launch_pdl(logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
         static_cast<const __half*>(zd), static_cast<const __half*>(zt), zd_ref, zt_ref, lse_d,
         lse_t, weight, weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
-  else
-    logits_grad_kernel<float, float><<<grid, kGradThreads, 0, s>>>(
-        static_cast<const float*>(zd), static_cast<const float*>(zt), nullptr, nullptr, lse_d,
+  return launch_pdl(logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+        static_cast<const float*>(zd), static_cast<const float*>(zt), zd_ref, zt_ref, lse_d,
         lse_t, weight, weight_sum, lam, N, V, rows, static_cast<float*>(G));
-  return cudaGetLastError();
 }
 
 }  // namespace alr

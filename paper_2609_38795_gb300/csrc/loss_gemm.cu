@@ -2,6 +2,7 @@
 // single-CTA forms, built here; the cluster form of the dual modes is launched through
 // libalr_cluster.so (cluster_forms.h).
 #include "cluster_forms.h"
+#include "launch.h"
 #include "loss_gemm_kernel.cuh"
 
 namespace alr {
@@ -16,8 +17,7 @@ cudaError_t launch_impl(const CUtensorMap& a0, const CUtensorMap& a1, const CUte
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kSmem));
   if (e != cudaSuccess) return e;
-  kern<<<args.plan.grid, S::kThreads, S::kSmem, s>>>(a0, a1, w, g, g2, args);
-  return cudaGetLastError();
+  return launch_pdl(kern, args.plan.grid, S::kThreads, S::kSmem, s, a0, a1, w, g, g2, args);
 }
 
 template <typename Elem, int kMode>

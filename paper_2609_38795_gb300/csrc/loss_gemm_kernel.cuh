@@ -505,7 +505,6 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
     }
     mbar_init(drain_bar, 1);
     *abort_word = 0;
-    if (blockIdx.x == 0 && args.ticket != nullptr) *args.ticket = 0u;
     fence_mbar_init();
   }
   if (threadIdx.x == 32) {
@@ -520,6 +519,8 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
     tmem_relinquish();
   }
   tc_fence_before();
+  pdl_wait_and_release();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && args.ticket != nullptr) *args.ticket = 0u;
   __syncthreads();
   if constexpr (kMc) cluster_sync();   // the peer's copies and commits find initialised barriers
   tc_fence_after();

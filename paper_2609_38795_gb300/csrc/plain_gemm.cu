@@ -3,12 +3,14 @@
 // (cluster_forms.h).
 #include <atomic>
 
+#include "launch.h"
 #include "plain_gemm_kernel.cuh"
 
 namespace alr {
 namespace {
 
-// Launch configuration of a split-K cluster of n_cta CTAs (attr must outlive the launch).
+// Launch configuration of a split-K cluster of n_cta CTAs (attr, two entries, must outlive the
+// launch).
 cudaLaunchConfig_t split_config(cudaLaunchAttribute* attr, int n_cta, int n_tiles, cudaStream_t s) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = unsigned(n_cta);
@@ -19,8 +21,9 @@ cudaLaunchConfig_t split_config(cudaLaunchAttribute* attr, int n_cta, int n_tile
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cfg;
 }
 
@@ -38,7 +41,7 @@ cudaError_t launch_split_t(const CUtensorMap& a, const CUtensorMap& b, const Gem
   auto kern = plain_gemm_kernel<Elem, kAMN, kBMN, kAcc, SplitCluster>;
   cudaError_t e = split_attributes(kern);
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = split_config(attr, args.split, args.n_tiles, s);
   return cudaLaunchKernelEx(&cfg, kern, a, b, args);
 }
@@ -51,8 +54,7 @@ cudaError_t launch_t(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs&
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
-  kern<<<args.grid, kThreads, kSmemBytes, s>>>(a, b, args);
-  return cudaGetLastError();
+  return launch_pdl(kern, args.grid, kThreads, kSmemBytes, s, a, b, args);
 }
 
 template <typename Elem>
@@ -89,7 +91,7 @@ int plain_gemm_split_clusters(int n_cta) {
   const int known = cached[dev][n_cta].load(std::memory_order_relaxed);
   if (known != 0) return known > 0 ? known : 0;
   auto kern = plain_gemm_kernel<__nv_bfloat16, false, false, false, SplitCluster>;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = split_config(attr, n_cta, 1, nullptr);
   int n = 0;
   if (split_attributes(kern) != cudaSuccess ||

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
   }
   tc_fence_before();
+  pdl_wait_and_release();
   __syncthreads();
   if constexpr (kMc) cluster_sync();   // the peer's copies and commits find initialised barriers
   tc_fence_after();

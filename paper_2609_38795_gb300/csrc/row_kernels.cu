@@ -4,6 +4,7 @@
 // grad_kernels.cu.)
 
 #include "kernels.h"
+#include "launch.h"
 #include "tc_common.cuh"
 
 namespace alr {
@@ -13,32 +14,6 @@ namespace {
 // One warp per output row; each lane moves 16-byte vectors, issuing a batch of loads before
 // the matching stores so that many requests are in flight per SM.
 constexpr int kGatherBatch = 16;
-
-// Programmatic dependent launch of the gathers: each is launched so that it may be scheduled
-// while the kernel before it in the stream is still running, waits (griddepcontrol.wait) until
-// that kernel has completed and its writes are visible before touching global memory, and
-// lets the kernel after it be scheduled early in turn.  A kernel launched without the
-// attribute, or preceded by one that never triggers, behaves as under plain stream order.
-ALR_DEV void pdl_wait_and_release() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, cudaStream_t s,
-                       Args... args) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
 
 __global__ void __launch_bounds__(256) gather_kernel(const uint4* __restrict__ feat, int S, int L,
                                                      int vec_per_row,
@@ -101,9 +76,10 @@ __device__ __forceinline__ float gate_for_lane(bool active, int lane, bool hard,
 
 // Eq. 1 from sums that the caller reduced over the shards of a batch: L = lambda * wl / ws,
 // 0 when ws = 0 (no supervised slot anywhere in the batch).
-__global__ void loss_from_sums_kernel(const float* __restrict__ wl_sum,
-                                      const float* __restrict__ weight_sum, float lam,
-                                      float* __restrict__ loss_total) {
+__global__ void loss_from_sums_kernel(const float* wl_sum,
+                                      const float* weight_sum, float lam,
+                                      float* loss_total) {
+  pdl_wait_and_release();
   const double ws = *weight_sum;
   *loss_total = ws > 0.0 ? float(double(lam) * double(*wl_sum) / ws) : 0.f;
 }
@@ -111,8 +87,8 @@ __global__ void loss_from_sums_kernel(const float* __restrict__ wl_sum,
 // ------------------------------------------------------------- accepted length ---
 // One warp per anchor: the count of leading slots whose greedy drafter token equals the
 // greedy target token (and whose row is active).
-ALR_DEV int accepted_slots(const int32_t* __restrict__ am_d, const int32_t* __restrict__ am_t,
-                           const float* __restrict__ active_w, int a, int B, int lane) {
+ALR_DEV int accepted_slots(const int32_t* am_d, const int32_t* am_t,
+                           const float* active_w, int a, int B, int lane) {
   bool ok = false;
   if (lane < B) {
     const int r = a * B + lane;
@@ -123,11 +99,12 @@ ALR_DEV int accepted_slots(const int32_t* __restrict__ am_d, const int32_t* __re
   return bal == 0xffffffffu ? 32 : __ffs(~bal) - 1;
 }
 
-__global__ void __launch_bounds__(256) accept_len_kernel(const int32_t* __restrict__ am_d,
-                                                         const int32_t* __restrict__ am_t,
-                                                         const float* __restrict__ active_w,
-                                                         int A, int B, int32_t* __restrict__ acc,
-                                                         unsigned long long* __restrict__ hist) {
+__global__ void __launch_bounds__(256) accept_len_kernel(const int32_t* am_d,
+                                                         const int32_t* am_t,
+                                                         const float* active_w,
+                                                         int A, int B, int32_t* acc,
+                                                         unsigned long long* hist) {
+  pdl_wait_and_release();
   const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (a >= A) return;
@@ -144,10 +121,11 @@ __global__ void __launch_bounds__(256) accept_len_kernel(const int32_t* __restri
 constexpr int kAcceptOneBlock = 256;
 
 __global__ void __launch_bounds__(1024) accept_len_one_block_kernel(
-    const int32_t* __restrict__ am_d, const int32_t* __restrict__ am_t,
-    const float* __restrict__ active_w, int A, int B, int32_t* __restrict__ acc,
-    unsigned long long* __restrict__ hist) {
+    const int32_t* am_d, const int32_t* am_t,
+    const float* active_w, int A, int B, int32_t* acc,
+    unsigned long long* hist) {
   __shared__ int count[33];
+  pdl_wait_and_release();
   const int lane = threadIdx.x & 31, n_warps = blockDim.x / 32;
   if (threadIdx.x < 32) {
     count[threadIdx.x] = 0;
@@ -168,9 +146,10 @@ __global__ void __launch_bounds__(1024) accept_len_one_block_kernel(
 
 // ---------------------------------------------------------- erase weights ---
 __global__ void __launch_bounds__(256) erase_weights_kernel(
-    const float* __restrict__ logp_x, const int32_t* __restrict__ corpus_tok,
-    const int32_t* __restrict__ argmax_t, const float* __restrict__ row_mask, int A, int B,
-    float gamma, int hard, float* __restrict__ weight) {
+    const float* logp_x, const int32_t* corpus_tok,
+    const int32_t* argmax_t, const float* row_mask, int A, int B,
+    float gamma, int hard, float* weight) {
+  pdl_wait_and_release();
   const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (a >= A) return;
@@ -196,11 +175,12 @@ __global__ void __launch_bounds__(256) erase_weights_kernel(
 // primary i's rollout at offset j.  Emits the label-row gather (seq, pos, valid_len) over
 // the primary label buffer [S * P, K, d], the anchor token and the rollout context length.
 __global__ void __launch_bounds__(256) ira_blocks_kernel(
-    int S, int K, int max_blocks, const int32_t* __restrict__ valid_anchors,
-    const int32_t* __restrict__ rollout_len, const int32_t* __restrict__ offsets,
-    const int32_t* __restrict__ rollout_tok, const int32_t* __restrict__ corpus_anchor_tok,
-    int32_t* __restrict__ seq, int32_t* __restrict__ pos, int32_t* __restrict__ vlen,
-    int32_t* __restrict__ ctx_len, int32_t* __restrict__ anchor_tok) {
+    int S, int K, int max_blocks, const int32_t* valid_anchors,
+    const int32_t* rollout_len, const int32_t* offsets,
+    const int32_t* rollout_tok, const int32_t* corpus_anchor_tok,
+    int32_t* seq, int32_t* pos, int32_t* vlen,
+    int32_t* ctx_len, int32_t* anchor_tok) {
+  pdl_wait_and_release();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)S * max_blocks) return;
   const int s = int(t / max_blocks), b = int(t - (long long)s * max_blocks);
@@ -255,12 +235,13 @@ using Pair = unsigned long long;           // key << 32 | position
 constexpr Pair kNoPair = ~0ull;            // an invalid position (no valid one: position < 2^14)
 
 __global__ void __launch_bounds__(kDrawThreads)
-    ira_draw_kernel(int L, int K, int max_blocks, const uint8_t* __restrict__ anchor_ok,
-                    const uint32_t* __restrict__ keys, const uint32_t* __restrict__ offset_u,
-                    int32_t* __restrict__ n_valid, int32_t* __restrict__ anchor_pos,
-                    int32_t* __restrict__ offsets) {
+    ira_draw_kernel(int L, int K, int max_blocks, const uint8_t* anchor_ok,
+                    const uint32_t* keys, const uint32_t* offset_u,
+                    int32_t* n_valid, int32_t* anchor_pos,
+                    int32_t* offsets) {
   extern __shared__ Pair cand[];           // [L]
   __shared__ int hist[256], s_valid, s_cand, s_digit, s_below, s_in;
+  pdl_wait_and_release();
   const int s = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const size_t row = size_t(s) * size_t(L);
   if (tid < 256) hist[tid] = 0;
@@ -403,10 +384,11 @@ __global__ void __launch_bounds__(256) ira_context_kernel(
 
 // ------------------------------------------------------------------ transpose ---
 // out[c * ld_out + r] = in[r * C + c] for 32-bit elements, 32 x 32 tiles through shared memory.
-__global__ void __launch_bounds__(256) transpose32_kernel(const float* __restrict__ in,
-                                                          float* __restrict__ out, int R, int C,
+__global__ void __launch_bounds__(256) transpose32_kernel(const float* in,
+                                                          float* out, int R, int C,
                                                           int ld_out) {
   __shared__ float tile[32][33];
+  pdl_wait_and_release();
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int i = threadIdx.y; i < 32; i += 8) {
     const int r = r0 + i, c = c0 + threadIdx.x;
@@ -427,10 +409,9 @@ cudaError_t launch_ira_blocks(int S, int K, int max_blocks, const int32_t* valid
                               int32_t* seq, int32_t* pos, int32_t* vlen, int32_t* ctx_len,
                               int32_t* anchor_tok, cudaStream_t s) {
   const long long n = (long long)S * max_blocks;
-  ira_blocks_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(
-      S, K, max_blocks, valid_anchors, rollout_len, offsets, rollout_tok, corpus_anchor_tok, seq,
+  return launch_pdl(
+      ira_blocks_kernel, unsigned((n + 255) / 256), 256, 0, s, S, K, max_blocks, valid_anchors, rollout_len, offsets, rollout_tok, corpus_anchor_tok, seq,
       pos, vlen, ctx_len, anchor_tok);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_ira_draw(int S, int L, int K, int max_blocks, const uint8_t* anchor_ok,
@@ -441,9 +422,8 @@ cudaError_t launch_ira_draw(int S, int L, int K, int max_blocks, const uint8_t* 
                                        int(smem));
   if (e != cudaSuccess) return e;
   const int threads = L <= 256 ? 256 : L <= 512 ? 512 : kDrawThreads;
-  ira_draw_kernel<<<S, threads, smem, s>>>(L, K, max_blocks, anchor_ok, keys, offset_u, n_valid,
+  return launch_pdl(ira_draw_kernel, S, threads, smem, s, L, K, max_blocks, anchor_ok, keys, offset_u, n_valid,
                                         anchor_pos, offsets);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_ira_context(const void* store, int C, int F, int elem_bytes, int S, int K,
@@ -453,7 +433,7 @@ cudaError_t launch_ira_context(const void* store, int C, int F, int elem_bytes, 
   const long long rows = (long long)S * (max_blocks / 2) * C;
   const int vec = int((long long)F * elem_bytes / 16);
   if (rows == 0) return cudaSuccess;
-  return launch_pdl(ira_context_kernel, unsigned((rows + 7) / 8), 256, s,
+  return launch_pdl(ira_context_kernel, unsigned((rows + 7) / 8), 256, 0, s,
                     static_cast<const uint4*>(store), C, vec, S, K, max_blocks, n_valid,
                     rollout_len, offsets, anchor_pos, static_cast<uint4*>(ctx), ctx_len,
                     prefix_end);
@@ -462,8 +442,7 @@ cudaError_t launch_ira_context(const void* store, int C, int F, int elem_bytes, 
 cudaError_t launch_transpose32(const float* in, float* out, int R, int C, int ld_out,
                                cudaStream_t s) {
   dim3 grid((C + 31) / 32, (R + 31) / 32);
-  transpose32_kernel<<<grid, dim3(32, 8), 0, s>>>(in, out, R, C, ld_out);
-  return cudaGetLastError();
+  return launch_pdl(transpose32_kernel, grid, dim3(32, 8), 0, s, in, out, R, C, ld_out);
 }
 
 cudaError_t launch_gather(const void* feat, int S, int L, int d, int elem_bytes,
@@ -473,14 +452,13 @@ cudaError_t launch_gather(const void* feat, int S, int L, int d, int elem_bytes,
   const int vec = int((long long)d * elem_bytes / 16);
   const long long blocks = (rows + 7) / 8;
   if (blocks == 0) return cudaSuccess;
-  return launch_pdl(gather_kernel, unsigned(blocks), 256, s, static_cast<const uint4*>(feat), S,
+  return launch_pdl(gather_kernel, unsigned(blocks), 256, 0, s, static_cast<const uint4*>(feat), S,
                     L, vec, seq, pos, valid_len, A, B, static_cast<uint4*>(out), row_valid);
 }
 
 cudaError_t launch_loss_from_sums(const float* wl_sum, const float* weight_sum, float lam,
                                   float* loss_total, cudaStream_t s) {
-  loss_from_sums_kernel<<<1, 1, 0, s>>>(wl_sum, weight_sum, lam, loss_total);
-  return cudaGetLastError();
+  return launch_pdl(loss_from_sums_kernel, 1, 1, 0, s, wl_sum, weight_sum, lam, loss_total);
 }
 
 cudaError_t launch_accept_len(const int32_t* am_d, const int32_t* am_t, const float* active,
@@ -489,23 +467,21 @@ cudaError_t launch_accept_len(const int32_t* am_d, const int32_t* am_t, const fl
   if (A <= kAcceptOneBlock) {
     // at least 33 threads: one per histogram entry
     const int threads = A < 2 ? 64 : A < 32 ? 32 * A : 1024;
-    accept_len_one_block_kernel<<<1, threads, 0, s>>>(am_d, am_t, active, A, B, acc, h);
-    return cudaGetLastError();
+    return launch_pdl(accept_len_one_block_kernel, 1, threads, 0, s, am_d, am_t, active, A, B, acc,
+                      h);
   }
   if (hist != nullptr) {
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int64_t) * size_t(B + 1), s);
     if (e != cudaSuccess) return e;
   }
-  accept_len_kernel<<<(A + 7) / 8, 256, 0, s>>>(am_d, am_t, active, A, B, acc, h);
-  return cudaGetLastError();
+  return launch_pdl(accept_len_kernel, (A + 7) / 8, 256, 0, s, am_d, am_t, active, A, B, acc, h);
 }
 
 cudaError_t launch_erase_weights(const float* logp_x, const int32_t* corpus_tok,
                                  const int32_t* argmax_t, const float* row_mask, int A, int B,
                                  float gamma, int hard, float* weight, cudaStream_t s) {
-  erase_weights_kernel<<<(A + 7) / 8, 256, 0, s>>>(logp_x, corpus_tok, argmax_t, row_mask, A, B,
+  return launch_pdl(erase_weights_kernel, (A + 7) / 8, 256, 0, s, logp_x, corpus_tok, argmax_t, row_mask, A, B,
                                                    gamma, hard, weight);
-  return cudaGetLastError();
 }
 
 }  // namespace alr

@@ -88,6 +88,14 @@ ALR_DEV float max3(float a, float b, float c) {
   return r;
 }
 
+// Programmatic dependent launch (launch.h): every thread calls this before its first global
+// access.  Kernels read what an earlier one wrote through plain pointers: a load that the compiler
+// may take for invariant (const __restrict__) is not ordered by the wait's memory clobber.
+ALR_DEV void pdl_wait_and_release() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier ---
 ALR_DEV void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)

@@ -6,6 +6,7 @@
 // multicast reads of device memory never happen in a multi-rank process.
 #pragma once
 
+#include "launch.h"
 #include "tc_common.cuh"
 
 namespace alr {
@@ -118,8 +119,8 @@ ALR_DEV void mma_commit_pair(uint64_t* bar, uint16_t cta_mask) {
       : "memory");
 }
 
-// Host side: the launch configuration of a kernel on clusters of `ctas` CTAs along x (attr
-// must outlive the launch).
+// Host side: the launch configuration of a kernel on clusters of `ctas` CTAs along x (attr, two
+// entries, must outlive the launch).
 inline cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, unsigned ctas, unsigned grid,
                                          unsigned threads, size_t smem, cudaStream_t s) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -131,8 +132,9 @@ inline cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, unsigned cta
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cfg;
 }
 

@@ -25,7 +25,7 @@ cudaError_t launch_cluster(const CUtensorMap& a0, const CUtensorMap& a1, const C
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   int known = max_clusters[dev].load(std::memory_order_relaxed);
   if (known == 0) {
     cudaLaunchConfig_t q = cluster_config(attr, 2, 2, S::kThreads, S::kSmem, s);

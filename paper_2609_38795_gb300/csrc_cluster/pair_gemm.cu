@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish_pair();
   }
   tc_fence_before();
+  pdl_wait_and_release();
   __syncthreads();
   cluster_sync();   // both CTAs' barriers are initialised before any remote arrival
   tc_fence_after();
@@ -260,7 +261,7 @@ cudaError_t launch_t(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs&
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = cluster_config(attr, 2, unsigned(args.grid), kThreads, kSmemBytes, s);
   return cudaLaunchKernelEx(&cfg, kern, a, b, args);
 }
@@ -283,7 +284,7 @@ int alr_cluster_pair_gemm_max_pairs(void) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(kSmemBytes)) != cudaSuccess)
     return 0;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = cluster_config(attr, 2, 2, kThreads, kSmemBytes, nullptr);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) return 0;
