@@ -361,7 +361,9 @@ struct GemmChoice {
 //           512 x 4000: 23 -> 15 (5).  No gain past one tile per SM (1920 x 4096 x 151936: 1663
 //           against 1762).  Taken where it promises 10 %.
 constexpr double kPairFlops = 1.5e13;
-constexpr int64_t kPairMinBlocks = 32;   // below, the start of a pair's tile costs what it saves
+// Below, the start of a pair's tile costs what it saves (dW at d = 4096, V = 151936: K = 1024 1206
+// mcast, 1220 pair; 1920 1831 mcast, 1691 pair).
+constexpr int64_t kPairMinBlocks = 24;
 
 GemmChoice choose_gemm(int dtype, int M, int Nc, int K, int sms) {
   GemmChoice best{gemm_form(dtype), 1};
@@ -419,6 +421,12 @@ uint32_t gemm_b_rows(const GemmChoice& c) {
   }
 }
 
+// Up to this K the accumulating products are bound by the traffic of C, which the L2 prefetch helps
+// (dW at d = 4096, V = 151936: K = 128 1060 -> 968 us, 512 1091 -> 1079); beyond, it only competes
+// with the operands' loads (1024: 1206 -> 1226, 1920: 1691 -> 1780).  With a tile or two per CTA
+// there is nothing to run ahead of.
+constexpr int kPrefetchK = 512;
+
 alr::GemmArgs gemm_plan(int M, int Nc, int K, float* C, int64_t ldc, int sms) {
   alr::GemmArgs g{};
   g.M = M;
@@ -430,6 +438,7 @@ alr::GemmArgs gemm_plan(int M, int Nc, int K, float* C, int64_t ldc, int sms) {
   g.n_nb = (Nc + 255) / 256;
   g.group_m = g.n_mb < 16 ? g.n_mb : 16;
   g.n_tiles = g.n_mb * g.n_nb;
+  g.prefetch_c = K <= kPrefetchK && g.n_tiles >= 2 * sms ? 1 : 0;
   g.grid = sms < g.n_tiles ? sms : g.n_tiles;
   return g;
 }
@@ -446,6 +455,7 @@ alr::GemmArgs pair_gemm_plan(int M, int Nc, int K, float* C, int64_t ldc, int pa
   g.n_nb = (Nc + 255) / 256;
   g.group_m = g.n_mb < 8 ? g.n_mb : 8;
   g.n_tiles = g.n_mb * g.n_nb;
+  g.prefetch_c = K <= kPrefetchK && g.n_tiles >= 2 * pairs ? 1 : 0;
   g.grid = 2 * (pairs < g.n_tiles ? pairs : g.n_tiles);
   return g;
 }

@@ -125,6 +125,7 @@ struct GemmArgs {
   int group_m;      // m-blocks per raster group
   int n_tiles;
   int grid;
+  int prefetch_c;   // accumulating form: bring the next tile's rows of C into L2 a tile ahead
   int split;        // CTAs that share one tile's K blocks (split form; 0 or 1: not split)
   int* status;
   int withhold_first_stage;   // test hook: the producer never fills its first stage

@@ -257,7 +257,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_addr = tmem_base + (uint32_t(q * 32) << 16);
     int abuf = 0;
     uint32_t aphase = 0;
+    auto prefetch_c = [&](int t) {
+      if (!kAcc || kSplit || !args.prefetch_c || t >= args.n_tiles) return;
+      int mb, nb;
+      decode_tile(args, t, mb, nb);
+      if (kMc) mb = kMc * mb + rank;
+      prefetch_row(args, mb * kBM + q * 32, nb * kBN, kBN, lane);
+    };
+    prefetch_c(t0);
     for (int t = t0; t < args.n_tiles; t += t_step) {
+      prefetch_c(t + t_step);
       int mb, nb;
       decode_tile(args, t, mb, nb);
       if (kMc) mb = kMc * mb + rank;
@@ -279,13 +288,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       if constexpr (kSplit) {
         // every product of the tile is complete, so the stages hold nothing any more
 #pragma unroll 1
-        for (int c = 0; c < kBN / kEpiBlock; ++c) {
-          if (m0 >= args.M || n0 + c * kEpiBlock >= args.Nc) break;
+        for (int c = 0; c < kBN / kSplitBlock; ++c) {
+          if (m0 >= args.M || n0 + c * kSplitBlock >= args.Nc) break;
           uint32_t r[32];
-          tmem_ld32(lane_addr + c * kEpiBlock, r);
+          tmem_ld32(lane_addr + c * kSplitBlock, r);
           tmem_ld_wait();
           reg_fence(r);
-          put_row(r, smem + (q * (kBN / kEpiBlock) + c) * kEpiStageBytes, lane);
+          put_row(r, smem + (q * (kBN / kSplitBlock) + c) * kSplitBlockBytes, lane);
         }
         break;   // the cluster's only tile
       } else {
@@ -309,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster_sync();   // every CTA's partial sums are in its shared memory
     int mb, nb;
     decode_tile(args, t0, mb, nb);
-    reduce_split<kAcc, kBM / kEpiBlock, kBN / kEpiBlock>(args, mb * kBM, nb * kBN, smem, rank,
+    reduce_split<kAcc, kBM / kSplitBlock, kBN / kSplitBlock>(args, mb * kBM, nb * kBN, smem, rank,
                                                          int(cluster_nctarank()), warp,
                                                          kThreads / 32, lane);
     __syncwarp();

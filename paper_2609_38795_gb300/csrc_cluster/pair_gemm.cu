@@ -39,13 +39,12 @@ constexpr int kKE = 64;                     // K elements per stage
 constexpr int kMmaK = 16;                   // K per MMA
 constexpr int kChunkMN = 64;                // MN elements per 128-byte chunk
 constexpr uint32_t kChunkBytes = kKE * 128;
-// Slack after the last stage: an operand tile read past its own extent still lands in this
-// CTA's allocation.
-constexpr int kGuardBytes = 16 * 1024;
 constexpr int kCtrlBytes = 256;
-constexpr int kEpiBytes = kEpiWarps * kEpiStageBytes;   // the epilogue warps' staging
-constexpr size_t kSmemBytes =
-    1024 + size_t(kStages) * kStageBytes + kGuardBytes + kEpiBytes + kCtrlBytes;
+// The epilogue warps' staging, after the last stage: an operand tile read past its own extent
+// (at most 16 KB) still lands in this CTA's allocation.
+constexpr int kEpiBytes = kEpiWarps * kEpiStageBytes;
+static_assert(kEpiBytes >= 16 * 1024, "slack after the last stage");
+constexpr size_t kSmemBytes = 1024 + size_t(kStages) * kStageBytes + kEpiBytes + kCtrlBytes;
 static_assert((2 * kStages + 2 * 2 + 1) * 8 + 16 <= kCtrlBytes, "control block");
 
 ALR_DEV void decode_tile(const GemmArgs& a, int t, int& mb, int& nb) {
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      const __grid_constant__ CUtensorMap tm_b, const GemmArgs args) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_1024(smem_raw);
-  uint8_t* epi_stage = smem + kStages * kStageBytes + kGuardBytes;
+  uint8_t* epi_stage = smem + kStages * kStageBytes;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(epi_stage + kEpiBytes);
   uint64_t* empty_bar = full_bar + kStages;
   uint64_t* tfull_bar = empty_bar + kStages;
@@ -216,7 +215,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tempty_cl1 = cluster_smem_addr(&tempty_bar[1], 0);
     int abuf = 0;
     uint32_t aphase = 0;
+    auto prefetch_c = [&](int t) {
+      if (!kAcc || !args.prefetch_c || t >= args.n_tiles) return;
+      int mb, nb;
+      decode_tile(args, t, mb, nb);
+      prefetch_row(args, mb * 2 * kRows + int(rank) * kRows + q * 32, nb * kCols, kCols, lane);
+    };
+    prefetch_c(pair);
     for (int t = pair; t < args.n_tiles; t += n_pairs) {
+      prefetch_c(t + n_pairs);
       int mb, nb;
       decode_tile(args, t, mb, nb);
       const int m0 = mb * 2 * kRows + int(rank) * kRows + q * 32, n0 = nb * kCols;
