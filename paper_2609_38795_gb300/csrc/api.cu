@@ -166,11 +166,6 @@ int check_kept(const alr_params* p, const void* Z, const void* ref, const char* 
   return ALR_OK;
 }
 
-// Vocabulary tile width of the fused loss kernels (columns of z_d and of z_t per tile).
-#ifndef ALR_LOSS_BN
-#define ALR_LOSS_BN 256
-#endif
-
 // The fused loss kernels run on single CTAs unless the environment variable ALR_LOSS_FORM is
 // "mcast" (bf16 inputs): clusters of two CTAs sharing every head tile by TMA multicast, from
 // libalr_cluster.so, which only a single-process run loads (alr::cluster_forms() is nullptr in
@@ -179,9 +174,29 @@ int check_kept(const alr_params* p, const void* Z, const void* ref, const char* 
 // lower in clock for ~1 % fewer L2 bytes per product: it is not faster, so it is not the
 // default.  Both forms give bit-identical results.
 bool loss_multicast(const alr_params* p) {
-  if (p->dtype != ALR_BF16 || ALR_LOSS_BN != 256) return false;
+  if (p->dtype != ALR_BF16) return false;
   const char* v = getenv("ALR_LOSS_FORM");
   return v != nullptr && strcmp(v, "mcast") == 0 && alr::cluster_forms() != nullptr;
+}
+
+enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
+
+// Vocabulary columns per tile.  256-column products read each operand byte from shared memory for
+// twice the work, but their two accumulators fill tensor memory, so a tile's epilogue (6000 to
+// 10000 cycles) is not hidden; 128-column tiles are double-buffered, their products 25 % slower.
+// Narrow tiles pay in the forwards up to 10 K blocks (4096 x d x 32000, us, 256 -> 128 columns: d =
+// 256 forward 202 -> 183, keeping 246 -> 225, readout 199 -> 179; d = 512 261 -> 258, 309 -> 289,
+// 232 -> 210; d = 1000 410 -> 460), and everywhere when wide ones would not give each SM a tile
+// (192 x 320 x 1400: forward 18.4 -> 17.2, gradient 7.4 -> 5.6; d = 3072 42 -> 32 and 30 -> 21).
+// A loss form asked for by name runs on 256 columns, which the multicast form needs.
+constexpr int kNarrowBlocks = 10;
+
+int loss_tile_columns(const alr_params* p, int sms, bool bwd, int64_t n_rb) {
+  const char* v = getenv("ALR_LOSS_FORM");
+  if (v != nullptr && *v != '\0') return 256;
+  if (n_rb * ((p->V + 255) / 256) <= sms) return 128;
+  const int n_kb = (p->d + int(k_per_row(p->dtype)) - 1) / int(k_per_row(p->dtype));
+  return !bwd && n_kb <= kNarrowBlocks ? 128 : 256;
 }
 
 // Vocabulary splits of a forward over `rb` row blocks (row-block pairs in the two-row modes).
@@ -189,25 +204,30 @@ bool loss_multicast(const alr_params* p) {
 // with 19 splits throughout, 9 row blocks are 171 units on 152 CTAs, two rounds for the work of
 // one.  The split count is the one whose rounds times unit length (in vocabulary tiles, plus
 // the fixed cost of a unit) is smallest; `base` (one round over `group` row blocks, 19 splits
-// for 8) stays unless another promises 2 %.  More splits are more partial records: they take
-// at most kPartBytes beyond base's, so every problem the no-workspace forward took still fits.
+// for 8) stays unless another promises 2 %.  More splits are more partial records: they take at
+// most kPartBytes, or what 19 splits of 256-column tiles take, so every problem the no-workspace
+// forward took still fits.
 // Measured (us, 19 splits -> chosen): forward of 1152 x 1024 x 60000 358 -> 223, 2176 x 2048 x
 // 100000 1443 -> 1150, 8320 x 1024 x 32000 857 -> 760, 1920 x 4096 x 151936 2770 -> 2677; label
 // readout of 4096 x 2048 x 32000 533 -> 431.
 constexpr int64_t kPartBytes = 48ll << 20;
 constexpr int64_t kMaxRecordBytes = 4 * int64_t(sizeof(float)) * alr::kPFields;   // per row and split
 
-enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
-
-int forward_splits(const alr_params* p, int sms, int rb, int n_vt, int group, PlanKind kind) {
-  const int base = std::min(n_vt, std::max(1, sms / std::min(rb, group)));
-  const int64_t fit = p->dtype == ALR_BF16 ? kPartBytes / (p->N * kMaxRecordBytes) : 0;
-  const int most = int(std::min<int64_t>(n_vt, std::max<int64_t>(base, fit)));
+int forward_splits(const alr_params* p, int sms, int rb, int bn, int n_vt, int group,
+                   PlanKind kind) {
+  const int round = std::max(1, sms / std::min(rb, group));
+  // 19 splits of 256-column tiles, 15 fields: the records the no-workspace limit was set for
+  const int64_t wide = std::min((p->V + 255) / 256, round) * 4 * 15 * int64_t(sizeof(float));
+  const int64_t fit = std::max((wide * p->N - 2048) / (kMaxRecordBytes * p->N),
+                               p->dtype == ALR_BF16 ? kPartBytes / (kMaxRecordBytes * p->N) : 0);
+  const int most = int(std::min<int64_t>(n_vt, std::max<int64_t>(1, fit)));
+  const int base = std::min(most, round);
   // cycles of one tile: two 128 x 256 products over d (about 1090 per 64 of d) and an epilogue of
-  // about 7000; a unit adds its first loads and its record, about 2500, and in the readout the
+  // about 7000, or half of both, overlapped, the products 30 % slower; a unit adds its first loads and its record, about 2500, and in the readout the
   // filling of its top-8 lists, about 25000; a split adds its records' trip through memory (at
   // about 2800 bytes a cycle)
-  const double tile = 1090.0 * ((p->d + 63) / 64) * (p->dtype == ALR_BF16 ? 1 : 2) + 7000.0;
+  const double products = 1090.0 * ((p->d + 63) / 64) * (p->dtype == ALR_BF16 ? 1 : 2);
+  const double tile = bn == 256 ? products + 7000.0 : std::max(0.65 * products, 4500.0);
   const double per_unit = (kind == kPlanReadout ? 27500.0 : 2500.0) / tile;
   const double per_split = 2.0 * double(p->N) * kMaxRecordBytes / 2800.0 / tile;
   auto cost = [&](int vs) {
@@ -235,7 +255,6 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   P.d = p->d;
   P.V = p->V;
   P.B = p->B;
-  P.bn = ALR_LOSS_BN;
   P.mc = (!two_rows && loss_multicast(p)) ? 1 : 0;
   // row blocks; row-block pairs for the two-row modes and for the multicast form (which
   // places sms / 2 clusters).  Forward: the splits of forward_splits (the same for both
@@ -245,6 +264,7 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   const bool pairs = P.mc || two_rows;
   P.n_rb = pairs ? (rb + 1) / 2 : rb;
   const int group = pairs ? 4 : 8;
+  P.bn = loss_tile_columns(p, sms, bwd, P.n_rb);
   P.n_vt = (p->V + P.bn - 1) / P.bn;
   // two rounds per raster group: twice the row blocks share each W split, so W leaves DRAM
   // about half as often, with the same number of units per CTA (forward 49.8 against 50.0 ms at
@@ -254,14 +274,14 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   if (bwd) {
     P.n_vs = P.n_vt;  // one tile per unit
   } else {
-    P.n_vs = forward_splits(p, sms, two_rows ? P.n_rb : rb, P.n_vt, two_rows ? 4 : 8, kind);
+    P.n_vs = forward_splits(p, sms, two_rows ? P.n_rb : rb, P.bn, P.n_vt, two_rows ? 4 : 8, kind);
     // groups of equal size: 17 row blocks are 9 + 8, not 16 + 1 (in the backward's short units
     // the smaller groups only cost sharing: 2176 x 2048 x 100000 1071 -> 1105 us)
     const int n_groups = (P.n_rb + P.group_rows - 1) / P.group_rows;
     P.group_rows = (P.n_rb + n_groups - 1) / n_groups;
   }
   // partial records per row and split: one per epilogue column group
-  P.n_parts = P.n_vs * (P.bn / (two_rows ? 128 : 64));
+  P.n_parts = P.n_vs * (two_rows ? 2 : 4);
   P.n_units = P.n_rb * P.n_vs;
   P.grid = sms < P.n_units ? sms : P.n_units;
   return P;
@@ -504,13 +524,14 @@ int launch_gemm(const GemmChoice& c, int dt, bool a_mn, bool b_mn, bool acc, con
 
 // Tensor map of the head operand of the fused loss kernels: MN-major tiles straight from
 // W [d, V] for bf16; for fp32, W is first transposed into `wt` and read K-major.
-int head_map(CUtensorMap* m, const alr_params* p, const void* W, void* wt, cudaStream_t s) {
+int head_map(CUtensorMap* m, const alr_params* p, const void* W, void* wt, int bn,
+             cudaStream_t s) {
   const uint32_t kke = k_per_row(p->dtype);
   if (p->dtype == ALR_BF16) return make_map(m, W, ALR_BF16, p->V, p->d, uint64_t(p->V) * 2, kke, kke);
   cudaError_t e = alr::launch_transpose32(static_cast<const float*>(W), static_cast<float*>(wt),
                                           p->d, p->V, p->d, s);
   if (e != cudaSuccess) return cuda_fail(e, "head transpose launch");
-  return make_map(m, wt, ALR_F32, p->d, p->V, uint64_t(p->d) * 4, kke, ALR_LOSS_BN);
+  return make_map(m, wt, ALR_F32, p->d, p->V, uint64_t(p->d) * 4, kke, uint32_t(bn));
 }
 
 // The full-vocabulary forward; with Zd / Zt given, the fused kernel also writes both logit
@@ -548,10 +569,9 @@ int fwd_impl(const alr_params* p, const void* Hd, const void* Ht, const void* W,
   CUtensorMap m_hd, m_ht, m_w;
   if ((rc = make_map(&m_hd, Hd, dt, p->d, p->N, p->d * es, kke, 128)) != ALR_OK) return rc;
   if ((rc = make_map(&m_ht, Ht, dt, p->d, p->N, p->d * es, kke, 128)) != ALR_OK) return rc;
-  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, s)) != ALR_OK) return rc;
-
   alr::LossArgs args{};
   args.plan = loss_plan(p, info.sms, false);
+  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, args.plan.bn, s)) != ALR_OK) return rc;
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
   args.ticket = reinterpret_cast<unsigned*>(ws + lay.ticket_off);
   args.corpus_tok = p->mode != ALR_MODE_ALR ? corpus_tok : nullptr;
@@ -739,13 +759,14 @@ int logit_grad_impl(const alr_params* p, const void* Hd, const void* Ht, const v
   if ((rc = make_map(&m_hd, Hd, dt, p->d, p->N, p->d * es, kke, 128)) != ALR_OK) return rc;
   m_ht = m_hd;
   if (!topk && (rc = make_map(&m_ht, Ht, dt, p->d, p->N, p->d * es, kke, 128)) != ALR_OK) return rc;
-  if ((rc = head_map(&m_w, p, W, wt, s)) != ALR_OK) return rc;
+  const alr::LossPlan plan = loss_plan(p, info.sms, true, topk ? kPlanTopk : kPlanFwd);
+  if ((rc = head_map(&m_w, p, W, wt, plan.bn, s)) != ALR_OK) return rc;
   m_gs = m_w;
   if (dt == ALR_BF16 &&
       (rc = make_map(&m_gs, G, dt, p->V, p->N, p->V * es, 16, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) != ALR_OK)
     return rc;
   alr::LossArgs args{};
-  args.plan = loss_plan(p, info.sms, true, topk ? kPlanTopk : kPlanFwd);
+  args.plan = plan;
   args.G = G;
   args.lse_d = lse_d;
   args.lse_t = lse_t;
@@ -967,9 +988,9 @@ int alr_label_readout(const alr_params* p, const void* Ht, const void* W,
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CUtensorMap m_h, m_w;
   if ((rc = make_map(&m_h, Ht, dt, p->d, p->N, p->d * es, k_per_row(dt), 128)) != ALR_OK) return rc;
-  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, s)) != ALR_OK) return rc;
   alr::LossArgs args{};
   args.plan = loss_plan(p, info.sms, false, kPlanReadout);
+  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, args.plan.bn, s)) != ALR_OK) return rc;
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
   args.corpus_tok = corpus_tok;
   args.status = alr::device_status_ptr();
@@ -1018,9 +1039,9 @@ int topk_fwd_impl(const alr_params* p, const void* Hd, const void* W, const int3
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CUtensorMap m_h, m_w;
   if ((rc = make_map(&m_h, Hd, dt, p->d, p->N, p->d * es, k_per_row(dt), 128)) != ALR_OK) return rc;
-  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, s)) != ALR_OK) return rc;
   alr::LossArgs args{};
   args.plan = loss_plan(p, info.sms, false, kPlanTopk);
+  if ((rc = head_map(&m_w, p, W, ws + lay.wt_off, args.plan.bn, s)) != ALR_OK) return rc;
   args.part = reinterpret_cast<float*>(ws + lay.part_off);
   args.ticket = reinterpret_cast<unsigned*>(ws + lay.ticket_off);
   args.top_idx = top_idx;

@@ -18,7 +18,7 @@ struct LossPlan {
   int n_rb;        // ceil(N / 128)
   int n_vt;        // ceil(V / bn)
   int n_vs;        // vocabulary splits
-  int n_parts;     // partial records per row: n_vs * (bn / 64), one per split and 64-column group
+  int n_parts;     // partial records per row: one per split and column group (4, or 2 in two-row modes)
   int group_rows;  // row blocks per group
   int n_units;     // n_rb * n_vs
   int grid;        // persistent CTAs

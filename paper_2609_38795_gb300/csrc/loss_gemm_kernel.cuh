@@ -51,7 +51,6 @@ namespace {
 constexpr int kBM = 128;                 // rows per tile = TMEM lanes
 constexpr int kEpiWarp0 = 2;
 constexpr int kEpiBarrier = 1;           // named barrier of the epilogue warps (0 is __syncthreads)
-constexpr int kColsPerWarp = 64;
 constexpr int kSub = 16;                 // columns per TMEM load / processing step
 constexpr int kATileBytes = kBM * 128;   // a 128-row operand over 128 bytes of K
 constexpr int kCtrlBytes = 256;
@@ -89,9 +88,9 @@ struct Shape {
   static constexpr int kStageBytes = kATiles * kATileBytes + kBTileBytes;
   static constexpr int kAccCols = kATiles * kBN;       // first tile's columns, then the second's
   static constexpr int kAccBufs = 512 / kAccCols;
-  static constexpr int kWarpCols = kTwoRows ? 2 * kColsPerWarp : kColsPerWarp;
-  static constexpr int kColGroups = kBN / kWarpCols;   // partial records per row and split
-  static constexpr int kEpiWarps = 4 * (kBN / kColsPerWarp);
+  static constexpr int kEpiWarps = 16;                 // four per lane quarter
+  static constexpr int kColGroups = kTwoRows ? 2 : 4;  // partial records per row and split
+  static constexpr int kWarpCols = kBN / kColGroups;
   static constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
   static constexpr int kStaging = kStaged ? kEpiWarps * 2 * kGStageBytes : 0;
   static constexpr int kFit = (kSmemBudget - 1024 - kCtrlBytes - kStaging) / kStageBytes;

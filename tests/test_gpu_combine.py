@@ -112,8 +112,8 @@ def test_forward_workspace_stays_within_the_fixed_scratch():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     limit = 64 << 20
     up = lambda x: (x + 1023) // 1024 * 1024  # noqa: E731
-    for N in list(range(16, 4096, 112)) + list(range(4096, 16000, 592)):
-        for d, V in ((64, 1000), (1000, 60000), (4096, 151936)):
+    for N in list(range(16, 4096, 112)) + list(range(4096, 16000, 592)) + list(range(16000, 120000, 4112)):
+        for d, V in ((64, 200), (64, 1000), (256, 8000), (1000, 60000), (4096, 151936)):
             n_vt, rb = (V + 255) // 256, (N + 127) // 128
             vs = min(n_vt, max(1, sms // min(rb, 8)))
             start = up(15 * 4 * vs * 4 * N) + up(16 * (N // 16))
