@@ -140,14 +140,21 @@ ALR_DEV void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr));
 }
 
-// Maximum of 16 values: seven three-input maxima, depth 3 (max is exact, so any order gives
-// the same value).
-ALR_DEV float max16(const float (&z)[16]) {
-  const float a = max3(z[0], z[1], z[2]), b = max3(z[3], z[4], z[5]);
-  const float c = max3(z[6], z[7], z[8]), d = max3(z[9], z[10], z[11]);
-  const float e = max3(z[12], z[13], z[14]);
-  return max3(max3(a, b, c), max3(d, e, z[15]), -INFINITY);
+// Maximum of 16 values with the maxima of columns 3 k .. 3 k + 2 on the way to it: three-input
+// maxima (max is exact, so any order gives the same value).
+struct Max16 {
+  float g[5], m;
+};
+
+ALR_DEV Max16 max16_groups(const float (&z)[16]) {
+  Max16 r;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) r.g[k] = max3(z[3 * k], z[3 * k + 1], z[3 * k + 2]);
+  r.m = max3(max3(r.g[0], r.g[1], r.g[2]), max3(r.g[3], r.g[4], z[15]), -INFINITY);
+  return r;
 }
+
+ALR_DEV float max16(const float (&z)[16]) { return max16_groups(z).m; }
 
 // The sub-chunk's values, with columns at or past nv set to -inf.
 template <bool kFull>
@@ -198,9 +205,38 @@ ALR_DEV int first_at(const float (&z)[16], float cm) {
   return jj;
 }
 
-// top2_update for a sub-chunk whose new leader (cm > best) sits at column jj.
-ALR_DEV void top2_lead(float& best, float& sec, int& idx, const float (&z)[16], float cm, int jj,
-                       int v0) {
+// A new leader's column and the sub-chunk's second value, from the group maxima: the first group
+// that holds the maximum, then the column in it, about 50 instructions.
+ALR_DEV void top2_lead_groups(float& best, float& sec, int& idx, const float (&z)[16],
+                              const Max16& mx, int v0) {
+  // the selected group (from the last, column 15 alone, down to the first that holds the
+  // maximum), and the maximum of the groups not selected
+  float x0 = z[15], x1 = -INFINITY, x2 = -INFINITY, gm = z[15], rest = -INFINITY;
+  int j = 15;
+#pragma unroll
+  for (int k = 4; k >= 0; --k) {
+    const bool here = mx.g[k] == mx.m;
+    rest = fmaxf(rest, here ? gm : mx.g[k]);
+    gm = here ? mx.g[k] : gm;
+    x0 = here ? z[3 * k] : x0;
+    x1 = here ? z[3 * k + 1] : x1;
+    x2 = here ? z[3 * k + 2] : x2;
+    j = here ? 3 * k : j;
+  }
+  const bool at0 = x0 == mx.m, at1 = !at0 && x1 == mx.m;
+  // the two other columns of the group: (1, 2), (0, 2) or (0, 1)
+  const float c2 = max3(rest, at0 ? x1 : x0, at0 || at1 ? x2 : x1);
+  sec = fmaxf(best, c2);
+  best = mx.m;
+  idx = v0 + j + (at0 ? 0 : at1 ? 1 : 2);
+}
+
+// The same by comparing and masking all 16 columns, about 80 instructions but no group maxima to
+// hold: in the forward keeping the logits those spill (4096 x 256 x 32000: 225 us, 255 with the
+// groups; the plain forward 183 us, 158 with them).
+ALR_DEV void top2_lead_columns(float& best, float& sec, int& idx, const float (&z)[16], float cm,
+                               int v0) {
+  const int jj = first_at(z, cm);
   float c2 = -INFINITY;
 #pragma unroll
   for (int j = 0; j < kSub; ++j) c2 = fmaxf(c2, j == jj ? -INFINITY : z[j]);
@@ -209,10 +245,15 @@ ALR_DEV void top2_lead(float& best, float& sec, int& idx, const float (&z)[16], 
   idx = v0 + jj;
 }
 
-ALR_DEV void top2_update(float& best, float& sec, int& idx, const float (&z)[16], float cm,
+// In seven of ten sub-chunks of a short unit some lane of a warp meets a new leader.
+template <bool kGroups>
+ALR_DEV void top2_update(float& best, float& sec, int& idx, const float (&z)[16], const Max16& mx,
                          int v0) {
-  sec = fmaxf(sec, fminf(cm, best));
-  if (cm > best) top2_lead(best, sec, idx, z, cm, first_at(z, cm), v0);  // a new leader
+  sec = fmaxf(sec, fminf(mx.m, best));
+  if (mx.m > best) {   // a new leader
+    if constexpr (kGroups) top2_lead_groups(best, sec, idx, z, mx, v0);
+    else top2_lead_columns(best, sec, idx, z, mx.m, v0);
+  }
 }
 
 // Insert (v, i) into a list sorted by value descending; an equal value stays below the
@@ -255,14 +296,15 @@ ALR_DEV void stats_init(RowStats& st) {
 
 // Fold one 16-column sub-chunk (nv valid columns) into the full-vocabulary statistics.
 // cd, ct: the sub-chunk's maxima of z_d and z_t (over its valid columns), returned.
-template <bool kFull>
+template <bool kFull, bool kGroups>
 ALR_DEV void stats_sub(RowStats& st, const uint32_t (&rd)[16], const uint32_t (&rt)[16], int v0,
                        int nv, int x, float& cd, float& ct) {
   float zd[16], zt[16];
   load_masked<kFull>(zd, rd, nv);
   load_masked<kFull>(zt, rt, nv);
-  cd = max16(zd);
-  ct = max16(zt);
+  const Max16 md = max16_groups(zd), mt = max16_groups(zt);
+  cd = md.m;
+  ct = mt.m;
   const float nbt = fmaxf(st.best_t, ct), nbd = fmaxf(st.best_d, cd);
   const float bt = -nbt * kLog2e, bd = -nbd * kLog2e;
   // per column: T = (z_t - nbt) log2 e, D = (z_d - nbd) log2 e, E = 2^T; sums of E, 2^D,
@@ -311,8 +353,8 @@ ALR_DEV void stats_sub(RowStats& st, const uint32_t (&rd)[16], const uint32_t (&
   sum2_scaled(st.s_t, st.c_t, sct, s0 + s1);
   sum2_scaled(st.s_d, st.c_d, scd, d0 + d1);
   // greedy top-2 of both sides (moves best_d / best_t to the new maxima nbd / nbt)
-  top2_update(st.best_d, st.sec_d, st.i_d, zd, cd, v0);
-  top2_update(st.best_t, st.sec_t, st.i_t, zt, ct, v0);
+  top2_update<kGroups>(st.best_d, st.sec_d, st.i_d, zd, md, v0);
+  top2_update<kGroups>(st.best_t, st.sec_t, st.i_t, zt, mt, v0);
   const int xr = x - v0;
   if (xr >= 0 && xr < (kFull ? kSub : nv)) {
 #pragma unroll
@@ -756,8 +798,9 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
 
           if constexpr (is_fwd(kMode)) {
             float cd, ct;   // the sub-chunk's maxima, which also give the kept references
-            if (nv == kSub) stats_sub<true>(st, r0, r1, v0, kSub, x, cd, ct);
-            else stats_sub<false>(st, r0, r1, v0, nv, x, cd, ct);
+            constexpr bool kGroups = kMode == kModeFwd;
+            if (nv == kSub) stats_sub<true, kGroups>(st, r0, r1, v0, kSub, x, cd, ct);
+            else stats_sub<false, kGroups>(st, r0, r1, v0, nv, x, cd, ct);
             if constexpr (kMode == kModeFwdKeep) {
               if constexpr (kStaged) {
                 const __half hd = group_ref(cd), ht = group_ref(ct);
@@ -777,7 +820,8 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
             float z[16];
             if (nv == kSub) load_masked<true>(z, r0, nv);
             else load_masked<false>(z, r0, nv);
-            const float cm = max16(z);
+            const Max16 mx = max16_groups(z);
+            const float cm = mx.m;
             if constexpr (kMode == kModeTopkFwdKeep) {
               if constexpr (kStaged) {
                 const __half h = group_ref(cm);
@@ -811,7 +855,7 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
                 c = max16(z);
               }
             } else {
-              top2_update(best, sec, bidx, z, cm, v0);
+              top2_update<true>(best, sec, bidx, z, mx, v0);
               // the label tokens' exponentials, the very terms lse_update added to s, so that
               // s - s_in is the drafter's mass outside the label (the tail bin's q) without a
               // cancellation between separately rounded sums
