@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(32 * kWarps)
 // anchor, with 16 warps over the records (32 warps leave a thread 64 registers
 // and spill).
 constexpr int kManyBlocks = 304;
+constexpr int kReadoutFewRows = 1024;
 
 struct MergeShape {
   int rows, warps, rows_per_block, blocks;
@@ -602,10 +603,18 @@ cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool
                                    int32_t* top_idx, float* top_prob, float* tail, float* lse_t,
                                    int32_t* argmax_t, float* gap_t, float* logp_x,
                                    cudaStream_t s) {
-  const MergeShape m = merge_shape(plan.N, 1);
-  auto kern = m.warps == 8 ? readout_combine_kernel<32, 8> : readout_combine_kernel<8, 16>;
-  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, has_corpus ? 1 : 0, top_idx, top_prob, tail,
-                                         lse_t, argmax_t, gap_t, logp_x);
+  // a merge of two top-8 lists costs several times a plain record's, so with more rows fewer lanes
+  // share one: 64, 16 from 1024 rows, 8 (readout with 16 instead of 64: 1920 x 64 x 151936 243 ->
+  // 229 us, 9000 x 64 x 20000 231 -> 191; 768 x 64 x 151936 130 -> 131)
+  MergeShape m = merge_shape(plan.N, 1);
+  auto kern = readout_combine_kernel<32, 8>;
+  if (m.rows < 32) {
+    const bool few = plan.N < kReadoutFewRows;
+    kern = few ? readout_combine_kernel<8, 16> : readout_combine_kernel<16, 8>;
+    m = few ? MergeShape{8, 16, 8, (plan.N + 7) / 8} : MergeShape{16, 8, 16, (plan.N + 15) / 16};
+  }
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, has_corpus ? 1 : 0, top_idx,
+                    top_prob, tail, lse_t, argmax_t, gap_t, logp_x);
 }
 
 cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const float* top_prob,

@@ -25,9 +25,10 @@ def _lib():
 
 
 # (A, B): one row; a partial 8-row block; anchors of 3 and 8 in 8 rows; 9 and 16 in 16; 17 and
-# 32 in 32; the last shape of the small form (303 blocks of 30 rows) and the first of the large
+# 32 in 32; the last shape of the small form (303 blocks of 30 rows) and the first of the large;
+# the two sides of the readout's choice of lanes per row
 SHAPES = [(1, 1), (13, 1), (5, 3), (3, 8), (3, 9), (7, 16), (4, 17), (3, 32), (606, 15),
-          (607, 15), (9729, 1)]
+          (607, 15), (9729, 1), (1023, 1), (1024, 1)]
 
 
 @pytest.mark.parametrize("mode", [alr.ALR_MODE_ERASE_SOFT, alr.ALR_MODE_ERASE_HARD])
