@@ -442,8 +442,8 @@ uint32_t gemm_b_rows(const GemmChoice& c) {
 }
 
 // Up to this K the accumulating products are bound by the traffic of C, which the L2 prefetch helps
-// (dW at d = 4096, V = 151936: K = 128 1060 -> 968 us, 512 1091 -> 1079); beyond, it only competes
-// with the operands' loads (1024: 1206 -> 1226, 1920: 1691 -> 1780).  With a tile or two per CTA
+// (dW at d = 4096, V = 151936, with two pieces ahead: K = 128 1060 -> 968 us, 512 1091 -> 1079);
+// beyond, it only competes with the operands' loads (1024: 1206 -> 1226, 1920: 1691 -> 1780).  With a tile or two per CTA
 // there is nothing to run ahead of.
 constexpr int kPrefetchK = 512;
 

@@ -5,14 +5,16 @@
 // form waits for every one of its reads.  Each warp therefore turns 32 x 64 blocks around in its
 // own 8 KB of shared memory (16-byte columns XOR-swizzled by the row, conflict-free both ways)
 // and touches global memory in 256-byte row pieces, two rows per instruction.  The accumulating
-// form has the old values of the next two 16-row halves in flight while it adds one, and where K
-// is so small that C's traffic sets the time it asks for the next tile's rows, 1 KB each, to be
-// brought into L2 a tile ahead (prefetch_row).
+// form has the old values of the next 16-row half in flight while it adds one, and where K is so
+// small that C's traffic sets the time it asks for the next tile's rows, 1 KB each, to be brought
+// into L2 a tile ahead (prefetch_row).
 // Bound by the 8 bytes per element of C when K is small: dW += H_d^T G at d = 4096, V = 151936 (5
-// GB of C) takes 968 us with 128 rows, against 2968 us written straight from the lanes, 1197 in
+// GB of C) takes 922 us with 128 rows, against 2968 us written straight from the lanes, 1197 in
 // 128-byte pieces without the L2 prefetch and 1002 with it, 1060 in 256-byte pieces without it.
 // DRAM serves short pieces of scattered rows badly: the same traffic alone, without products,
 // takes 1286, 980 and, in 256-byte pieces with the prefetch, 803 us; one stream over C takes 701.
+// More reads in flight only queue up: 968 us with two halves ahead, 1044 with none, 1105 with
+// eight epilogue warps.
 #pragma once
 
 #include "kernels.h"
@@ -87,22 +89,19 @@ ALR_DEV void store_piece(const CPiece& old, const GemmArgs& a, int m0, int n0, i
   }
 }
 
-// A warp's 32 x kCols strip of C, with its old values two pieces ahead of their use.
+// A warp's 32 x kCols strip of C, with its old values one piece ahead of their use.
 template <bool kAcc, int kCols>
 struct CStrip {
   static constexpr int kPieces = 2 * kCols / kEpiWide;
-  CPiece old[3];
+  CPiece old[2];
 
   ALR_DEV void load(int s, const GemmArgs& a, int m0, int n0, int lane) {
-    old[s % 3].load(a, m0 + 16 * (s & 1), n0 + (s >> 1) * kEpiWide, lane);
+    old[s & 1].load(a, m0 + 16 * (s & 1), n0 + (s >> 1) * kEpiWide, lane);
   }
 
   // Before the tile's accumulator is ready.
   ALR_DEV void begin(const GemmArgs& a, int m0, int n0, int lane) {
-    if (kAcc) {
-      load(0, a, m0, n0, lane);
-      load(1, a, m0, n0, lane);
-    }
+    if (kAcc) load(0, a, m0, n0, lane);
   }
 
   // The accumulator (tensor-memory address `taddr`, this warp's lanes) is ready; `release` is
@@ -112,7 +111,7 @@ struct CStrip {
                       Release release) {
 #pragma unroll
     for (int s = 0; s < kPieces; ++s) {
-      if (kAcc && s + 2 < kPieces) load(s + 2, a, m0, n0, lane);
+      if (kAcc && s + 1 < kPieces) load(s + 1, a, m0, n0, lane);
       if ((s & 1) == 0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -125,7 +124,7 @@ struct CStrip {
         }
         __syncwarp();
       }
-      store_piece<kAcc>(old[s % 3], a, m0 + 16 * (s & 1), n0 + (s >> 1) * kEpiWide, s & 1, stage,
+      store_piece<kAcc>(old[s & 1], a, m0 + 16 * (s & 1), n0 + (s >> 1) * kEpiWide, s & 1, stage,
                         lane);
       if ((s & 1) == 1) __syncwarp();   // the staging is read before the next block goes in
     }
