@@ -252,12 +252,15 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
                                     const float* weight, const float* weight_sum, float lam, int N,
                                     int V, void* G, cudaStream_t s) {
   const int rows = grad_rows(N, V);
+  const double size = 2000.0 * N * V;   // as long as this many flop of a product
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
-    return launch_pdl(topk_logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
+    return launch_pdl_sized(
+        size, topk_logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
         static_cast<const __half*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
         weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
-  return launch_pdl(topk_logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+  return launch_pdl_sized(
+        size, topk_logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
         static_cast<const float*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
         weight_sum, lam, N, V, rows, static_cast<float*>(G));
 }
@@ -267,12 +270,15 @@ cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const 
                                const float* weight, const float* weight_sum, float lam, int N,
                                int V, void* G, cudaStream_t s) {
   const int rows = grad_rows(N, V);
+  const double size = 2000.0 * N * V;   // as long as this many flop of a product
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
-    return launch_pdl(logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
+    return launch_pdl_sized(
+        size, logits_grad_kernel<__half, __nv_bfloat16>, grid, kGradThreads, 0, s,
         static_cast<const __half*>(zd), static_cast<const __half*>(zt), zd_ref, zt_ref, lse_d,
         lse_t, weight, weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
-  return launch_pdl(logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+  return launch_pdl_sized(
+        size, logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
         static_cast<const float*>(zd), static_cast<const float*>(zt), zd_ref, zt_ref, lse_d,
         lse_t, weight, weight_sum, lam, N, V, rows, static_cast<float*>(G));
 }

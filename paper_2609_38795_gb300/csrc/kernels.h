@@ -22,6 +22,7 @@ struct LossPlan {
   int group_rows;  // row blocks per group
   int n_units;     // n_rb * n_vs
   int grid;        // persistent CTAs
+  double flops() const { return 4.0 * N * d * V; }   // two products of a tile
   int mc;          // 1: clusters of two CTAs share each head tile by TMA multicast (bf16,
                    // 256-column tiles); n_rb and group_rows then count row-block pairs and
                    // the grid is sized from the clusters that fit
@@ -118,6 +119,7 @@ cudaError_t launch_loss_kernel(int mode, int dtype, const CUtensorMap& a0, const
 // Plain GEMM C[M, Nc] (+)= A[M, K] B[K, Nc] with fp32 output (plain_gemm_kernel.cuh, single-CTA
 // form launched from plain_gemm.cu).
 struct GemmArgs {
+  double flops() const { return 2.0 * M * Nc * K; }
   int M, Nc, K;
   float* C;
   int64_t ldc;

@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
     tmem_relinquish();
   }
   tc_fence_before();
-  pdl_wait_and_release();
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0 && args.ticket != nullptr) *args.ticket = 0u;
   __syncthreads();
   if constexpr (kMc) cluster_sync();   // the peer's copies and commits find initialised barriers
@@ -970,6 +970,7 @@ __global__ void __launch_bounds__(Shape<kMode, kBN, is_staged(kMode, sizeof(Elem
 
   tc_fence_before();
   __syncthreads();
+  pdl_release();   // past the barrier: idle lanes and warps are here early
   if constexpr (kMc) cluster_sync();   // no CTA leaves while its peer may still write into it
   if (warp == 1) {
     tc_fence_after();

@@ -54,7 +54,7 @@ cudaError_t launch_t(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs&
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, args.grid, kThreads, kSmemBytes, s, a, b, args);
+  return launch_pdl_sized(args.flops(), kern, args.grid, kThreads, kSmemBytes, s, a, b, args);
 }
 
 template <typename Elem>

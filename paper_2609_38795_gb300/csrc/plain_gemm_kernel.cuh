@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
   }
   tc_fence_before();
-  pdl_wait_and_release();
+  pdl_wait();
   __syncthreads();
   if constexpr (kMc) cluster_sync();   // the peer's copies and commits find initialised barriers
   tc_fence_after();
@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   tc_fence_before();
   __syncthreads();
+  pdl_release();   // past the barrier: idle lanes and warps are here early
   if constexpr (kSplit) {
     cluster_sync();   // every CTA's partial sums are in its shared memory
     int mb, nb;

@@ -122,7 +122,8 @@ ALR_DEV void mma_commit_pair(uint64_t* bar, uint16_t cta_mask) {
 // Host side: the launch configuration of a kernel on clusters of `ctas` CTAs along x (attr, two
 // entries, must outlive the launch).
 inline cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, unsigned ctas, unsigned grid,
-                                         unsigned threads, size_t smem, cudaStream_t s) {
+                                         unsigned threads, size_t smem, cudaStream_t s,
+                                         double flops = 0.0) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = ctas;
   attr[0].val.clusterDim.y = 1;
@@ -132,7 +133,7 @@ inline cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, unsigned cta
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  attr[1] = pdl_attribute();
+  attr[1] = pdl_attribute(flops);
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cfg;

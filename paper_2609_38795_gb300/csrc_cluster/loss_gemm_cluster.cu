@@ -36,7 +36,8 @@ cudaError_t launch_cluster(const CUtensorMap& a0, const CUtensorMap& a1, const C
     known = n;
   }
   const int clusters = known < args.plan.n_units ? known : args.plan.n_units;
-  cudaLaunchConfig_t cfg = cluster_config(attr, 2, unsigned(2 * clusters), S::kThreads, S::kSmem, s);
+  cudaLaunchConfig_t cfg = cluster_config(attr, 2, unsigned(2 * clusters), S::kThreads, S::kSmem, s,
+                                          args.plan.flops());
   return cudaLaunchKernelEx(&cfg, kern, a0, a1, w, g, g2, args);
 }
 

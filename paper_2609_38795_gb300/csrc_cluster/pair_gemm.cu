@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish_pair();
   }
   tc_fence_before();
-  pdl_wait_and_release();
+  pdl_wait();
   __syncthreads();
   cluster_sync();   // both CTAs' barriers are initialised before any remote arrival
   tc_fence_after();
@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   tc_fence_before();
   __syncthreads();
+  pdl_release();   // past the barrier: idle lanes and warps are here early
   cluster_sync();   // the even CTA's products into both tensor memories are complete
   if (warp == 1) {
     tc_fence_after();
@@ -269,7 +270,8 @@ cudaError_t launch_t(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = cluster_config(attr, 2, unsigned(args.grid), kThreads, kSmemBytes, s);
+  cudaLaunchConfig_t cfg = cluster_config(attr, 2, unsigned(args.grid), kThreads, kSmemBytes, s,
+                                          args.flops());
   return cudaLaunchKernelEx(&cfg, kern, a, b, args);
 }
 

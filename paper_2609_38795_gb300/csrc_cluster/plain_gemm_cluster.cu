@@ -17,7 +17,8 @@ cudaError_t launch_t(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = cluster_config(attr, kMc, unsigned(args.grid), kThreads, kSmemBytes, s);
+  cudaLaunchConfig_t cfg = cluster_config(attr, kMc, unsigned(args.grid), kThreads, kSmemBytes, s,
+                                          args.flops());
   return cudaLaunchKernelEx(&cfg, kern, a, b, args);
 }
 
