@@ -464,7 +464,7 @@ class Step:
     in place of z_d; otherwise G is computed by recomputing both head products."""
     N_PHASES = 6
     PHASES = ["gather", "fwd", "accept_len", "logit_grad", "dH_gemm", "dW_gemm"]
-    KERNELS_PER_STEP = 8   # gather, fwd (loss, combine, finalize), accept, logit grad, dH, dW
+    KERNELS_PER_STEP = 7   # gather, fwd (loss, merge), accept, logit grad, dH, dW
 
     def __init__(self, wl, inputs, device, keep=True, mode=0, corpus_tok=None):
         import torch
@@ -510,7 +510,7 @@ class TopkStep:
     accepted length -> logit gradient from the kept z_d (in place) -> dH = G W^T ->
     dW += H_d^T G.  It reuses the full-vocabulary step's z_d buffer."""
     PHASES = ["readout", "fwd", "accept_len", "logit_grad", "dH_gemm", "dW_gemm"]
-    KERNELS_PER_STEP = 8   # readout (+ merge), fwd (+ merge, finalize), accept, grad, dH, dW
+    KERNELS_PER_STEP = 8   # readout (+ merge), fwd (+ merge), accept, grad, dH, dW
 
     def __init__(self, step):
         import torch
@@ -683,7 +683,7 @@ def time_other_workloads(device, K, warmup):
         "workload": f"small: d={wl.d} V={wl.V} B={wl.B} A={wl.A} rows={wl.N}",
         "ms": ms, "rows_per_s": wl.N / (ms / 1e3),
         "tflops_4NdV": 4 * wl.N * wl.d * wl.V / (ms / 1e3) / 1e12,
-        "l2": "flushed (256 MB write) before every repetition", "gpu_launches": 3 * K}
+        "l2": "flushed (256 MB write) before every repetition", "gpu_launches": 2 * K}
     del sl, bt, flush
     torch.cuda.empty_cache()
     return out

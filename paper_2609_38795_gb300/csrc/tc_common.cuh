@@ -92,9 +92,9 @@ ALR_DEV float max3(float a, float b, float c) {
 // access.  Kernels read what an earlier one wrote through plain pointers: a load that the compiler
 // may take for invariant (const __restrict__) is not ordered by the wait's memory clobber.
 // pdl_release lets the next kernel be scheduled once some thread of every block has called it (or
-// the block has ended).  The tensor-core kernels call it when their work is done: blocks of the next kernel that sit on the
-// SMs for the whole of a long kernel, waiting, cost power (the text8b step 106.4 -> 109.1 ms with
-// the call at their start).
+// the block has ended).  The tensor-core kernels call it when their work is done: blocks of the
+// next kernel that sit on the SMs for the whole of a long kernel, waiting, cost power (the text8b
+// step 106.4 -> 109.1 ms with the call at their start).
 ALR_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 ALR_DEV void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 ALR_DEV void pdl_wait_and_release() {
