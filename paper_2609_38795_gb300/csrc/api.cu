@@ -183,7 +183,7 @@ enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
 
 // Vocabulary columns per tile.  256-column products read each operand byte from shared memory for
 // twice the work, but their two accumulators fill tensor memory, so a tile's epilogue (6000 to
-// 10000 cycles) is not hidden; 128-column tiles are double-buffered, their products 25 % slower.
+// 10000 cycles) is not hidden; 128-column tiles are double-buffered, their products slower.
 // Narrow tiles pay in the forwards up to 10 K blocks (4096 x d x 32000, us, 256 -> 128 columns: d =
 // 256 forward 202 -> 183, keeping 246 -> 225, readout 199 -> 179; d = 512 261 -> 258, 309 -> 289,
 // 232 -> 210; d = 1000 410 -> 460), and everywhere when wide ones would not give each SM a tile
@@ -367,11 +367,11 @@ struct GemmChoice {
 // The form of a product when none is asked for by name: the cheapest by a cost in 0.01 us, from
 // the rounds a form needs over the SMs and a fixed time per K block (64 bf16) and per launch,
 // fitted to the measurements below (us, random operands, timed alone).
-//   pair    27 per K block: six 32 KB stages per CTA ride out the load latency that four 48 KB
-//           stages do not (500-520 against 600-690 cycles per K block, 512 being the tensor
-//           pipe's time), and B is read once per pair.  It draws more power per product, though: at
+//   pair    27 per K block: six 32 KB stages per CTA ride out more load latency than four 48 KB
+//           ones (which take 600-690 cycles per K block, 512 being the tensor pipe's time), and
+//           B is read once per pair.  It draws more power per product, though: at
 //           the text8b size (4.1e13 flop per product, the step at the power cap throughout) dH
-//           and dW gain 2.6 ms and the forward behind them loses 5, 102.5 -> 106.1 ms per step;
+//           and dW gain 1.5 ms and the forward behind them loses 5, 102.5 -> 106.1 ms per step;
 //           at 1.0e13 the step gains 1 %, at 2.4e12 4 %, at 5.4e11 5 %.  So: up to kPairFlops.
 //   mcast   35.5 per K block; single 42, but no cluster has to be placed and an odd row block
 //           leaves no CTA idle (128 x 32000 x 512: 9.4 against 15.4 us).

@@ -8,7 +8,7 @@
 namespace alr {
 
 // Row-block x vocabulary-split work plan of the fused loss kernels.
-//   A "unit" is one 128-row block times one contiguous range of 128-column vocabulary tiles.
+//   A "unit" is one 128-row block times one contiguous range of vocabulary tiles.
 //   Units are numbered group by group: a group holds `group_rows` consecutive row blocks,
 //   and inside a group the row block varies fastest, so the CTAs running at the same time
 //   share both their hidden-state tiles and their head tiles through L2.

@@ -6,8 +6,8 @@
 //   kModeFwd     z_d = H_d W and z_t = H_t W (both share every W stage): running per-row
 //                statistics (online max / sum-exp of both sides, the label-weighted sums behind
 //                the soft cross-entropy of Eq. 1, greedy top-2 with lowest-index ties, z_t at
-//                the corpus token), one partial record per row, vocabulary split and 64-column
-//                group;
+//                the corpus token), one partial record per row, vocabulary split and column
+//                group (below);
 //   kModeFwdKeep the same, and both logit tiles are also written to global memory (fp16
 //                relative to per-16-column-group references for bf16 inputs, fp32 for fp32
 //                inputs) so that the backward need not recompute them;
@@ -20,15 +20,16 @@
 //   kModeTopkBwd z_d only, recomputed: the gradient of that loss;
 //   kModeTopkFwdKeep  kModeTopkFwd that also writes z_d (as kModeFwdKeep).
 //
-// Accumulators: 2 x kBN TMEM columns per tile (single-buffered at kBN = 256).  The dual modes
+// Accumulators: 2 x kBN TMEM columns per tile (kBN = 256: all of tensor memory, one tile at a
+// time; kBN = 128: two tiles, the next one's products behind this one's epilogue).  The dual modes
 // hold z_d and z_t of one 128-row block; the single-operand modes (readout, top-k) hold one
 // logit tile of each of two row blocks (rows 256 i .. 256 i + 255), so that they too read every
 // head tile from shared memory once for two products.
 //
 // Warp roles: warp 0 issues TMA loads, warp 1 owns tensor memory and issues the MMAs from one
 // lane, warps 2.. run the epilogue: warp w reads TMEM lanes 32(w%4)..+31 (one row per thread)
-// in 16-column sub-chunks; in the dual modes it takes columns [64 g, 64 g + 64) of both tiles,
-// g = (w-2)/4; in the two-row modes columns [128 h, 128 h + 128) of row block b's tile,
+// in 16-column sub-chunks; in the dual modes it takes quarter g of both tiles' columns,
+// g = (w-2)/4; in the two-row modes half h of the columns of row block b's tile,
 // b = ((w-2)/4) % 2, h = (w-2)/8.
 // Every pipeline wait is bounded (tc_common.cuh).
 //
