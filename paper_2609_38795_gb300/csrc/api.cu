@@ -816,12 +816,10 @@ int head_grads_impl(const alr_params* p, const void* Hd, const void* W, const vo
     // K-major operands from transposed copies H_d^T [d, N'] and G^T [V, N'].
     float* hdt = reinterpret_cast<float*>(ws + lay.hdt_off);
     float* gt = reinterpret_cast<float*>(ws + lay.gt_off);
-    if ((e = alr::launch_transpose32(static_cast<const float*>(Hd), hdt, int(p->N), p->d,
-                                     int(lay.ld_n), s)) != cudaSuccess)
-      return cuda_fail(e, "H_d transpose launch");
-    if ((e = alr::launch_transpose32(static_cast<const float*>(G), gt, int(p->N), p->V,
-                                     int(lay.ld_n), s)) != cudaSuccess)
-      return cuda_fail(e, "G transpose launch");
+    if ((e = alr::launch_transpose32_pair(static_cast<const float*>(Hd), hdt, p->d,
+                                          static_cast<const float*>(G), gt, p->V, int(p->N),
+                                          int(lay.ld_n), s)) != cudaSuccess)
+      return cuda_fail(e, "H_d and G transpose launch");
     if ((rc = make_map(&m_ha, hdt, dt, p->N, p->d, lay.ld_n * 4, kke, 128)) != ALR_OK) return rc;
     if ((rc = make_map(&m_gb, gt, dt, p->N, p->V, lay.ld_n * 4, kke, gemm_b_rows(dw))) != ALR_OK)
       return rc;

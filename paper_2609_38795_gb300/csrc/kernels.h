@@ -216,6 +216,10 @@ cudaError_t launch_ira_context(const void* store, int C, int F, int elem_bytes, 
 cudaError_t launch_transpose32(const float* in, float* out, int R, int C, int ld_out,
                                cudaStream_t s);
 
+// The same for a [R, Ca] and b [R, Cb] in one launch (both outputs with ld_out).
+cudaError_t launch_transpose32_pair(const float* a, float* a_out, int Ca, const float* b, float* b_out,
+                                    int Cb, int R, int ld_out, cudaStream_t s);
+
 // Record `msg` as this host thread's alr_last_error() text and return `code` (api.cu).
 int set_last_error(int code, const char* msg);
 

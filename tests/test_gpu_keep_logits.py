@@ -181,3 +181,26 @@ def test_keep_logits_small_workload():
     assert P.max_norm_rel(P.np64(dH), G @ W64.T) <= P.GRAD_RTOL
     cols = np.arange(0, wl.V, 4)
     assert P.max_norm_rel(P.np64(dW)[:, cols], Hd64.T @ G[:, cols]) <= P.GRAD_RTOL
+
+
+@pytest.mark.parametrize("A,B,d,V", [(1, 1, 8, 8), (3, 11, 40, 1032), (2, 16, 32, 32),
+                                     (65, 1, 64, 4096), (1, 31, 256, 8)])
+def test_fp32_head_gradient_transposes(A, B, d, V):
+    """fp32 dW += H_d^T G reads both operands K-major, from copies transposed by one launch:
+    element by element against fp64 with the GPU's own G, at one row, one 32 x 32 tile exactly,
+    tails in every direction.  Each tf32 operand keeps 10 mantissa bits, so a product is within
+    2^-9 (1 + 2^-11) of itself; 2^-24 per fp32 addition on top of the rows' sum and of dW0."""
+    N = A * B
+    Hd, Ht, W = _inputs(d, V, A, B, 0.5, torch.float32, seed=d + V)
+    sl = alr.SlotLoss(N, d, V, B, dtype=torch.float32, keep_logits=True)
+    sl.forward(Hd, Ht, W)
+    dH = torch.empty(N, d, device="cuda")
+    dW0 = torch.randn(d, V, device="cuda") * 1e-3
+    dW = dW0.clone()
+    sl.backward(Hd, Ht, W, dH, dW)
+    torch.cuda.synchronize()
+    h, G = P.np64(Hd), P.np64(sl.G)
+    ref, mag = P.np64(dW0) + h.T @ G, np.abs(h).T @ np.abs(G)
+    bound = mag * (2.0 ** -9 * 1.01 + N * 2.0 ** -23) + (np.abs(ref) + np.abs(P.np64(dW0))) * 2.0 ** -23
+    assert np.all(np.abs(P.np64(dW) - ref) <= bound + 1e-36)
+    assert alr.alr_device_status() == alr.ALR_OK
