@@ -92,11 +92,11 @@ __device__ __forceinline__ void store1(float* p, float v) { *p = v; }
 // Reference of the group that holds vector i (8 columns; two vectors per 16-column group) of
 // row r, from the group-major array, scaled by log2 e: a warp's 32 vectors of one row read 16
 // groups, and the next rows of the block read the same sectors again (32 rows of a group are
-// 64 contiguous bytes), so the loads go through the read-only cache.  fp32 logits have none.
+// 64 contiguous bytes), from L1.  fp32 logits have none.
 template <typename Z>
 __device__ __forceinline__ float ref_l2e(const uint16_t* ref, int N, int g, int r) {
   if constexpr (sizeof(Z) == 2)
-    return __half2float(__ushort_as_half(__ldg(ref + size_t(g) * size_t(N) + r))) * kLog2e;
+    return __half2float(__ushort_as_half(ref[size_t(g) * size_t(N) + r])) * kLog2e;
   else
     return 0.f;
 }

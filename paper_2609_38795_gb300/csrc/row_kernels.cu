@@ -15,13 +15,10 @@ namespace {
 // the matching stores so that many requests are in flight per SM.
 constexpr int kGatherBatch = 16;
 
-__global__ void __launch_bounds__(256) gather_kernel(const uint4* __restrict__ feat, int S, int L,
-                                                     int vec_per_row,
-                                                     const int32_t* __restrict__ seq,
-                                                     const int32_t* __restrict__ pos,
-                                                     const int32_t* __restrict__ valid_len,
-                                                     int A, int B, uint4* __restrict__ out,
-                                                     float* __restrict__ row_valid) {
+__global__ void __launch_bounds__(256) gather_kernel(const uint4* feat, int S, int L,
+                                                     int vec_per_row, const int32_t* seq,
+                                                     const int32_t* pos, const int32_t* valid_len,
+                                                     int A, int B, uint4* out, float* row_valid) {
   pdl_wait_and_release();
   const long long r = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -44,7 +41,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const uint4* __restrict__ f
 #pragma unroll
     for (int j = 0; j < kGatherBatch; ++j) {
       const int i = base + j * 32 + lane;
-      if (i < vec_per_row) v[j] = __ldg(src + i);
+      if (i < vec_per_row) v[j] = src[i];
     }
 #pragma unroll
     for (int j = 0; j < kGatherBatch; ++j) {
@@ -339,10 +336,9 @@ __global__ void __launch_bounds__(kDrawThreads)
 // primary i's stored rollout features when secondary i of sample s exists and r < j - 1,
 // zero otherwise.  One warp per output row, 16-byte vectors in batches as in the gather.
 __global__ void __launch_bounds__(256) ira_context_kernel(
-    const uint4* __restrict__ store, int C, int vec_per_row, int S, int K, int max_blocks,
-    const int32_t* __restrict__ n_valid, const int32_t* __restrict__ rollout_len,
-    const int32_t* __restrict__ offsets, const int32_t* __restrict__ anchor_pos,
-    uint4* __restrict__ ctx, int32_t* __restrict__ ctx_len, int32_t* __restrict__ prefix_end) {
+    const uint4* store, int C, int vec_per_row, int S, int K, int max_blocks,
+    const int32_t* n_valid, const int32_t* rollout_len, const int32_t* offsets,
+    const int32_t* anchor_pos, uint4* ctx, int32_t* ctx_len, int32_t* prefix_end) {
   pdl_wait_and_release();
   const int H = max_blocks / 2, P = max_blocks - H;
   const long long t = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
@@ -372,7 +368,7 @@ __global__ void __launch_bounds__(256) ira_context_kernel(
 #pragma unroll
     for (int k = 0; k < kGatherBatch; ++k) {
       const int e = base + k * 32 + lane;
-      if (e < vec_per_row) v[k] = __ldg(src + e);
+      if (e < vec_per_row) v[k] = src[e];
     }
 #pragma unroll
     for (int k = 0; k < kGatherBatch; ++k) {

@@ -89,8 +89,9 @@ ALR_DEV float max3(float a, float b, float c) {
 }
 
 // Programmatic dependent launch (launch.h): every thread calls pdl_wait before its first global
-// access.  Kernels read what an earlier one wrote through plain pointers: a load that the compiler
-// may take for invariant (const __restrict__) is not ordered by the wait's memory clobber.
+// access.  Kernels read what an earlier one wrote through plain pointers and loads: the read-only
+// path (__ldg, and what the compiler makes of const __restrict__) is for data that no one writes
+// during the kernel's whole lifetime, which begins before the wait, so the wait does not order it.
 // pdl_release lets the next kernel be scheduled once some thread of every block has called it (or
 // the block has ended).  The tensor-core kernels call it when their work is done: blocks of the
 // next kernel that sit on the SMs for the whole of a long kernel, waiting, cost power (the text8b

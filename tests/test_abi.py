@@ -275,3 +275,18 @@ def test_cluster_forms_are_built_apart():
                  "alr_cluster_gemm_max_clusters", "alr_cluster_launch_pair_gemm",
                  "alr_cluster_pair_gemm_max_pairs"):
         assert hasattr(h, name), name
+
+
+def test_kernels_read_no_memory_through_the_read_only_path():
+    """Every kernel is launched so that its lifetime overlaps the end of the one before it
+    (programmatic dependent launch) and reads what that one wrote after its wait.  The read-only
+    load path is for memory that nobody writes during a kernel's lifetime, and no wait orders
+    it, so no kernel uses it: neither __ldg nor the pointers the compiler may take for
+    invariant."""
+    pat = re.compile(r"__ldg\s*\(|__restrict__|ld\.global\.nc|ld\.global\.L\w+::\w+\.nc")
+    for d in (build_lib.CSRC, build_lib.CSRC_CLUSTER):
+        for f in sorted(os.listdir(d)):
+            with open(os.path.join(d, f)) as fh:
+                code = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
+            code = "\n".join(line.split("//")[0] for line in code.splitlines())
+            assert not pat.search(code), (f, pat.search(code).group(0))

@@ -119,3 +119,58 @@ def test_ira_draw_select_digits(L, max_b, bits):
     n_valid, anchor_pos, _ = orc.ira_draw(ok.numpy(), _u32(keys), _u32(off_u), K, max_b)
     assert np.array_equal(P.npi(out["n_valid"]), n_valid)
     assert np.array_equal(P.npi(out["anchor_pos"]), anchor_pos)
+
+
+def test_chained_calls_read_what_the_call_before_wrote():
+    """draw -> context, and draw -> plan -> label gather, issued back to back without a
+    synchronisation, each call overlapping the end of the one before, over the same buffers with
+    other keys, masks and offsets every round: each round's rows, bit for bit, against the
+    oracle.  Stale draws or plans of the round before would move whole rows."""
+    S, L, K, max_b, C, F, d, rounds = 5, 600, 15, 64, 13, 64, 32, 24
+    Pn, H = max_b - max_b // 2, max_b // 2
+    g = torch.Generator().manual_seed(77)
+    u32 = lambda *s: torch.randint(-(1 << 31), 1 << 31, s, generator=g,  # noqa: E731
+                                   dtype=torch.int64).to(torch.int32)
+    i32 = lambda *s: torch.empty(*s, dtype=torch.int32, device="cuda")  # noqa: E731
+    store = torch.randn(S * Pn, C, F, generator=g).to(torch.bfloat16)
+    labels = torch.randn(S * Pn, K, d, generator=g).to(torch.bfloat16)
+    rlen = torch.randint(1, K + 1, (S * Pn,), generator=g, dtype=torch.int32)
+    store_c, labels_c, rlen_c = store.cuda(), labels.cuda(), rlen.cuda()
+    ins, dev = [], []
+    for _ in range(rounds):
+        density = torch.rand(S, 1, generator=g) * 0.3
+        ins.append(((torch.rand(S, L, generator=g) < density).to(torch.uint8), u32(S, L), u32(S, H)))
+        dev.append([x.cuda() for x in ins[-1]])
+    out = dict(n_valid=i32(S), anchor_pos=i32(S, max_b), offsets=i32(S, H))
+    plan = {k: i32(S * max_b) for k in ("seq", "pos", "valid_len")}
+    new = lambda *s: [torch.empty(*s, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+                      for _ in range(rounds)]
+    ctx, rows = new(S, H, C, F), new(S * max_b * K, d)
+    row_valid = [torch.empty(S * max_b * K, device="cuda") for _ in range(rounds)]
+    ctx_len, prefix_end = [[i32(S, H) for _ in range(rounds)] for _ in range(2)]
+    torch.cuda.synchronize()
+    for i, (ok, keys, off_u) in enumerate(dev):
+        alr.alr_ira_draw(K, max_b, ok, keys, off_u, out)
+        alr.alr_ira_context(K, max_b, store_c, out["n_valid"], rlen_c, out["offsets"],
+                            out["anchor_pos"], ctx[i], ctx_len[i], prefix_end[i])
+        alr.alr_ira_draw(K, max_b, ok, keys, off_u, out)
+        alr.alr_ira_blocks(K, max_b, out["n_valid"], rlen_c, out["offsets"], plan)
+        alr.alr_gather_ira_blocks(labels_c, plan["seq"], plan["pos"], K, rows[i], row_valid[i],
+                                  valid_len=plan["valid_len"])
+    torch.cuda.synchronize()
+    lens = rlen.numpy().reshape(S, Pn)
+    for i, (ok, keys, off_u) in enumerate(ins):
+        n_valid, anchor_pos, offsets = orc.ira_draw(ok.numpy(), _u32(keys), _u32(off_u), K, max_b)
+        c, cl, pe = orc.ira_context(store.float().numpy(), n_valid, lens, offsets, anchor_pos, K,
+                                    max_b)
+        assert torch.equal(ctx[i].float().cpu(), torch.from_numpy(c).float()), i
+        assert np.array_equal(P.npi(ctx_len[i]), cl) and np.array_equal(P.npi(prefix_end[i]), pe), i
+        ref = orc.ira_blocks(n_valid, lens, offsets, K, max_b)
+        seq, pos, vl = (ref[k].reshape(-1, 1) for k in ("seq", "pos", "valid_len"))
+        at = pos + np.arange(K)
+        live = (seq >= 0) & (at < np.minimum(vl, K))
+        want = labels.float().numpy()[np.where(live, seq, 0), np.where(live, at, 0)]
+        want[~live] = 0.0
+        assert np.array_equal(rows[i].float().cpu().numpy().reshape(want.shape), want), i
+        assert np.array_equal(row_valid[i].cpu().numpy().reshape(live.shape), live), i
+    assert alr.alr_device_status() == alr.ALR_OK
