@@ -317,11 +317,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_release();   // past the barrier: idle lanes and warps are here early
   if constexpr (kSplit) {
     cluster_sync();   // every CTA's partial sums are in its shared memory
-    int mb, nb;
-    decode_tile(args, t0, mb, nb);
-    reduce_split<kAcc, kBM / kSplitBlock, kBN / kSplitBlock>(args, mb * kBM, nb * kBN, smem, rank,
-                                                         int(cluster_nctarank()), warp,
-                                                         kThreads / 32, lane);
+    // A CTA whose wait ran out has none (its epilogue posted 0 for the cluster's only tile): then
+    // no CTA of the cluster touches C, as in the other forms.
+    const int n_cta = int(cluster_nctarank());
+    const bool posted =
+        lane >= n_cta ||
+        ld_cluster_s32(cluster_smem_addr(const_cast<const int*>(tile_ready), uint32_t(lane))) != 0;
+    if (__all_sync(0xffffffffu, posted)) {
+      int mb, nb;
+      decode_tile(args, t0, mb, nb);
+      reduce_split<kAcc, kBM / kSplitBlock, kBN / kSplitBlock>(args, mb * kBM, nb * kBN, smem,
+                                                               rank, n_cta, warp, kThreads / 32,
+                                                               lane);
+    }
     __syncwarp();
   }
   // no CTA leaves while its peers may still write into it, or read its partial sums

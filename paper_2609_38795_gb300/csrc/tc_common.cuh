@@ -347,6 +347,12 @@ ALR_DEV uint32_t cluster_smem_addr(const void* p, uint32_t rank) {
   return r;
 }
 
+ALR_DEV int ld_cluster_s32(uint32_t cluster_addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
+
 ALR_DEV float4 ld_cluster_v4(uint32_t cluster_addr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"

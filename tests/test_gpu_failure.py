@@ -78,6 +78,36 @@ def test_withheld_gemm_stage_times_out_and_context_survives(form, monkeypatch):
     assert P.max_norm_rel(P.np64(C), ref) <= 1e-3
 
 
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("shape", [(128, 64, 8200), (304, 512, 4000), (2200, 2056, 520),
+                                   (104, 8200, 72)])
+def test_withheld_stage_of_the_chosen_form_leaves_c_alone(shape, accumulate, monkeypatch):
+    """The forms products take by size: K split over clusters of 16 and of 5 CTAs, multicast
+    clusters, single CTAs.  No tile's sum is complete when the waits run out, so none is stored
+    or added: C keeps every bit.  The next product is correct."""
+    monkeypatch.delenv("ALR_GEMM_FORM", raising=False)
+    M, Nc, K = shape
+    g = torch.Generator(device="cuda").manual_seed(5)
+    A = torch.randn(M, K, device="cuda", generator=g).to(torch.bfloat16)
+    Bm = torch.randn(Nc, K, device="cuda", generator=g).to(torch.bfloat16)
+    C = torch.randn(M, Nc, device="cuda", generator=g)
+    before = C.clone()
+    assert alr.alr_device_status(clear=True) == alr.ALR_OK
+    alr.alr_debug_withhold_next_stage(True)
+    t0 = time.monotonic()
+    alr.alr_gemm(A, Bm, C, M, Nc, K, accumulate=accumulate)
+    rc = alr.alr_device_status(clear=True)
+    waited = time.monotonic() - t0
+    assert rc == alr.ALR_ERR_TIMEOUT, alr.alr_last_error()
+    assert waited < 20.0
+    assert torch.equal(C, before)
+    alr.alr_gemm(A, Bm, C, M, Nc, K, accumulate=accumulate)
+    torch.cuda.synchronize()
+    assert alr.alr_device_status() == alr.ALR_OK
+    ref = P.np64(A) @ P.np64(Bm).T + (P.np64(before) if accumulate else 0.0)
+    assert P.max_norm_rel(P.np64(C), ref) <= 1e-3
+
+
 def test_binding_refuses_wrong_device_buffers():
     """Buffers the kernels would read or write out of bounds, or misread, are refused by the
     binding with the argument's name, and nothing is launched (the status stays clean)."""
