@@ -1,14 +1,16 @@
 // Merge of the fused loss kernels' partial records into the per-row results, the slot weights and
 // the batch sums of Eq. 1: the full-vocabulary forward, the label readout and the top-k forward.
 //
-// A row has one partial record per vocabulary split and column group (up to 608 of them), so
-// the merge is a reduction over records as much as a map over rows.  A block takes kRows rows
+// A row has one partial record per vocabulary split and column group (tens to some 2400 of them),
+// so the merge is a reduction over records as much as a map over rows.  A block takes kRows rows
 // (whole anchors) and kWarps warps; a lane holds one row and walks every (kWarps * 32 / kRows)-th
 // record of it, the lanes of a row are then merged by shuffles and the warps through shared
-// memory, in a fixed order.  Latency-bound (a chain of dependent record loads per lane), so the
-// split over records is what sets its time: 23 us at 128 rows and 608 records and 25 us at 4096
-// rows and 76 records, against 1087 and 230 us with one warp per anchor (for the readout one
-// thread per row: 512 us at 768 rows and 200 records, now 34) walking all records in fp64.
+// memory, in a fixed order.  The row's maxima over all records are found first, so every record's
+// sums are multiplied by one factor only, and all sums of exponentials are held in fp64.  Bound by
+// latency (record loads) and, in few blocks, by the fp64 rate, so the split over records is what
+// sets its time: 31 us at 128 rows and 608 records (25 with two-float sums and the maxima moved
+// record by record, whose results were further from the fp64 reference), 16 us at 2000 rows and
+// 76 records, against 1087 us at 128 rows with one warp per anchor walking all records.
 #include <cfloat>
 
 #include "kernels.h"
@@ -20,40 +22,37 @@ namespace {
 
 ALR_DEV float quiet_nan() { return __int_as_float(0x7fc00000); }
 
-// ------------------------------------------------------------- two-float sums ---
-// A sum of exponentials is held as s + c (c: the rounding errors of s), about 2^-44 relative:
-// with a sharp softmax its logarithm is the near-zero part of the loss and the entropy.  fp64
-// would do the same at 1/64 of the fp32 rate.
-ALR_DEV void scale2(float& s, float& c, float f) {
-  const float h = s * f;
-  c = fmaf(c, f, fmaf(s, f, -h));
-  s = h;
-}
-ALR_DEV void add2(float& s, float& c, float s2, float c2) {
-  const float t = s + s2, b = t - s;
-  const float e = (s - (t - b)) + (s2 - b);
-  s = t;
-  c += c2 + e;
-}
-ALR_DEV double value2(float s, float c) { return double(s) + double(c); }
-
-// (s, c) divided by 2^r, the factor its exponentials carry (r: the exponent residual of their
-// reference, |r| <= 4e-3 over the fp16 range of logits): 2^-r = 1 - y, y = x - x^2 / 2 with
-// x = r ln 2, within 1e-8 relative (1e-14 for |r| <= 3e-5, |logit| < 1000).
-ALR_DEV void unscale_residual(float& s, float& c, float r) {
-  const float x = r * kLn2;
-  const float y = fmaf(-0.5f * x, x, x);
-  add2(s, c, -s * y, -c * y);
+// ----------------------------------------------------------------- record sums ---
+// A part's sum of exponentials arrives as s + c (c: the rounding errors of s) and is merged in
+// fp64: with a sharp softmax its logarithm is the near-zero part of the loss and the entropy.
+// fp64 instructions, conversions to it among them, run at 1/64 of the fp32 rate, so a value is
+// widened by moving its bits (normal numbers and zero; smaller ones become zero).
+ALR_DEV double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+  const unsigned hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u + (b & 0x80000000u);
+  return __hiloint2double(int(e == 0 ? 0u : hi), int(e == 0 ? 0u : b << 29));
 }
 
-// Factor exp(m - nm) of a sum moved from reference m to nm >= m (1 when they are equal).
-ALR_DEV float rescale(float m, float nm) { return ex2((m - nm) * kLog2e); }
+// acc + f (s + c)
+ALR_DEV double add_part(double acc, float f, float s, float c) {
+  const double f64 = widen(f);
+  return fma(f64, widen(s), fma(f64, widen(c), acc));
+}
 
-// Top-2 of two disjoint column sets (the leaders' values are the running maxima); equal leaders go
-// to the lower token id.
-ALR_DEV void merge_top2(float best, float& sec, int& id, float best2, float sec2, int id2) {
+// The row's sums carry the factor 2^r of its maximum m (exp_residual): the sum divided by it, and
+// its natural logarithm.  With x = r ln 2, 1 - x + x^2 / 2 leaves x^3 / 6, 5e-9 at |r| = 4e-3
+// (the fp16 range of logits) and 1e-14 at 6e-5 (|logit| < 1000).
+ALR_DEV double ln_residual(float m) { return double(exp_residual(m)) * 0.6931471805599453; }
+ALR_DEV double without_residual(double s, float m) {
+  const double x = ln_residual(m);
+  return s * (1.0 - x + 0.5 * x * x);
+}
+
+// Top-2 of two disjoint column sets; equal leaders go to the lower token id.
+ALR_DEV void merge_top2(float& best, float& sec, int& id, float best2, float sec2, int id2) {
   if (best2 > best || (best2 == best && id2 < id)) {
     sec = fmaxf(best, sec2);
+    best = best2;
     id = id2;
   } else {
     sec = fmaxf(sec, best2);
@@ -61,57 +60,67 @@ ALR_DEV void merge_top2(float best, float& sec, int& id, float best2, float sec2
 }
 
 // ------------------------------------------------------------------ row states ---
-// Each state is a plain record of 32-bit words: init() is a row with no columns, load() reads one
-// partial record (field stride fs), merge() folds in the state of other columns.
+// A state holds sums measured from the row's maxima over all records (`ref`, kRefs of them, found
+// first), so that every record's sums are multiplied by one factor, whatever the order of the
+// merge.  kWords: its 32-bit words, without padding.  init() is a row with no columns, Record one partial record (field stride fs), add()
+// folds a record in, merge() another state of the same row.
 struct FullState {
-  float md, sd, cd, mt, st, ct, u, w, secd, sect, zx;
+  double sd, st;
+  float u, w, bd, secd, bt, sect, zx;
   int id, it;
 
+  static constexpr int kWords = 13, kRefs = 2;
+  static ALR_DEV constexpr int ref_field(int i) { return i == 0 ? kPMd : kPMt; }
+
+  struct Record {
+    float md, sd, cd, mt, st, ct, u, w, secd, sect, zx;
+    int id, it;
+
+    ALR_DEV void load(const float* p, size_t fs) {
+      md = p[kPMd * fs];
+      sd = p[kPSd * fs];
+      cd = p[kPSdLo * fs];
+      mt = p[kPMt * fs];
+      st = p[kPSt * fs];
+      ct = p[kPStLo * fs];
+      u = p[kPU * fs];
+      w = p[kPW * fs];
+      secd = p[kPSecd * fs];
+      sect = p[kPSect * fs];
+      zx = p[kPZx * fs];
+      id = __float_as_int(p[kPId * fs]);
+      it = __float_as_int(p[kPIt * fs]);
+    }
+    ALR_DEV float ref(int i) const { return i == 0 ? md : mt; }
+  };
+
   ALR_DEV void init() {
-    md = mt = secd = sect = -INFINITY;
-    sd = cd = st = ct = u = w = 0.f;
+    sd = st = 0.0;
+    u = w = 0.f;
+    bd = bt = secd = sect = -INFINITY;
     zx = quiet_nan();
     id = it = 0x7fffffff;
   }
-  ALR_DEV void load(const float* p, size_t fs) {
-    md = p[kPMd * fs];
-    sd = p[kPSd * fs];
-    cd = p[kPSdLo * fs];
-    mt = p[kPMt * fs];
-    st = p[kPSt * fs];
-    ct = p[kPStLo * fs];
-    u = p[kPU * fs];
-    w = p[kPW * fs];
-    secd = p[kPSecd * fs];
-    sect = p[kPSect * fs];
-    zx = p[kPZx * fs];
-    id = __float_as_int(p[kPId * fs]);
-    it = __float_as_int(p[kPIt * fs]);
+  // u and w are measured from their part's maxima (z_d - md, z_t - mt): moved to the row's.
+  ALR_DEV void add(const Record& o, const float (&ref)[kRefs]) {
+    if (!(o.mt > -INFINITY)) return;       // no columns
+    const float dd = ref_step(o.md, -ref[0] * kLog2e), dt = ref_step(o.mt, -ref[1] * kLog2e);
+    const float ft = ex2(dt);
+    sd = add_part(sd, ex2(dd), o.sd, o.cd);
+    st = add_part(st, ft, o.st, o.ct);
+    u = fmaf(ft, fmaf(dd * kLn2, o.st, o.u), u);
+    w = fmaf(ft, fmaf(dt * kLn2, o.st, o.w), w);
+    merge_top2(bd, secd, id, o.md, o.secd, o.id);
+    merge_top2(bt, sect, it, o.mt, o.sect, o.it);
+    if (o.zx == o.zx) zx = o.zx;
   }
-  // u and w are measured from their own maxima (z_d - md, z_t - mt): both sides move to the
-  // merged references before they are added.
   ALR_DEV void merge(const FullState& o) {
-    if (!(o.mt > -INFINITY)) return;       // no columns: adds nothing
-    if (!(mt > -INFINITY)) {
-      *this = o;
-      return;
-    }
-    const float nmd = fmaxf(md, o.md), nmt = fmaxf(mt, o.mt);
-    const float ft = rescale(mt, nmt), fo = rescale(o.mt, nmt);
-    u = fmaf(md - nmd, st, u) * ft + fmaf(o.md - nmd, o.st, o.u) * fo;
-    w = fmaf(mt - nmt, st, w) * ft + fmaf(o.mt - nmt, o.st, o.w) * fo;
-    float s2 = o.st, c2 = o.ct;
-    scale2(st, ct, ft);
-    scale2(s2, c2, fo);
-    add2(st, ct, s2, c2);
-    s2 = o.sd, c2 = o.cd;
-    scale2(sd, cd, rescale(md, nmd));
-    scale2(s2, c2, rescale(o.md, nmd));
-    add2(sd, cd, s2, c2);
-    merge_top2(md, secd, id, o.md, o.secd, o.id);
-    merge_top2(mt, sect, it, o.mt, o.sect, o.it);
-    md = nmd;
-    mt = nmt;
+    sd += o.sd;
+    st += o.st;
+    u += o.u;
+    w += o.w;
+    merge_top2(bd, secd, id, o.bd, o.secd, o.id);
+    merge_top2(bt, sect, it, o.bt, o.sect, o.it);
     if (o.zx == o.zx) zx = o.zx;
   }
 };
@@ -133,13 +142,35 @@ ALR_DEV void insert_ranked(float (&t)[kTopK], int (&ti)[kTopK], float v, int id)
 }
 
 struct ReadoutState {
-  float m, s, c, zx;
-  float t[kTopK];
+  double s;
+  float zx;
+  float t[kTopK];               // t[0]: the row's maximum
   int ti[kTopK];
 
+  static constexpr int kWords = 3 + 2 * kTopK, kRefs = 1;
+  static ALR_DEV constexpr int ref_field(int) { return kRM; }
+
+  struct Record {
+    float m, s, c, zx;
+    float t[kTopK];
+    int ti[kTopK];
+
+    ALR_DEV void load(const float* p, size_t fs) {
+      m = p[kRM * fs];
+      s = p[kRS * fs];
+      c = p[kRSLo * fs];
+      zx = p[kRZx * fs];
+#pragma unroll
+      for (int i = 0; i < kTopK; ++i) {
+        t[i] = p[(kRTop + i) * fs];
+        ti[i] = __float_as_int(p[(kRIdx + i) * fs]);
+      }
+    }
+    ALR_DEV float ref(int) const { return m; }
+  };
+
   ALR_DEV void init() {
-    m = -INFINITY;
-    s = c = 0.f;
+    s = 0.0;
     zx = quiet_nan();
 #pragma unroll
     for (int i = 0; i < kTopK; ++i) {
@@ -147,94 +178,78 @@ struct ReadoutState {
       ti[i] = 0x7fffffff;
     }
   }
-  ALR_DEV void load(const float* p, size_t fs) {
-    m = p[kRM * fs];
-    s = p[kRS * fs];
-    c = p[kRSLo * fs];
-    zx = p[kRZx * fs];
+  // The other list's entries largest first: the first that stays out ends the merge.  Entries
+  // past a part's columns are -inf with the largest id and never enter.
+  ALR_DEV void merge_list(const float (&t2)[kTopK], const int (&ti2)[kTopK]) {
 #pragma unroll
     for (int i = 0; i < kTopK; ++i) {
-      t[i] = p[(kRTop + i) * fs];
-      ti[i] = __float_as_int(p[(kRIdx + i) * fs]);
+      const float v = t2[i];
+      const bool in = v > t[kTopK - 1] || (v == t[kTopK - 1] && ti2[i] < ti[kTopK - 1]);
+      if (!in) break;
+      insert_ranked(t, ti, v, ti2[i]);
     }
-    if (m > -INFINITY) unscale_residual(s, c, exp_residual(m));
+  }
+  ALR_DEV void add(const Record& o, const float (&ref)[kRefs]) {
+    if (!(o.m > -INFINITY)) return;
+    s = add_part(s, ex2(ref_step(o.m, -ref[0] * kLog2e)), o.s, o.c);
+    if (o.zx == o.zx) zx = o.zx;
+    merge_list(o.t, o.ti);
   }
   ALR_DEV void merge(const ReadoutState& o) {
-    if (!(o.m > -INFINITY)) return;
-    if (!(m > -INFINITY)) {
-      *this = o;
-      return;
-    }
-    const float nm = fmaxf(m, o.m);
-    float s2 = o.s, c2 = o.c;
-    scale2(s, c, rescale(m, nm));
-    scale2(s2, c2, rescale(o.m, nm));
-    add2(s, c, s2, c2);
-    m = nm;
+    s += o.s;
     if (o.zx == o.zx) zx = o.zx;
-    // the other list's entries largest first: the first that stays out ends the merge.  Entries
-    // past a part's columns are -inf with the largest id and never enter.
-#pragma unroll
-    for (int i = 0; i < kTopK; ++i) {
-      const float v = o.t[i];
-      const bool in = v > t[kTopK - 1] || (v == t[kTopK - 1] && o.ti[i] < ti[kTopK - 1]);
-      if (!in) break;
-      insert_ranked(t, ti, v, o.ti[i]);
-    }
+    merge_list(o.t, o.ti);
   }
 };
 
 struct TopkState {
-  float m, s, c, so, co, sec;   // s + c: all columns; so + co: the columns outside the label
+  double s, so;                 // all columns; the columns outside the label
+  float best, sec;
   int id;
   float z[kTopK];               // z_d at the label tokens, NaN until their column is met
 
+  static constexpr int kWords = 7 + kTopK, kRefs = 1;
+  static ALR_DEV constexpr int ref_field(int) { return kKM; }
+
+  struct Record {
+    float m, s, c, in, sec;
+    int id;
+    float z[kTopK];
+
+    ALR_DEV void load(const float* p, size_t fs) {
+      m = p[kKM * fs];
+      s = p[kKS * fs];
+      c = p[kKSLo * fs];
+      in = p[kKSIn * fs];
+      sec = p[kKSec * fs];
+      id = __float_as_int(p[kKIdx * fs]);
+#pragma unroll
+      for (int i = 0; i < kTopK; ++i) z[i] = p[(kKZ + i) * fs];
+    }
+    ALR_DEV float ref(int) const { return m; }
+  };
+
   ALR_DEV void init() {
-    m = sec = -INFINITY;
-    s = c = so = co = 0.f;
+    s = so = 0.0;
+    best = sec = -INFINITY;
     id = 0x7fffffff;
 #pragma unroll
     for (int i = 0; i < kTopK; ++i) z[i] = quiet_nan();
   }
-  ALR_DEV void load(const float* p, size_t fs) {
-    m = p[kKM * fs];
-    s = p[kKS * fs];
-    c = p[kKSLo * fs];
-    const float in = p[kKSIn * fs];
-    sec = p[kKSec * fs];
-    id = __float_as_int(p[kKIdx * fs]);
+  ALR_DEV void add(const Record& o, const float (&ref)[kRefs]) {
+    if (!(o.m > -INFINITY)) return;
+    const float f = ex2(ref_step(o.m, -ref[0] * kLog2e));
+    s = add_part(s, f, o.s, o.c);
+    so = fma(widen(f), (widen(o.s) - widen(o.in)) + widen(o.c), so);
+    merge_top2(best, sec, id, o.m, o.sec, o.id);
 #pragma unroll
-    for (int i = 0; i < kTopK; ++i) z[i] = p[(kKZ + i) * fs];
-    so = s;
-    co = 0.f;
-    add2(so, co, -in, 0.f);
-    const float lo = co + c;               // back to a leading value and its small error
-    co = 0.f;
-    add2(so, co, lo, 0.f);
-    if (m > -INFINITY) {
-      const float r = exp_residual(m);
-      unscale_residual(s, c, r);
-      unscale_residual(so, co, r);
-    }
+    for (int i = 0; i < kTopK; ++i)
+      if (o.z[i] == o.z[i]) z[i] = o.z[i];
   }
   ALR_DEV void merge(const TopkState& o) {
-    if (!(o.m > -INFINITY)) return;
-    if (!(m > -INFINITY)) {
-      *this = o;
-      return;
-    }
-    const float nm = fmaxf(m, o.m);
-    const float f = rescale(m, nm), fo = rescale(o.m, nm);
-    float s2 = o.s, c2 = o.c;
-    scale2(s, c, f);
-    scale2(s2, c2, fo);
-    add2(s, c, s2, c2);
-    s2 = o.so, c2 = o.co;
-    scale2(so, co, f);
-    scale2(s2, c2, fo);
-    add2(so, co, s2, c2);
-    merge_top2(m, sec, id, o.m, o.sec, o.id);
-    m = nm;
+    s += o.s;
+    so += o.so;
+    merge_top2(best, sec, id, o.best, o.sec, o.id);
 #pragma unroll
     for (int i = 0; i < kTopK; ++i)
       if (o.z[i] == o.z[i]) z[i] = o.z[i];
@@ -242,34 +257,32 @@ struct TopkState {
 };
 
 template <class St>
-constexpr int kWords = int(sizeof(St) / 4);
-
-template <class St>
 ALR_DEV St shfl_xor_state(const St& s, int mask) {
   St o;
   const uint32_t* a = reinterpret_cast<const uint32_t*>(&s);
   uint32_t* b = reinterpret_cast<uint32_t*>(&o);
 #pragma unroll
-  for (int i = 0; i < kWords<St>; ++i) b[i] = __shfl_xor_sync(0xffffffffu, a[i], mask);
+  for (int i = 0; i < St::kWords; ++i) b[i] = __shfl_xor_sync(0xffffffffu, a[i], mask);
   return o;
 }
 
 // Shared memory of the merge: one state per warp and row, word-major so that a warp's rows are
-// consecutive words.
+// consecutive words, and the warps' maxima.
 template <class St, int kRows, int kWarps>
 struct MergeSmem {
-  uint32_t w[kWarps][kWords<St>][kRows];
+  uint32_t w[kWarps][St::kWords][kRows];
+  float ref[kWarps][St::kRefs][kRows];
 
   ALR_DEV void put(int warp, int rr, const St& s) {
     const uint32_t* a = reinterpret_cast<const uint32_t*>(&s);
 #pragma unroll
-    for (int i = 0; i < kWords<St>; ++i) w[warp][i][rr] = a[i];
+    for (int i = 0; i < St::kWords; ++i) w[warp][i][rr] = a[i];
   }
   ALR_DEV St get(int warp, int rr) const {
     St s;
     uint32_t* a = reinterpret_cast<uint32_t*>(&s);
 #pragma unroll
-    for (int i = 0; i < kWords<St>; ++i) a[i] = w[warp][i][rr];
+    for (int i = 0; i < St::kWords; ++i) a[i] = w[warp][i][rr];
     return s;
   }
 };
@@ -284,14 +297,46 @@ ALR_DEV void merge_rows(const LossPlan& P, const float* part, int row0, int n_ro
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rr = lane % kRows, slot = lane / kRows;
   const size_t fs = size_t(P.n_parts) * size_t(P.N);
+  const float* col = part + size_t(row0 + rr);
+  const int k0 = warp * kSlots + slot, step = kWarps * kSlots;
+  const bool any = rr < n_rows && k0 < P.n_parts;
+  // this lane's first record, on its way while the maxima are found
+  typename St::Record first;
+  if (any) first.load(col + size_t(k0) * size_t(P.N), fs);
+  // the row's maxima
+  float ref[St::kRefs];
+#pragma unroll
+  for (int i = 0; i < St::kRefs; ++i) ref[i] = any ? first.ref(i) : -INFINITY;
+  if (rr < n_rows) {
+#pragma unroll 8
+    for (int k = k0 + step; k < P.n_parts; k += step) {
+#pragma unroll
+      for (int i = 0; i < St::kRefs; ++i)
+        ref[i] = fmaxf(ref[i], col[size_t(k) * size_t(P.N) + size_t(St::ref_field(i)) * fs]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < St::kRefs; ++i) {
+#pragma unroll
+    for (int off = kRows; off < 32; off <<= 1)
+      ref[i] = fmaxf(ref[i], __shfl_xor_sync(0xffffffffu, ref[i], off));
+    if (lane < kRows) sm.ref[warp][i][rr] = ref[i];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < St::kRefs; ++i)
+#pragma unroll
+    for (int n = 0; n < kWarps; ++n) ref[i] = fmaxf(ref[i], sm.ref[n][i][rr]);
+
   St st;
   st.init();
+  if (any) st.add(first, ref);
   if (rr < n_rows) {
 #pragma unroll 2
-    for (int k = warp * kSlots + slot; k < P.n_parts; k += kWarps * kSlots) {
-      St o;
-      o.load(part + size_t(k) * size_t(P.N) + size_t(row0 + rr), fs);
-      st.merge(o);
+    for (int k = k0 + step; k < P.n_parts; k += step) {
+      typename St::Record o;
+      o.load(col + size_t(k) * size_t(P.N), fs);
+      st.add(o, ref);
     }
   }
 #pragma unroll
@@ -399,7 +444,7 @@ struct FullOut {
 };
 
 template <int kRows, int kWarps>
-__global__ void __launch_bounds__(32 * kWarps)
+__global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
     combine_kernel(LossPlan P, const float* part, int rows_per_block, int mode,
                    float gamma, const float* row_mask,
                    const int32_t* corpus_tok, FullOut o, BatchOut bo) {
@@ -410,26 +455,28 @@ __global__ void __launch_bounds__(32 * kWarps)
   merge_rows<FullState, kRows, kWarps>(P, part, row0, n_rows, sm);
   const bool erase = mode != 0;
   // one thread per row and side: both are log S - X / S_t with X = u (drafter: the loss) or w
-  // (target: the entropy), two non-negative terms, in fp64
+  // (target: the entropy), two non-negative terms, in fp64.  The residual of the side's maximum
+  // is in log S and in X / S_t alike (X's terms are the exponents themselves), and cancels.
   const int side = threadIdx.x / kRows, sr = threadIdx.x % kRows;
   if (side < 2 && sr < n_rows) {
     const FullState st = sm.get(0, sr);
     const int r = row0 + sr;
-    const double ls = log(side == 0 ? value2(st.sd, st.cd) : value2(st.st, st.ct));
+    const double ls = log(side == 0 ? st.sd : st.st);
     const double x = double(side == 0 ? st.u : st.w);
-    const float v = float(ls - x / value2(st.st, st.ct));
-    const float lse = (side == 0 ? st.md : st.mt) + float(ls);
+    const float v = float(ls - x / st.st);
+    const float m = side == 0 ? st.bd : st.bt;
+    const float lse = m + float(ls - ln_residual(m));
     if (side == 0) {
       o.loss_row[r] = v;
       s_loss[sr] = v;
       o.lse_d[r] = lse;
       o.argmax_d[r] = st.id;
-      if (o.gap_d) o.gap_d[r] = st.md - st.secd;
+      if (o.gap_d) o.gap_d[r] = st.bd - st.secd;
     } else {
       if (o.ent_row) o.ent_row[r] = v;
       o.lse_t[r] = lse;
       o.argmax_t[r] = st.it;
-      if (o.gap_t) o.gap_t[r] = st.mt - st.sect;
+      if (o.gap_t) o.gap_t[r] = st.bt - st.sect;
       s_logp[sr] = st.zx - lse;
       if (erase && o.logp_x) o.logp_x[r] = st.zx - lse;
     }
@@ -461,7 +508,7 @@ __global__ void __launch_bounds__(32 * kWarps)
 // and the tail mass (S - sum_k exp(t_k - M)) / S, the greedy token with its top-1 minus top-2
 // gap, and log p at the corpus token.  Rows are independent.
 template <int kRows, int kWarps>
-__global__ void __launch_bounds__(32 * kWarps)
+__global__ void __launch_bounds__(32 * kWarps, 1)
     readout_combine_kernel(LossPlan P, const float* part, int has_corpus,
                            int32_t* top_idx, float* top_prob,
                            float* tail, float* lse_t,
@@ -485,26 +532,27 @@ __global__ void __launch_bounds__(32 * kWarps)
           ti = st.t[j];
           id = st.ti[j];
         }
-      const double e = exp(double(ti) - double(st.m));
+      const double e = exp(double(ti) - double(st.t[0]));
+      const double S = without_residual(st.s, st.t[0]);
       s_e[i][rr] = e;
       top_idx[size_t(row0 + rr) * kTopK + i] = id;
-      top_prob[size_t(row0 + rr) * kTopK + i] = float(e / value2(st.s, st.c));
+      top_prob[size_t(row0 + rr) * kTopK + i] = float(e / S);
     }
   }
   __syncthreads();
   if (int(threadIdx.x) < n_rows) {
     const int rr = threadIdx.x, r = row0 + rr;
     const ReadoutState st = sm.get(0, rr);
-    const double S = value2(st.s, st.c), ls = log(S);
+    const double S = without_residual(st.s, st.t[0]), ls = log(S);
     double inside = 0.0;
 #pragma unroll
     for (int i = 0; i < kTopK; ++i) inside += s_e[i][rr];
     // with V <= k every token is in the list and the tail is empty by definition
     tail[r] = P.V <= kTopK ? 0.f : float(fmax(0.0, (S - inside) / S));
-    if (lse_t) lse_t[r] = st.m + float(ls);
+    if (lse_t) lse_t[r] = st.t[0] + float(ls);
     if (argmax_t) argmax_t[r] = st.ti[0];
     if (gap_t) gap_t[r] = st.t[0] - st.t[1];
-    if (has_corpus && logp_x) logp_x[r] = float((double(st.zx) - double(st.m)) - ls);
+    if (has_corpus && logp_x) logp_x[r] = float((double(st.zx) - double(st.t[0])) - ls);
   }
 }
 
@@ -519,7 +567,7 @@ struct TopkOut {
 };
 
 template <int kRows, int kWarps>
-__global__ void __launch_bounds__(32 * kWarps)
+__global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
     topk_combine_kernel(LossPlan P, const float* part, int rows_per_block,
                         const float* top_prob, const float* tail,
                         const float* row_mask, const float* weight_in,
@@ -532,13 +580,13 @@ __global__ void __launch_bounds__(32 * kWarps)
   if (int(threadIdx.x) < n_rows) {         // n_rows <= 32: the first warp
     const int s = threadIdx.x % P.B, r = row0 + threadIdx.x;
     const TopkState st = sm.get(0, threadIdx.x);
-    const double S = value2(st.s, st.c), ls = log(S);
+    const double S = without_residual(st.s, st.best), ls = log(S);
     // log q_i = (z_i - M) - log S: the difference z_i - M is exact in fp64
     double ce = 0.0;
 #pragma unroll
     for (int i = 0; i < kTopK; ++i)
-      ce -= double(top_prob[size_t(r) * kTopK + i]) * ((double(st.z[i]) - double(st.m)) - ls);
-    const double tq = fmax(value2(st.so, st.co) / S, 1e-30);
+      ce -= double(top_prob[size_t(r) * kTopK + i]) * ((double(st.z[i]) - double(st.best)) - ls);
+    const double tq = fmax(st.so / st.s, 1e-30);
     const float tl = tail[r];
     if (tl > 0.f) ce -= double(tl) * log(tq);
     const float loss = float(ce);
@@ -546,10 +594,10 @@ __global__ void __launch_bounds__(32 * kWarps)
                         ? weight_in[r]
                         : expf(-float(s) / gamma) * (row_mask ? row_mask[r] : 1.f);
     o.loss_row[r] = loss;
-    o.lse_d[r] = st.m + float(ls);
+    o.lse_d[r] = st.best + float(ls);
     o.tail_q[r] = float(tq);
     o.argmax_d[r] = st.id;
-    if (o.gap_d) o.gap_d[r] = st.m - st.sec;
+    if (o.gap_d) o.gap_d[r] = st.best - st.sec;
     o.weight[r] = w;
     wl = double(w) * double(loss);
     ws = double(w);

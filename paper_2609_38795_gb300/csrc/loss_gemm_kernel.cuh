@@ -183,8 +183,8 @@ ALR_DEV void sum2_scaled(float& s, float& c, float sc, float x) {
 // were rescaled by.
 ALR_DEV float lse_update(float& m, float& s, float& c, const float (&z)[16], float cm) {
   const float nm = fmaxf(m, cm);
-  const float sc = ex2((m - nm) * kLog2e);
   const float b = -nm * kLog2e;
+  const float sc = ex2(ref_step(m, b));
   const uint64_t l2e = f2_pack(kLog2e, kLog2e), b2 = f2_pack(b, b);
   uint64_t r = f2_pack(0.f, 0.f);
 #pragma unroll
@@ -345,10 +345,10 @@ ALR_DEV void stats_sub(RowStats& st, const uint32_t (&rd)[16], const uint32_t (&
   // u, w: move to the new references (skipped while nothing has been summed: the old
   // reference is still -inf), rescale, add this sub-chunk
   const bool any = st.s_t > 0.f;
-  const float u_sh = any ? fmaf(st.best_d - nbd, st.s_t + st.c_t, st.u) : 0.f;
-  const float w_sh = any ? fmaf(st.best_t - nbt, st.s_t + st.c_t, st.w) : 0.f;
-  const float sct = ex2((st.best_t - nbt) * kLog2e);
-  const float scd = ex2((st.best_d - nbd) * kLog2e);
+  const float step_t = ref_step(st.best_t, bt), step_d = ref_step(st.best_d, bd);
+  const float u_sh = any ? fmaf(step_d * kLn2, st.s_t + st.c_t, st.u) : 0.f;
+  const float w_sh = any ? fmaf(step_t * kLn2, st.s_t + st.c_t, st.w) : 0.f;
+  const float sct = ex2(step_t), scd = ex2(step_d);
   st.u = fmaf(u_sh, sct, (u0 + u1) * kLn2);
   st.w = fmaf(w_sh, sct, (w0 + w1) * kLn2);
   sum2_scaled(st.s_t, st.c_t, sct, s0 + s1);

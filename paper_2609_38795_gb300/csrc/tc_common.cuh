@@ -38,11 +38,18 @@ ALR_DEV float ex2(float x) {
   return y;
 }
 
-// The exponent every column gets relative to the reference m is fma(z, log2 e, -m log2 e),
-// which at z = m is not 0 but the rounding residual of m log2 e (exactly representable, up to
-// ~4e-6 at |m| ~ 40): every exponential summed against m carries the factor 2^r.  The merge
-// divides it out, so that log S and the log-probabilities taken from it keep their precision.
+// The exponent every column gets relative to the reference m is fma(z, log2 e, b(m)) with
+// b(m) = -m log2 e rounded, which at z = m is not 0 but the rounding residual of m log2 e (exactly
+// representable, up to ~4e-6 at |m| ~ 40): every exponential summed against m carries the factor
+// 2^r, which is divided out of the row's sums, so that log S and the log-probabilities taken
+// from it keep their precision.
 ALR_DEV float exp_residual(float m) { return fmaf(m, kLog2e, -m * kLog2e); }
+
+// Exponent of the step from the reference m to one with b = b(nm), nm >= m: the difference of the
+// rounded offsets, so that sums that carry m's factor 2^r carry nm's after it (multiplied by
+// exp(m - nm) instead, the terms met before each new maximum keep another factor than the rest:
+// 1e-6 at |m| ~ 30).
+ALR_DEV float ref_step(float m, float b) { return __fadd_rn(b, __fmul_rn(m, kLog2e)); }
 
 // ------------------------------------------------------ paired fp32 arithmetic ---
 // Two fp32 lanes in one 64-bit register, combined by the sm_100-family packed instructions:

@@ -106,6 +106,41 @@ def test_forward_at_uneven_row_blocks(N):
     assert alr.alr_device_status() == alr.ALR_OK
 
 
+@pytest.mark.parametrize("N,d,V", [(192, 320, 1400), (512, 256, 60000), (2000, 704, 20000)])
+def test_sums_keep_their_precision_at_large_logits(N, d, V):
+    """What the running sums and their merge lose, apart from the products: hidden states of -1, 0
+    and 1 and head weights in steps of 2^-8 make every logit exact in fp32 in any order of
+    summation (below 2^20 steps), with row maxima of 20 to 40.  Tiles of 128 and of 256 columns.
+
+    A result is rounded once (2^-24).  Its sums take one rounded exponent and one ex2.approx
+    (2^-22 at most, 2^-24 rms) per column, whose errors average out over the few columns that
+    matter: 2^-23 rms is left for a loss or an entropy, 2^-24 for log S (relative to its
+    size, about 30).  Terms summed against an earlier maximum that keep its exponent's
+    residual (2^-25 of 40 log2 e, 1.7e-6) do not average out: they gave 1.5e-7 to 3e-7."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    w = torch.randn(d, V, device="cuda", generator=g) * (20.0 / d ** 0.5)
+    W = (torch.clamp(torch.round(w * 256), -255, 255) / 256).to(torch.bfloat16)
+    draw = lambda: ((torch.rand(N, d, device="cuda", generator=g) < 0.25).float()  # noqa: E731
+                    * torch.randn(N, d, device="cuda", generator=g).sign()).to(torch.bfloat16)
+    Ht = draw()
+    Hd = torch.where(torch.rand(N, d, device="cuda", generator=g) < 0.2, draw(), Ht)
+    zd, zt = Hd.double() @ W.double(), Ht.double() @ W.double()
+    lse_d, lse_t = zd.logsumexp(1), zt.logsumexp(1)
+    p = (zt - lse_t[:, None]).exp()
+    ref = dict(loss_row=lse_d - (p * zd).sum(1), ent_row=lse_t - (p * zt).sum(1), lse_d=lse_d,
+               lse_t=lse_t)
+    assert lse_d.min() > 15.0
+    out = P.gpu_forward(Hd, Ht, W, 16 if N % 16 == 0 else 8).out
+    lab = T.gpu_readout(Ht, W, 16 if N % 16 == 0 else 8)
+    ref["top_prob"] = p.gather(1, lab["top_idx"].long())
+    for k, x in ref.items():
+        got = (lab if k == "top_prob" else out)[k].double()
+        err = float((got - x).norm() / x.norm())
+        print(N, k, err)
+        assert err <= 2.0 ** (-24 if k in ("lse_d", "lse_t", "top_prob") else -23), (k, err)
+    assert alr.alr_device_status() == alr.ALR_OK
+
+
 def test_forward_workspace_stays_within_the_fixed_scratch():
     """Every bf16 problem whose records at 19 splits (15 fp32 fields per row, split and
     64-column group: what the no-workspace forward's limit was set for) fit the fixed 64 MiB
