@@ -172,7 +172,9 @@ int check_kept(const alr_params* p, const void* Z, const void* ref, const char* 
 // a multi-rank process, and then the single form runs).  The dual-product modes already share
 // each head tile between z_d and z_t, and at the power cap the multicast form settles ~4 %
 // lower in clock for ~1 % fewer L2 bytes per product: it is not faster, so it is not the
-// default.  Both forms give bit-identical results.
+// default.  It needs 256-column tiles: where loss_tile_columns takes 128, single CTAs run.  The tiles
+// and splits depend on the problem alone, so both forms give bit-identical results and take the
+// same workspace.
 bool loss_multicast(const alr_params* p) {
   if (p->dtype != ALR_BF16) return false;
   const char* v = getenv("ALR_LOSS_FORM");
@@ -188,12 +190,9 @@ enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
 // 256 forward 202 -> 183, keeping 246 -> 225, readout 199 -> 179; d = 512 261 -> 258, 309 -> 289,
 // 232 -> 210; d = 1000 410 -> 460), and everywhere when wide ones would not give each SM a tile
 // (192 x 320 x 1400: forward 18.4 -> 17.2, gradient 7.4 -> 5.6; d = 3072 42 -> 32 and 30 -> 21).
-// A loss form asked for by name runs on 256 columns, which the multicast form needs.
 constexpr int kNarrowBlocks = 10;
 
 int loss_tile_columns(const alr_params* p, int sms, bool bwd, int64_t n_rb) {
-  const char* v = getenv("ALR_LOSS_FORM");
-  if (v != nullptr && *v != '\0') return 256;
   if (n_rb * ((p->V + 255) / 256) <= sms) return 128;
   const int n_kb = (p->d + int(k_per_row(p->dtype)) - 1) / int(k_per_row(p->dtype));
   return !bwd && n_kb <= kNarrowBlocks ? 128 : 256;
@@ -255,16 +254,16 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   P.d = p->d;
   P.V = p->V;
   P.B = p->B;
-  P.mc = (!two_rows && loss_multicast(p)) ? 1 : 0;
   // row blocks; row-block pairs for the two-row modes and for the multicast form (which
   // places sms / 2 clusters).  Forward: the splits of forward_splits (the same for both
   // forms), in raster groups of up to two rounds of the grid at its base split (16 row blocks).
   // Recomputing backward: one vocabulary tile per unit, raster groups of 16 row blocks as well.
   const int rb = int((p->N + 127) / 128);
+  P.bn = loss_tile_columns(p, sms, bwd, two_rows ? (rb + 1) / 2 : rb);
+  P.mc = !two_rows && P.bn == 256 && loss_multicast(p) ? 1 : 0;
   const bool pairs = P.mc || two_rows;
   P.n_rb = pairs ? (rb + 1) / 2 : rb;
   const int group = pairs ? 4 : 8;
-  P.bn = loss_tile_columns(p, sms, bwd, P.n_rb);
   P.n_vt = (p->V + P.bn - 1) / P.bn;
   // two rounds per raster group: twice the row blocks share each W split, so W leaves DRAM
   // about half as often, with the same number of units per CTA (forward 49.8 against 50.0 ms at

@@ -24,14 +24,16 @@ def _lib():
     assert alr.alr_device_supported() == alr.ALR_OK, alr.alr_last_error()
 
 
-@pytest.mark.parametrize("form", ["single", "mcast"])
-def test_withheld_stage_times_out_and_context_survives(form, monkeypatch):
-    """Both forms of the fused kernel: single CTAs, and clusters of two CTAs that feed each
-    other's stages by multicast (every CTA of the cluster then runs out on its own barriers
+@pytest.mark.parametrize("form,d,V", [("single", 256, 1024), ("mcast", 256, 1024),
+                                      ("single", 648, 20000), ("mcast", 648, 20000)])
+def test_withheld_stage_times_out_and_context_survives(form, d, V, monkeypatch):
+    """The fused kernel on 128-column tiles (two accumulator buffers, single CTAs under either
+    name) and on 256-column ones (one buffer): single CTAs, and clusters of two CTAs that feed
+    each other's stages by multicast (every CTA of the cluster then runs out on its own barriers
     and both meet at the closing cluster barrier)."""
     monkeypatch.setenv("ALR_LOSS_FORM", form)
     assert alr.alr_kernel_forms()[1] == form, alr.alr_cluster_forms_error()
-    A, B, d, V = 16, 16, 256, 1024
+    A, B = 16, 16
     b = synthetic.slot_batch(d, V, A, B, 0.5, dtype=torch.bfloat16, device="cuda", seed=9)
     sl = alr.SlotLoss(A * B, d, V, B)
     assert alr.alr_device_status(clear=True) == alr.ALR_OK

@@ -446,23 +446,34 @@ def _all_outputs(Hd, Ht, W, B, mode, tok):
     return out
 
 
-@pytest.mark.parametrize("N", [272, 2048])
-def test_loss_kernel_forms_agree_bit_for_bit(N, monkeypatch):
-    """The multicast form of the fused kernels (clusters of two row blocks sharing each head
-    tile, ALR_LOSS_FORM=mcast) and the single-CTA default compute every unit identically, so all
-    outputs agree bit for bit: N = 272 has an odd number of row blocks (the last cluster's
-    second CTA has no rows), N = 2048 several raster groups of pairs."""
-    B, d, V = 16, 520, 3000
+@pytest.mark.parametrize("N,d,V", [(272, 520, 3000), (2048, 520, 3000), (272, 712, 13000),
+                                   (2048, 712, 3000)])
+def test_loss_kernel_forms_agree_bit_for_bit(N, d, V, monkeypatch):
+    """ALR_LOSS_FORM unset, single and mcast (clusters of two row blocks sharing each head tile,
+    where tiles have 256 columns) compute every unit identically and take the same workspaces, so
+    all outputs agree bit for bit.  N = 272 has an odd number of row blocks (the last cluster's
+    second CTA has no rows), N = 2048 several raster groups of pairs; d = 520 runs the forwards on
+    128-column tiles, d = 712 everything on 256 (13000 columns: enough tiles for three row
+    blocks)."""
+    B = 16
     Hd, Ht, W = _inputs(d, V, N // B, B, 0.5, torch.bfloat16, seed=N)
     tok = torch.randint(0, V, (N,), dtype=torch.int32, device="cuda")
-    monkeypatch.setenv("ALR_LOSS_FORM", "single")
-    single = _all_outputs(Hd, Ht, W, B, alr.ALR_MODE_ERASE_SOFT, tok)
-    monkeypatch.setenv("ALR_LOSS_FORM", "mcast")
-    assert alr.alr_kernel_forms()[1] == "mcast", alr.alr_cluster_forms_error()
-    mcast = _all_outputs(Hd, Ht, W, B, alr.ALR_MODE_ERASE_SOFT, tok)
-    for k in single:
-        a, b = single[k].cpu(), mcast[k].cpu()
-        if a.dtype.is_floating_point:
-            a, b = a.view(torch.int16 if a.element_size() == 2 else torch.int32), \
-                b.view(torch.int16 if b.element_size() == 2 else torch.int32)
-        assert torch.equal(a, b), k
+    params = alr.make_params(N, d, V, B, torch.bfloat16)
+    sizes, outs = [], []
+    for form in (None, "single", "mcast"):
+        monkeypatch.delenv("ALR_LOSS_FORM", raising=False)
+        if form is not None:
+            monkeypatch.setenv("ALR_LOSS_FORM", form)
+            assert alr.alr_kernel_forms()[1] == form, alr.alr_cluster_forms_error()
+        sizes.append([f(params) for f in (alr.alr_fwd_workspace_size, alr.alr_topk_fwd_workspace_size,
+                                          alr.alr_readout_workspace_size,
+                                          alr.alr_bwd_workspace_size)])
+        outs.append(_all_outputs(Hd, Ht, W, B, alr.ALR_MODE_ERASE_SOFT, tok))
+    assert sizes[0] == sizes[1] == sizes[2]
+    for other in outs[1:]:
+        for k in other:
+            a, b = outs[0][k].cpu(), other[k].cpu()
+            if a.dtype.is_floating_point:
+                a, b = a.view(torch.int16 if a.element_size() == 2 else torch.int32), \
+                    b.view(torch.int16 if b.element_size() == 2 else torch.int32)
+            assert torch.equal(a, b), k
