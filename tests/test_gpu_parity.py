@@ -477,3 +477,35 @@ def test_loss_kernel_forms_agree_bit_for_bit(N, d, V, monkeypatch):
                 a, b = a.view(torch.int16 if a.element_size() == 2 else torch.int32), \
                     b.view(torch.int16 if b.element_size() == 2 else torch.int32)
             assert torch.equal(a, b), k
+
+
+# (A, B, d, V): 256-column tiles (11 K blocks and more tiles than SMs, also counted over pairs of
+# row blocks) with edges everywhere: the last tile 8 or 248 columns wide, a K tail, a last row block
+# of 1 to 127 rows, an odd number of row blocks, anchors across row blocks
+@pytest.mark.parametrize("dtype,A,B,d,V", [(torch.bfloat16, 43, 3, 648, 39176),
+                                           (torch.bfloat16, 17, 15, 712, 39160),
+                                           (torch.bfloat16, 257, 1, 696, 19704),
+                                           (torch.float32, 24, 16, 328, 20248)])
+def test_wide_tiles_at_their_edges(dtype, A, B, d, V):
+    """The fused kernels' 256-column tiles at ragged sizes, which the smaller parity shapes run on
+    128 columns: forward (kept and not), both logit gradients, dH, dW, against the oracle."""
+    N = A * B
+    Hd, Ht, W = _inputs(d, V, A, B, 0.5, dtype, seed=N + d)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    mask = (torch.rand(N, generator=g, device="cuda") < 0.9).float()
+    mask[0] = 1.0
+    h, w, ht = P.np64(Hd), P.np64(W), P.np64(Ht)
+    r = orc.slot_loss_forward(h, ht, w, B, row_mask=P.np64(mask))
+    G_ref = orc.logit_grad(r["z_d"], r["z_t"], r["weight"], 1.0)
+    dH_ref, dW_ref = orc.slot_loss_backward(h, w, G_ref)
+    for keep in (False, True):
+        sl = alr.SlotLoss(N, d, V, B, dtype=dtype, keep_logits=keep)
+        sl.forward(Hd, Ht, W, row_mask=mask)
+        torch.cuda.synchronize()
+        P.compare_forward(P.fwd_to_numpy(sl), r)
+        dH, dW = torch.empty(N, d, device="cuda"), torch.zeros(d, V, device="cuda")
+        sl.backward(Hd, Ht, W, dH, dW)
+        torch.cuda.synchronize()
+        assert P.max_norm_rel(P.np64(dH), dH_ref) <= P.GRAD_RTOL
+        assert P.max_norm_rel(P.np64(dW), dW_ref) <= P.GRAD_RTOL
+    assert alr.alr_device_status() == alr.ALR_OK

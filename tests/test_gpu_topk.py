@@ -76,11 +76,14 @@ def compare_readout(g, r, prob_rtol=1e-3):
                                          (torch.bfloat16, (17, 16, 200, 1000)),
                                          (torch.float32, (64, 8, 256, 4096)),
                                          (torch.bfloat16, (64, 16, 2048, 32000)),
-                                         (torch.bfloat16, (125, 16, 1000, 60000))])
+                                         (torch.bfloat16, (125, 16, 1000, 60000)),
+                                         (torch.bfloat16, (43, 3, 648, 39176)),
+                                         (torch.bfloat16, (17, 15, 712, 39160))])
 def test_readout_matches_oracle(dtype, shape):
     """Row counts of 1.25, 2.1, 4, 8 and 15.6 row blocks of 128: the readout's units take two
-    row blocks each, so the last unit may hold a partial block or none; the last shape also
-    has a K tail (d = 1000) and a partial vocabulary tile (V = 60000)."""
+    row blocks each, so the last unit may hold a partial block or none; the fifth shape also
+    has a K tail (d = 1000) and a partial vocabulary tile (V = 60000).  The last two run on
+    256-column tiles with 129 and 255 rows and a last tile of 8 and 248 columns."""
     A, B, d, V = shape
     b = synthetic.slot_batch(d, V, A, B, 0.5, dtype=dtype, device="cuda", seed=A + V)
     N = A * B
