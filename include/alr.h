@@ -118,7 +118,8 @@ int alr_device_status(void* stream, int clear);
 
 /*
  * The kernel forms of this process (no device needed): the one ALR_GEMM_FORM names, or, with it
- * unset, the one the largest bf16 products take, and the loss kernels':
+ * unset, the one the largest bf16 products take (alr_gemm_form tells the form of a product of
+ * given sizes), and the loss kernels':
  *   *gemm: 0 single CTAs, 1 clusters of two sharing B tiles by TMA multicast, 2 CTA pairs
  *          (cta_group::2), 3 clusters of four with multicast;
  *   *loss: 0 single CTAs, 1 clusters of two sharing head tiles by TMA multicast.
@@ -135,8 +136,8 @@ const char* alr_cluster_forms_error(void);
 /*
  * Test hook for the failure-detection path (the paper has no counterpart).  With enable != 0,
  * the next launch, on any thread, of the fused loss kernel by a forward (alr_slot_loss_fwd,
- * alr_slot_loss_fwd_keep_logits, alr_slot_loss_fwd_noalloc) or of a tensor-core GEMM in the
- * single, multicast or split form (alr_gemm, and the dH / dW products of the backward entry points)
+ * alr_slot_loss_fwd_keep_logits, alr_slot_loss_fwd_noalloc) or of a tensor-core GEMM in any form
+ * (alr_gemm, and the dH / dW products of the backward entry points)
  * withholds the first pipeline stage of each CTA: nothing ever fills it, so the MMA issuer's
  * bounded wait runs out after about 1.5 s, every role of the CTA leaves its loop (copies in
  * flight are waited for, tensor memory is released) and the kernel records ALR_ERR_TIMEOUT in
@@ -561,6 +562,14 @@ int alr_erase_weights(const float* logp_x, const int32_t* corpus_tok, const int3
  */
 int alr_gemm(int32_t dtype, int32_t a_mn, int32_t b_mn, int32_t accumulate, const void* A,
              const void* B, float* C, int32_t M, int32_t Nc, int32_t K, void* stream);
+
+/*
+ * The form the next product of these sizes takes on the current device in this process (alr_gemm;
+ * the backward's dH_d is M = N, Nc = d, K = V and its dW is M = d, Nc = V, K = N):
+ *   *form:  as *gemm of alr_kernel_forms;
+ *   *split: CTAs that share each tile's K (1: not split; above 1, *form is 0).
+ */
+int alr_gemm_form(int32_t dtype, int32_t M, int32_t Nc, int32_t K, int32_t* form, int32_t* split);
 
 #ifdef __cplusplus
 }

@@ -111,6 +111,7 @@ SIGNATURES = {
                                    _c_p]),
     "alr_gemm": (_c_int, [_c_i32, _c_i32, _c_i32, _c_i32, _c_p, _c_p, _c_p, _c_i32, _c_i32,
                           _c_i32, _c_p]),
+    "alr_gemm_form": (_c_int, [_c_i32, _c_i32, _c_i32, _c_i32, _c_p, _c_p]),
 }
 
 
@@ -250,6 +251,13 @@ def alr_kernel_forms():
     g, l = ctypes.c_int32(), ctypes.c_int32()
     _check(lib().alr_kernel_forms(ctypes.byref(g), ctypes.byref(l)))
     return GEMM_FORMS[g.value], LOSS_FORMS[l.value]
+
+
+def alr_gemm_form(dtype, M, Nc, K):
+    """(form name, CTAs per tile's K) of the next product of these sizes on the current device."""
+    f, s = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().alr_gemm_form(dtype_code(dtype), M, Nc, K, ctypes.byref(f), ctypes.byref(s)))
+    return GEMM_FORMS[f.value], s.value
 
 
 def alr_cluster_forms_error() -> str:

@@ -46,7 +46,7 @@ struct Range {
 #define ALR_RANGE() const Range alr_nvtx_range_(__func__)
 
 // Test hook state: when set, the next launch of the fused loss kernel by a forward, or of the
-// plain GEMM (single or multicast form), withholds its first pipeline stage.
+// plain GEMM (any form), withholds its first pipeline stage.
 std::atomic<int> g_withhold_next{0};
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -405,8 +405,7 @@ GemmChoice choose_gemm(int dtype, int M, int Nc, int K, int sms) {
         best = GemmChoice{kGemmMcast, 1};
       }
     }
-    // (the withheld-stage hook is not in the pair form)
-    if (n_kb >= kPairMinBlocks && 2.0 * M * Nc * K <= kPairFlops && g_withhold_next.load() == 0) {
+    if (n_kb >= kPairMinBlocks && 2.0 * M * Nc * K <= kPairFlops) {
       const int pairs = cf->pair_gemm_max_pairs();
       const int64_t cost = pairs > 0 ? rounds(units, pairs) * n_kb * 27 + 150 : best_cost;
       if (cost < best_cost) {
@@ -492,6 +491,7 @@ int launch_gemm(const GemmChoice& c, int dt, bool a_mn, bool b_mn, bool acc, con
     alr::GemmArgs g = pair_gemm_plan(M, Nc, K, C, ldc, pairs);
     g.status = alr::device_status_ptr();
     if (g.status == nullptr) return fail(ALR_ERR_CUDA, "status word lookup failed");
+    g.withhold_first_stage = g_withhold_next.exchange(0);
     e = cf->launch_pair_gemm(a_mn, b_mn, acc, &ma, &mb, &g, s);
   } else if (form == kGemmMcast || form == kGemmMcast4) {
     const int cl = form == kGemmMcast4 ? 4 : 2;
@@ -1308,6 +1308,21 @@ int alr_erase_weights(const float* logp_x, const int32_t* corpus_tok, const int3
   cudaError_t e = alr::launch_erase_weights(logp_x, corpus_tok, argmax_t, row_mask, A, B, gamma,
                                             hard, weight, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "erase_weights launch");
+  return ALR_OK;
+}
+
+int alr_gemm_form(int32_t dtype, int32_t M, int32_t Nc, int32_t K, int32_t* form, int32_t* split) {
+  if (dtype != ALR_BF16 && dtype != ALR_F32) return fail(ALR_ERR_UNSUPPORTED, "dtype %d", dtype);
+  if (M < 1 || Nc < 1 || K < 1)
+    return fail(ALR_ERR_INVALID_ARG, "bad sizes M=%d Nc=%d K=%d", M, Nc, K);
+  if (form == nullptr || split == nullptr)
+    return fail(ALR_ERR_INVALID_ARG, "form and split must be non-NULL");
+  DevInfo info;
+  const int rc = require_sm103(&info);
+  if (rc != ALR_OK) return rc;
+  const GemmChoice c = choose_gemm(dtype, M, Nc, K, info.sms);
+  *form = int32_t(c.form);
+  *split = c.split;
   return ALR_OK;
 }
 

@@ -137,7 +137,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ------------------------------------------------------------- TMA producer ---
     if (lane == 0) {
-      int stage = 0;
+      // test hook: both CTAs start filling at stage 1 (as in plain_gemm_kernel.cuh), so the even
+      // CTA's issuer runs out on stage 0 and the odd CTA on the products that never come
+      int stage = args.withhold_first_stage ? 1 : 0;
       uint32_t phase = 0, armed = 0, armed_par = 0;
       bool ok = true;
       for (int t = pair; ok && t < args.n_tiles; t += n_pairs) {

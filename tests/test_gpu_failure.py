@@ -81,12 +81,16 @@ def test_withheld_gemm_stage_times_out_and_context_survives(form, monkeypatch):
 
 
 @pytest.mark.parametrize("accumulate", [False, True])
-@pytest.mark.parametrize("shape", [(128, 64, 8200), (304, 512, 4000), (2200, 2056, 520),
-                                   (104, 8200, 72)])
-def test_withheld_stage_of_the_chosen_form_leaves_c_alone(shape, accumulate, monkeypatch):
-    """The forms products take by size: K split over clusters of 16 and of 5 CTAs, multicast
-    clusters, single CTAs.  No tile's sum is complete when the waits run out, so none is stored
-    or added: C keeps every bit.  The next product is correct."""
+@pytest.mark.parametrize("shape,chosen", [((128, 64, 8200), ("single", 10)),
+                                          ((304, 512, 4000), ("single", 7)),
+                                          ((2200, 2056, 2056), ("pair", 1)),
+                                          ((2200, 2056, 520), ("mcast", 1)),
+                                          ((104, 8200, 72), ("single", 1))])
+def test_withheld_stage_of_the_chosen_form_leaves_c_alone(shape, chosen, accumulate, monkeypatch):
+    """The forms products take by size, whether or not the hook is armed: K split over clusters of
+    10 and of 7 CTAs, CTA pairs, multicast clusters, single CTAs.  No tile's sum is complete when
+    the waits run out, so none is stored or added: C keeps every bit.  The next product is
+    correct."""
     monkeypatch.delenv("ALR_GEMM_FORM", raising=False)
     M, Nc, K = shape
     g = torch.Generator(device="cuda").manual_seed(5)
@@ -96,6 +100,8 @@ def test_withheld_stage_of_the_chosen_form_leaves_c_alone(shape, accumulate, mon
     before = C.clone()
     assert alr.alr_device_status(clear=True) == alr.ALR_OK
     alr.alr_debug_withhold_next_stage(True)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert alr.alr_gemm_form(torch.bfloat16, M, Nc, K) == chosen
     t0 = time.monotonic()
     alr.alr_gemm(A, Bm, C, M, Nc, K, accumulate=accumulate)
     rc = alr.alr_device_status(clear=True)

@@ -66,19 +66,31 @@ def test_gemm_layouts(form, dtype, a_mn, b_mn, shape, monkeypatch):
     assert alr.alr_device_status() == alr.ALR_OK
 
 
+# (M, Nc, K) -> the (form, CTAs per tile's K) of bf16 and of tf32 products on 152 SMs
+CHOSEN = {(128, 64, 8200): (("single", 10), ("single", 12)),
+          (16, 2048, 4104): (("single", 6), ("single", 10)),
+          (304, 512, 4000): (("single", 7), ("single", 8)),
+          (136, 1000, 30008): (("single", 12), ("single", 12)),
+          (2000, 264, 2000): (("single", 4), ("single", 4)),
+          (8, 8, 1024): (("mcast", 1), ("single", 4)),
+          (2200, 2056, 2056): (("pair", 1), ("single", 1)),
+          (2200, 2056, 520): (("mcast", 1), ("single", 1)),
+          (104, 8200, 72): (("single", 1), ("single", 1))}
+
+
 @pytest.mark.parametrize("dtype,a_mn,b_mn", [(torch.float32, False, False)] + [
     (torch.bfloat16, a, b) for a, b in itertools.product([False, True], repeat=2)])
-@pytest.mark.parametrize("shape", [(128, 64, 8200), (16, 2048, 4104), (304, 512, 4000),
-                                   (136, 1000, 30008), (2000, 264, 2000), (8, 8, 1024),
-                                   (2200, 2056, 2056), (2200, 2056, 520), (104, 8200, 72)])
+@pytest.mark.parametrize("shape", list(CHOSEN))
 def test_gemm_form_chosen_by_size(dtype, a_mn, b_mn, shape, monkeypatch):
     """The form each size takes when none is named.  Few tiles and a long K split each tile's K
-    over a cluster (1 to 32 tiles: clusters of 16 down to 4 CTAs, K shares of unequal length, a
+    over a cluster (1 to 32 tiles: clusters of 12 down to 4 CTAs, K shares of unequal length, a
     K tail, partial tiles); 2200 x 2056 takes CTA pairs at K = 2056 and multicast clusters at
     520 (bf16); one row block and K = 72 single CTAs.  Against fp64, bit-identical from run to
     run, and adding to C exactly what the overwriting form writes."""
     monkeypatch.delenv("ALR_GEMM_FORM", raising=False)
     M, Nc, K = shape
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert alr.alr_gemm_form(dtype, M, Nc, K) == CHOSEN[shape][dtype == torch.float32]
     A_st, B_st, ref = _operands(M, Nc, K, dtype, a_mn, b_mn, seed=M + Nc + K)
     C = torch.full((M, Nc), float("nan"), device="cuda")
     C2 = C.clone()
