@@ -254,6 +254,7 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   P.d = p->d;
   P.V = p->V;
   P.B = p->B;
+  P.products = two_rows ? 1 : 2;
   // row blocks; row-block pairs for the two-row modes and for the multicast form (which
   // places sms / 2 clusters).  Forward: the splits of forward_splits (the same for both
   // forms), in raster groups of up to two rounds of the grid at its base split (16 row blocks).

@@ -22,7 +22,8 @@ struct LossPlan {
   int group_rows;  // row blocks per group
   int n_units;     // n_rb * n_vs
   int grid;        // persistent CTAs
-  double flops() const { return 4.0 * N * d * V; }   // two products of a tile
+  int products;    // head products per row: two, or one in two-row modes
+  double flops() const { return 2.0 * products * N * d * V; }
   int mc;          // 1: clusters of two CTAs share each head tile by TMA multicast (bf16,
                    // 256-column tiles); n_rb and group_rows then count row-block pairs and
                    // the grid is sized from the clusters that fit
