@@ -254,6 +254,7 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   P.d = p->d;
   P.V = p->V;
   P.B = p->B;
+  P.sms = sms;
   P.products = two_rows ? 1 : 2;
   // row blocks; row-block pairs for the two-row modes and for the multicast form (which
   // places sms / 2 clusters).  Forward: the splits of forward_splits (the same for both
@@ -926,7 +927,7 @@ int alr_logit_grad_from_logits(const alr_params* p, const void* Zd, const void* 
   DevInfo info;
   if ((rc = require_sm103(&info)) != ALR_OK) return rc;
   cudaError_t e = alr::launch_logits_grad(p->dtype, Zd, Zt, Zd_ref, Zt_ref, lse_d, lse_t, weight,
-                                          weight_sum, p->lambda, int(p->N), p->V, G,
+                                          weight_sum, p->lambda, int(p->N), p->V, G, info.sms,
                                           static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "logit-gradient launch");
   return ALR_OK;
@@ -1108,7 +1109,7 @@ int alr_topk_logit_grad_from_logits(const alr_params* p, const void* Zd, const u
   if ((rc = require_sm103(&info)) != ALR_OK) return rc;
   cudaError_t e = alr::launch_topk_logits_grad(p->dtype, Zd, Zd_ref, top_idx, top_prob, tail,
                                                tail_q, lse_d, weight, weight_sum, p->lambda,
-                                               int(p->N), p->V, G,
+                                               int(p->N), p->V, G, info.sms,
                                                static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "top-k logit-gradient launch");
   return ALR_OK;

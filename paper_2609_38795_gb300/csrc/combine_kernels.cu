@@ -606,21 +606,20 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
 }
 
 // ------------------------------------------------------------------ launch shape ---
-// Enough 32-row blocks to fill the chip twice over: 32 rows and 8 warps per block, whose record
+// Enough 32-row blocks to fill the device twice over: 32 rows and 8 warps per block, whose record
 // reads are whole 128-byte lines.  Fewer: the smallest of 8, 16 or 32 rows that holds a whole
 // anchor, with 16 warps over the records (32 warps leave a thread 64 registers
 // and spill).
-constexpr int kManyBlocks = 304;
 constexpr int kReadoutFewRows = 1024;
 
 struct MergeShape {
   int rows, warps, rows_per_block, blocks;
 };
 
-MergeShape merge_shape(int N, int B) {
+MergeShape merge_shape(int N, int B, int sms) {
   const int per32 = 32 / B * B;
   MergeShape m{32, 8, per32, (N + per32 - 1) / per32};
-  if (m.blocks >= kManyBlocks) return m;
+  if (m.blocks >= 2 * sms) return m;
   m.rows = B <= 8 ? 8 : B <= 16 ? 16 : 32;
   m.warps = 16;
   m.rows_per_block = m.rows / B * B;
@@ -636,7 +635,7 @@ cudaError_t launch_combine(const LossPlan& plan, const float* part, int mode, fl
                            int32_t* argmax_t, float* gap_d, float* gap_t, float* logp_x,
                            float* weight, double* block_part, unsigned* ticket, float lam,
                            float* loss_total, float* weight_sum, float* wl_sum, cudaStream_t s) {
-  const MergeShape m = merge_shape(plan.N, plan.B);
+  const MergeShape m = merge_shape(plan.N, plan.B, plan.sms);
   const FullOut o{loss_row, ent_row, lse_d, lse_t, argmax_d, argmax_t, gap_d, gap_t, logp_x, weight};
   const BatchOut b{block_part, ticket, lam, loss_total, weight_sum, wl_sum};
   auto kern = m.warps == 8   ? combine_kernel<32, 8>
@@ -654,7 +653,7 @@ cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool
   // a merge of two top-8 lists costs several times a plain record's, so with more rows fewer lanes
   // share one: 64, 16 from 1024 rows, 8 (readout with 16 instead of 64: 1920 x 64 x 151936 243 ->
   // 229 us, 9000 x 64 x 20000 231 -> 191; 768 x 64 x 151936 130 -> 131)
-  MergeShape m = merge_shape(plan.N, 1);
+  MergeShape m = merge_shape(plan.N, 1, plan.sms);
   auto kern = readout_combine_kernel<32, 8>;
   if (m.rows < 32) {
     const bool few = plan.N < kReadoutFewRows;
@@ -672,7 +671,7 @@ cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const f
                                 double* block_part, unsigned* ticket, float lam,
                                 float* loss_total, float* weight_sum, float* wl_sum,
                                 cudaStream_t s) {
-  const MergeShape m = merge_shape(plan.N, plan.B);
+  const MergeShape m = merge_shape(plan.N, plan.B, plan.sms);
   const TopkOut o{loss_row, lse_d, tail_q, argmax_d, gap_d, weight};
   const BatchOut b{block_part, ticket, lam, loss_total, weight_sum, wl_sum};
   auto kern = m.warps == 8   ? topk_combine_kernel<32, 8>

@@ -25,13 +25,13 @@ constexpr int kGradRows = 32;              // most rows of a block
 constexpr int kGradCols = 2048;
 constexpr int kGradThreads = kGradCols / 8;
 
-// Rows per block: 32 where that gives eight blocks to each of 152 SMs, else halved down to one
+// Rows per block: 32 where that gives eight blocks to each SM, else halved down to one
 // pass of kLogitsUnroll rows, since the passes of a block follow one another, each a memory
 // round trip (192 rows of V = 1400: 6 blocks of 8 passes took 11.9 us, now 3.7).
-inline int grad_rows(int N, int V) {
+inline int grad_rows(int N, int V, int sms) {
   const long long cols = (V + kGradCols - 1) / kGradCols;
   int rows = kGradRows;
-  while (rows > kLogitsUnroll && (N + rows - 1) / rows * cols < 8 * 152) rows /= 2;
+  while (rows > kLogitsUnroll && (N + rows - 1) / rows * cols < 8 * sms) rows /= 2;
   return rows;
 }
 
@@ -250,8 +250,8 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
                                     const int32_t* top_idx, const float* top_prob,
                                     const float* tail, const float* tail_q, const float* lse_d,
                                     const float* weight, const float* weight_sum, float lam, int N,
-                                    int V, void* G, cudaStream_t s) {
-  const int rows = grad_rows(N, V);
+                                    int V, void* G, int sms, cudaStream_t s) {
+  const int rows = grad_rows(N, V, sms);
   const double size = 2000.0 * N * V;   // as long as this many flop of a product
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)
@@ -268,8 +268,8 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
 cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const uint16_t* zd_ref,
                                const uint16_t* zt_ref, const float* lse_d, const float* lse_t,
                                const float* weight, const float* weight_sum, float lam, int N,
-                               int V, void* G, cudaStream_t s) {
-  const int rows = grad_rows(N, V);
+                               int V, void* G, int sms, cudaStream_t s) {
+  const int rows = grad_rows(N, V, sms);
   const double size = 2000.0 * N * V;   // as long as this many flop of a product
   const dim3 grid(unsigned((N + rows - 1) / rows), unsigned((V + kGradCols - 1) / kGradCols));
   if (dtype == 0)

@@ -22,6 +22,7 @@ struct LossPlan {
   int group_rows;  // row blocks per group
   int n_units;     // n_rb * n_vs
   int grid;        // persistent CTAs
+  int sms;         // of the device
   int products;    // head products per row: two, or one in two-row modes
   double flops() const { return 2.0 * products * N * d * V; }
   int mc;          // 1: clusters of two CTAs share each head tile by TMA multicast (bf16,
@@ -178,7 +179,7 @@ cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const f
 cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const uint16_t* zd_ref,
                                const uint16_t* zt_ref, const float* lse_d, const float* lse_t,
                                const float* weight, const float* weight_sum, float lam, int N,
-                               int V, void* G, cudaStream_t s);
+                               int V, void* G, int sms, cudaStream_t s);
 // Gradient of the top-k + tail soft CE from kept z_d (as in launch_logits_grad):
 // G = c_r beta_r q outside the row's label tokens, c_r (q - prob_i) at label token i, with
 // q = exp(z_d - lse_d), c_r = lambda omega_r / sum omega, beta_r = 1 - tail_r / tail_q_r (1 when
@@ -188,7 +189,7 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
                                     const float* top_prob, const float* tail, const float* tail_q,
                                     const float* lse_d, const float* weight,
                                     const float* weight_sum, float lam, int N, int V, void* G,
-                                    cudaStream_t s);
+                                    int sms, cudaStream_t s);
 cudaError_t launch_accept_len(const int32_t* am_d, const int32_t* am_t, const float* active,
                               int A, int B, int32_t* acc, int64_t* hist, cudaStream_t s);
 cudaError_t launch_erase_weights(const float* logp_x, const int32_t* corpus_tok,

@@ -290,3 +290,14 @@ def test_kernels_read_no_memory_through_the_read_only_path():
                 code = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
             code = "\n".join(line.split("//")[0] for line in code.splitlines())
             assert not pat.search(code), (f, pat.search(code).group(0))
+
+
+def test_kernel_launches_take_the_sm_count_from_the_device():
+    """Rules that weigh a problem against the device read its SM count from the plan, which has it
+    from the device: no source holds the count of one chip (152, or 304 for twice over)."""
+    for d in (build_lib.CSRC, build_lib.CSRC_CLUSTER):
+        for f in sorted(os.listdir(d)):
+            with open(os.path.join(d, f)) as fh:
+                code = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
+            code = "\n".join(line.split("//")[0] for line in code.splitlines())
+            assert not re.search(r"\b(152|304)\b", code), f
