@@ -445,9 +445,8 @@ struct FullOut {
 
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
-    combine_kernel(LossPlan P, const float* part, int rows_per_block, int mode,
-                   float gamma, const float* row_mask,
-                   const int32_t* corpus_tok, FullOut o, BatchOut bo) {
+    combine_kernel(LossPlan P, const float* part, int rows_per_block, int mode, float gamma,
+                   const float* row_mask, const int32_t* corpus_tok, FullOut o, BatchOut bo) {
   __shared__ MergeSmem<FullState, kRows, kWarps> sm;
   __shared__ float s_loss[kRows], s_logp[kRows];
   const int row0 = blockIdx.x * rows_per_block;
@@ -509,11 +508,9 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
 // gap, and log p at the corpus token.  Rows are independent.
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, 1)
-    readout_combine_kernel(LossPlan P, const float* part, int has_corpus,
-                           int32_t* top_idx, float* top_prob,
-                           float* tail, float* lse_t,
-                           int32_t* argmax_t, float* gap_t,
-                           float* logp_x) {
+    readout_combine_kernel(LossPlan P, const float* part, int has_corpus, int32_t* top_idx,
+                           float* top_prob, float* tail, float* lse_t, int32_t* argmax_t,
+                           float* gap_t, float* logp_x) {
   static_assert(kRows * kTopK <= 32 * kWarps, "one thread per label");
   __shared__ MergeSmem<ReadoutState, kRows, kWarps> sm;
   __shared__ double s_e[kTopK][kRows];
@@ -568,9 +565,8 @@ struct TopkOut {
 
 template <int kRows, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
-    topk_combine_kernel(LossPlan P, const float* part, int rows_per_block,
-                        const float* top_prob, const float* tail,
-                        const float* row_mask, const float* weight_in,
+    topk_combine_kernel(LossPlan P, const float* part, int rows_per_block, const float* top_prob,
+                        const float* tail, const float* row_mask, const float* weight_in,
                         float gamma, TopkOut o, BatchOut bo) {
   __shared__ MergeSmem<TopkState, kRows, kWarps> sm;
   const int row0 = blockIdx.x * rows_per_block;
@@ -608,8 +604,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
 // ------------------------------------------------------------------ launch shape ---
 // Enough 32-row blocks to fill the device twice over: 32 rows and 8 warps per block, whose record
 // reads are whole 128-byte lines.  Fewer: the smallest of 8, 16 or 32 rows that holds a whole
-// anchor, with 16 warps over the records (32 warps leave a thread 64 registers
-// and spill).
+// anchor, with 16 warps over the records (32 warps leave a thread 64 registers and spill).
 constexpr int kReadoutFewRows = 1024;
 
 struct MergeShape {
@@ -636,14 +631,15 @@ cudaError_t launch_combine(const LossPlan& plan, const float* part, int mode, fl
                            float* weight, double* block_part, unsigned* ticket, float lam,
                            float* loss_total, float* weight_sum, float* wl_sum, cudaStream_t s) {
   const MergeShape m = merge_shape(plan.N, plan.B, plan.sms);
-  const FullOut o{loss_row, ent_row, lse_d, lse_t, argmax_d, argmax_t, gap_d, gap_t, logp_x, weight};
+  const FullOut o{loss_row, ent_row, lse_d,  lse_t,  argmax_d,
+                  argmax_t, gap_d,   gap_t,  logp_x, weight};
   const BatchOut b{block_part, ticket, lam, loss_total, weight_sum, wl_sum};
   auto kern = m.warps == 8   ? combine_kernel<32, 8>
               : m.rows == 8  ? combine_kernel<8, 16>
               : m.rows == 16 ? combine_kernel<16, 16>
                              : combine_kernel<32, 16>;
-  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, mode, gamma, row_mask,
-                                       corpus_tok, o, b);
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, mode, gamma,
+                    row_mask, corpus_tok, o, b);
 }
 
 cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool has_corpus,
@@ -678,8 +674,8 @@ cudaError_t launch_topk_combine(const LossPlan& plan, const float* part, const f
               : m.rows == 8  ? topk_combine_kernel<8, 16>
               : m.rows == 16 ? topk_combine_kernel<16, 16>
                              : topk_combine_kernel<32, 16>;
-  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, top_prob, tail, row_mask,
-                                       weight_in, gamma, o, b);
+  return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, m.rows_per_block, top_prob,
+                    tail, row_mask, weight_in, gamma, o, b);
 }
 
 }  // namespace alr

@@ -64,7 +64,8 @@ ALR_DEV void put_half_row(const uint32_t (&r)[32], int h, uint8_t* stage, int la
   for (int j = 0; j < 8; ++j) s[lane * 16 + 8 * h + (j ^ (lane & 7))] = vec4(r, j);
 }
 
-// Write (kAcc: add) rows 16 h .. 16 h + 15 of the staged block; (m0, n0): the piece's first element.
+// Write (kAcc: add) rows 16 h .. 16 h + 15 of the staged block; (m0, n0): the piece's first
+// element.
 template <bool kAcc>
 ALR_DEV void store_piece(const CPiece& old, const GemmArgs& a, int m0, int n0, int h,
                          const uint8_t* stage, int lane) {
@@ -171,7 +172,8 @@ ALR_DEV void reduce_split(const GemmArgs& a, int m0, int n0, const uint8_t* tile
       const uint32_t base = cluster_smem_addr(tile + b * kSplitBlockBytes, uint32_t(p));
       float4 v[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = ld_cluster_v4(base + 16u * uint32_t(block_vector(i, lane)));
+      for (int i = 0; i < 8; ++i)
+        v[i] = ld_cluster_v4(base + 16u * uint32_t(block_vector(i, lane)));
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         if (p == 0) {

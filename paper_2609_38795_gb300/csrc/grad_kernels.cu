@@ -110,10 +110,9 @@ __device__ __forceinline__ float row_factor(const float* weight, const float* we
 
 template <typename Z, typename Gt>
 __global__ void __launch_bounds__(kGradThreads) logits_grad_kernel(
-    const Z* zd, const Z* zt, const uint16_t* zd_ref,
-    const uint16_t* zt_ref, const float* lse_d,
-    const float* lse_t, const float* weight,
-    const float* weight_sum, float lam, int N, int V, int rows, Gt* G) {
+    const Z* zd, const Z* zt, const uint16_t* zd_ref, const uint16_t* zt_ref, const float* lse_d,
+    const float* lse_t, const float* weight, const float* weight_sum, float lam, int N, int V,
+    int rows, Gt* G) {
   __shared__ float s_c[kGradRows], s_ad[kGradRows], s_at[kGradRows];
   pdl_wait_and_release();
   const int r0 = blockIdx.x * rows, c0 = blockIdx.y * kGradCols;
@@ -169,11 +168,9 @@ __global__ void __launch_bounds__(kGradThreads) logits_grad_kernel(
 // buffer).  The label tokens of a row are distinct.
 template <typename Z, typename Gt>
 __global__ void __launch_bounds__(kGradThreads) topk_logits_grad_kernel(
-    const Z* zd, const uint16_t* zd_ref, const int32_t* top_idx,
-    const float* top_prob, const float* tail,
-    const float* tail_q, const float* lse_d,
-    const float* weight, const float* weight_sum, float lam, int N,
-    int V, int rows, Gt* G) {
+    const Z* zd, const uint16_t* zd_ref, const int32_t* top_idx, const float* top_prob,
+    const float* tail, const float* tail_q, const float* lse_d, const float* weight,
+    const float* weight_sum, float lam, int N, int V, int rows, Gt* G) {
   static_assert(kGradRows * kTopK <= kGradThreads, "one thread per label of the block's rows");
   __shared__ float s_c[kGradRows], s_cb[kGradRows], s_ad[kGradRows];
   __shared__ float lab_g[kGradRows * kTopK];
@@ -260,9 +257,9 @@ cudaError_t launch_topk_logits_grad(int dtype, const void* zd, const uint16_t* z
         static_cast<const __half*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
         weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
   return launch_pdl_sized(
-        size, topk_logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
-        static_cast<const float*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
-        weight_sum, lam, N, V, rows, static_cast<float*>(G));
+      size, topk_logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+      static_cast<const float*>(zd), zd_ref, top_idx, top_prob, tail, tail_q, lse_d, weight,
+      weight_sum, lam, N, V, rows, static_cast<float*>(G));
 }
 
 cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const uint16_t* zd_ref,
@@ -278,9 +275,9 @@ cudaError_t launch_logits_grad(int dtype, const void* zd, const void* zt, const 
         static_cast<const __half*>(zd), static_cast<const __half*>(zt), zd_ref, zt_ref, lse_d,
         lse_t, weight, weight_sum, lam, N, V, rows, static_cast<__nv_bfloat16*>(G));
   return launch_pdl_sized(
-        size, logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
-        static_cast<const float*>(zd), static_cast<const float*>(zt), zd_ref, zt_ref, lse_d,
-        lse_t, weight, weight_sum, lam, N, V, rows, static_cast<float*>(G));
+      size, logits_grad_kernel<float, float>, grid, kGradThreads, 0, s,
+      static_cast<const float*>(zd), static_cast<const float*>(zt), zd_ref, zt_ref, lse_d,
+      lse_t, weight, weight_sum, lam, N, V, rows, static_cast<float*>(G));
 }
 
 }  // namespace alr

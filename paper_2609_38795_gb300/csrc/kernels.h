@@ -18,7 +18,8 @@ struct LossPlan {
   int n_rb;        // ceil(N / 128)
   int n_vt;        // ceil(V / bn)
   int n_vs;        // vocabulary splits
-  int n_parts;     // partial records per row: one per split and column group (4, or 2 in two-row modes)
+  int n_parts;     // partial records per row: one per split and column group (4, or 2 in
+                   // two-row modes)
   int group_rows;  // row blocks per group
   int n_units;     // n_rb * n_vs
   int grid;        // persistent CTAs
@@ -219,8 +220,8 @@ cudaError_t launch_transpose32(const float* in, float* out, int R, int C, int ld
                                cudaStream_t s);
 
 // The same for a [R, Ca] and b [R, Cb] in one launch (both outputs with ld_out).
-cudaError_t launch_transpose32_pair(const float* a, float* a_out, int Ca, const float* b, float* b_out,
-                                    int Cb, int R, int ld_out, cudaStream_t s);
+cudaError_t launch_transpose32_pair(const float* a, float* a_out, int Ca, const float* b,
+                                    float* b_out, int Cb, int R, int ld_out, cudaStream_t s);
 
 // Record `msg` as this host thread's alr_last_error() text and return `code` (api.cu).
 int set_last_error(int code, const char* msg);

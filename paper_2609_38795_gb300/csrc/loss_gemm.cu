@@ -17,7 +17,8 @@ cudaError_t launch_impl(const CUtensorMap& a0, const CUtensorMap& a1, const CUte
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kSmem));
   if (e != cudaSuccess) return e;
-  return launch_pdl_sized(args.plan.flops(), kern, args.plan.grid, S::kThreads, S::kSmem, s, a0, a1, w, g, g2, args);
+  return launch_pdl_sized(args.plan.flops(), kern, args.plan.grid, S::kThreads, S::kSmem, s, a0, a1,
+                          w, g, g2, args);
 }
 
 template <typename Elem, int kMode>

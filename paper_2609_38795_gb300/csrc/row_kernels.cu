@@ -73,8 +73,7 @@ __device__ __forceinline__ float gate_for_lane(bool active, int lane, bool hard,
 
 // Eq. 1 from sums that the caller reduced over the shards of a batch: L = lambda * wl / ws,
 // 0 when ws = 0 (no supervised slot anywhere in the batch).
-__global__ void loss_from_sums_kernel(const float* wl_sum,
-                                      const float* weight_sum, float lam,
+__global__ void loss_from_sums_kernel(const float* wl_sum, const float* weight_sum, float lam,
                                       float* loss_total) {
   pdl_wait_and_release();
   const double ws = *weight_sum;
@@ -84,8 +83,8 @@ __global__ void loss_from_sums_kernel(const float* wl_sum,
 // ------------------------------------------------------------- accepted length ---
 // One warp per anchor: the count of leading slots whose greedy drafter token equals the
 // greedy target token (and whose row is active).
-ALR_DEV int accepted_slots(const int32_t* am_d, const int32_t* am_t,
-                           const float* active_w, int a, int B, int lane) {
+ALR_DEV int accepted_slots(const int32_t* am_d, const int32_t* am_t, const float* active_w, int a,
+                           int B, int lane) {
   bool ok = false;
   if (lane < B) {
     const int r = a * B + lane;
@@ -96,11 +95,9 @@ ALR_DEV int accepted_slots(const int32_t* am_d, const int32_t* am_t,
   return bal == 0xffffffffu ? 32 : __ffs(~bal) - 1;
 }
 
-__global__ void __launch_bounds__(256) accept_len_kernel(const int32_t* am_d,
-                                                         const int32_t* am_t,
-                                                         const float* active_w,
-                                                         int A, int B, int32_t* acc,
-                                                         unsigned long long* hist) {
+__global__ void __launch_bounds__(256)
+    accept_len_kernel(const int32_t* am_d, const int32_t* am_t, const float* active_w, int A,
+                      int B, int32_t* acc, unsigned long long* hist) {
   pdl_wait_and_release();
   const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -117,10 +114,9 @@ __global__ void __launch_bounds__(256) accept_len_kernel(const int32_t* am_d,
 // the gap between them).  Past kAcceptOneBlock anchors the rounds of one block cost more than that.
 constexpr int kAcceptOneBlock = 256;
 
-__global__ void __launch_bounds__(1024) accept_len_one_block_kernel(
-    const int32_t* am_d, const int32_t* am_t,
-    const float* active_w, int A, int B, int32_t* acc,
-    unsigned long long* hist) {
+__global__ void __launch_bounds__(1024)
+    accept_len_one_block_kernel(const int32_t* am_d, const int32_t* am_t, const float* active_w,
+                                int A, int B, int32_t* acc, unsigned long long* hist) {
   __shared__ int count[33];
   pdl_wait_and_release();
   const int lane = threadIdx.x & 31, n_warps = blockDim.x / 32;
@@ -142,10 +138,10 @@ __global__ void __launch_bounds__(1024) accept_len_one_block_kernel(
 }
 
 // ---------------------------------------------------------- erase weights ---
-__global__ void __launch_bounds__(256) erase_weights_kernel(
-    const float* logp_x, const int32_t* corpus_tok,
-    const int32_t* argmax_t, const float* row_mask, int A, int B,
-    float gamma, int hard, float* weight) {
+__global__ void __launch_bounds__(256)
+    erase_weights_kernel(const float* logp_x, const int32_t* corpus_tok, const int32_t* argmax_t,
+                         const float* row_mask, int A, int B, float gamma, int hard,
+                         float* weight) {
   pdl_wait_and_release();
   const int a = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -171,12 +167,11 @@ __global__ void __launch_bounds__(256) erase_weights_kernel(
 // first ceil(m/2) primary, the next floor(m/2) secondary (Sec. 3.2); secondary i sits in
 // primary i's rollout at offset j.  Emits the label-row gather (seq, pos, valid_len) over
 // the primary label buffer [S * P, K, d], the anchor token and the rollout context length.
-__global__ void __launch_bounds__(256) ira_blocks_kernel(
-    int S, int K, int max_blocks, const int32_t* valid_anchors,
-    const int32_t* rollout_len, const int32_t* offsets,
-    const int32_t* rollout_tok, const int32_t* corpus_anchor_tok,
-    int32_t* seq, int32_t* pos, int32_t* vlen,
-    int32_t* ctx_len, int32_t* anchor_tok) {
+__global__ void __launch_bounds__(256)
+    ira_blocks_kernel(int S, int K, int max_blocks, const int32_t* valid_anchors,
+                      const int32_t* rollout_len, const int32_t* offsets,
+                      const int32_t* rollout_tok, const int32_t* corpus_anchor_tok, int32_t* seq,
+                      int32_t* pos, int32_t* vlen, int32_t* ctx_len, int32_t* anchor_tok) {
   pdl_wait_and_release();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)S * max_blocks) return;
@@ -232,9 +227,8 @@ using Pair = unsigned long long;           // key << 32 | position
 constexpr Pair kNoPair = ~0ull;            // an invalid position (no valid one: position < 2^14)
 
 __global__ void __launch_bounds__(kDrawThreads)
-    ira_draw_kernel(int L, int K, int max_blocks, const uint8_t* anchor_ok,
-                    const uint32_t* keys, const uint32_t* offset_u,
-                    int32_t* n_valid, int32_t* anchor_pos,
+    ira_draw_kernel(int L, int K, int max_blocks, const uint8_t* anchor_ok, const uint32_t* keys,
+                    const uint32_t* offset_u, int32_t* n_valid, int32_t* anchor_pos,
                     int32_t* offsets) {
   extern __shared__ Pair cand[];           // [L]
   __shared__ int hist[256], s_valid, s_cand, s_digit, s_below, s_in;
@@ -271,7 +265,8 @@ __global__ void __launch_bounds__(kDrawThreads)
     for (int digit = 0; digit < 6; ++digit) {
       // the key's four digits, then the position's two (positions are below 2^14)
       shift = digit < 4 ? 56 - 8 * digit : 8 * (5 - digit);
-      const Pair above = digit == 0 ? 0 : digit == 4 ? prefix << 16 : prefix;   // bits over shift + 8
+      // the bits over shift + 8
+      const Pair above = digit == 0 ? 0 : digit == 4 ? prefix << 16 : prefix;
 #pragma unroll
       for (int j = 0; j < kDrawPer; ++j) {
         if (c[j] == kNoPair) continue;
@@ -415,9 +410,9 @@ cudaError_t launch_ira_blocks(int S, int K, int max_blocks, const int32_t* valid
                               int32_t* seq, int32_t* pos, int32_t* vlen, int32_t* ctx_len,
                               int32_t* anchor_tok, cudaStream_t s) {
   const long long n = (long long)S * max_blocks;
-  return launch_pdl(
-      ira_blocks_kernel, unsigned((n + 255) / 256), 256, 0, s, S, K, max_blocks, valid_anchors, rollout_len, offsets, rollout_tok, corpus_anchor_tok, seq,
-      pos, vlen, ctx_len, anchor_tok);
+  return launch_pdl(ira_blocks_kernel, unsigned((n + 255) / 256), 256, 0, s, S, K, max_blocks,
+                    valid_anchors, rollout_len, offsets, rollout_tok, corpus_anchor_tok, seq, pos,
+                    vlen, ctx_len, anchor_tok);
 }
 
 cudaError_t launch_ira_draw(int S, int L, int K, int max_blocks, const uint8_t* anchor_ok,
@@ -428,8 +423,8 @@ cudaError_t launch_ira_draw(int S, int L, int K, int max_blocks, const uint8_t* 
                                        int(smem));
   if (e != cudaSuccess) return e;
   const int threads = L <= 256 ? 256 : L <= 512 ? 512 : kDrawThreads;
-  return launch_pdl(ira_draw_kernel, S, threads, smem, s, L, K, max_blocks, anchor_ok, keys, offset_u, n_valid,
-                                        anchor_pos, offsets);
+  return launch_pdl(ira_draw_kernel, S, threads, smem, s, L, K, max_blocks, anchor_ok, keys,
+                    offset_u, n_valid, anchor_pos, offsets);
 }
 
 cudaError_t launch_ira_context(const void* store, int C, int F, int elem_bytes, int S, int K,
@@ -452,8 +447,8 @@ cudaError_t launch_transpose32(const float* in, float* out, int R, int C, int ld
                     (const float*)nullptr, (float*)nullptr, 0);
 }
 
-cudaError_t launch_transpose32_pair(const float* a, float* a_out, int Ca, const float* b, float* b_out,
-                                    int Cb, int R, int ld_out, cudaStream_t s) {
+cudaError_t launch_transpose32_pair(const float* a, float* a_out, int Ca, const float* b,
+                                    float* b_out, int Cb, int R, int ld_out, cudaStream_t s) {
   const unsigned tiles = (Ca + 31) / 32;
   dim3 grid(tiles + (Cb + 31) / 32, (R + 31) / 32);
   return launch_pdl(transpose32_kernel, grid, dim3(32, 8), 0, s, a, a_out, R, Ca, ld_out, tiles, b,
@@ -495,8 +490,8 @@ cudaError_t launch_accept_len(const int32_t* am_d, const int32_t* am_t, const fl
 cudaError_t launch_erase_weights(const float* logp_x, const int32_t* corpus_tok,
                                  const int32_t* argmax_t, const float* row_mask, int A, int B,
                                  float gamma, int hard, float* weight, cudaStream_t s) {
-  return launch_pdl(erase_weights_kernel, (A + 7) / 8, 256, 0, s, logp_x, corpus_tok, argmax_t, row_mask, A, B,
-                                                   gamma, hard, weight);
+  return launch_pdl(erase_weights_kernel, (A + 7) / 8, 256, 0, s, logp_x, corpus_tok, argmax_t,
+                    row_mask, A, B, gamma, hard, weight);
 }
 
 }  // namespace alr
