@@ -34,8 +34,8 @@
  *              fill the device (any element type, in any process; partial sums added in a fixed
  *              order).
  *              ALR_LOSS_FORM = single (default) | mcast selects the fused loss kernels' form; mcast
- *              applies to problems on 256-column vocabulary tiles (not to a short contraction or
- *              too few tiles to fill the device) and changes neither results nor workspace sizes.
+ *              applies to kernels on 256-column vocabulary tiles (the width follows from the
+ *              sizes and the element type) and changes neither results nor workspace sizes.
  *              fp32 (tf32) products share no tiles: they run on single CTAs or split K.
  *              The cluster forms (mcast, mcast4, pair, and the loss kernels' mcast) are built
  *              into a second library, libalr_cluster.so, which this library loads from its own

@@ -172,9 +172,9 @@ int check_kept(const alr_params* p, const void* Z, const void* ref, const char* 
 // a multi-rank process, and then the single form runs).  The dual-product modes already share
 // each head tile between z_d and z_t, and at the power cap the multicast form settles ~4 %
 // lower in clock for ~1 % fewer L2 bytes per product: it is not faster, so it is not the
-// default.  It needs 256-column tiles: where loss_tile_columns takes 128, single CTAs run.  The tiles
-// and splits depend on the problem alone, so both forms give bit-identical results and take the
-// same workspace.
+// default.  It needs 256-column tiles: where loss_tile_columns takes 128, single CTAs run.  The
+// tiles and splits depend on the problem alone, so both forms give bit-identical results and take
+// the same workspace.
 bool loss_multicast(const alr_params* p) {
   if (p->dtype != ALR_BF16) return false;
   const char* v = getenv("ALR_LOSS_FORM");
@@ -186,16 +186,31 @@ enum PlanKind { kPlanFwd, kPlanReadout, kPlanTopk };
 // Vocabulary columns per tile.  256-column products read each operand byte from shared memory for
 // twice the work, but their two accumulators fill tensor memory, so a tile's epilogue (6000 to
 // 10000 cycles) is not hidden; 128-column tiles are double-buffered, their products slower.
-// Narrow tiles pay in the forwards up to 10 K blocks (4096 x d x 32000, us, 256 -> 128 columns: d =
-// 256 forward 202 -> 183, keeping 246 -> 225, readout 199 -> 179; d = 512 261 -> 258, 309 -> 289,
-// 232 -> 210; d = 1000 410 -> 460), and everywhere when wide ones would not give each SM a tile
-// (192 x 320 x 1400: forward 18.4 -> 17.2, gradient 7.4 -> 5.6; d = 3072 42 -> 32 and 30 -> 21).
+// `n_rb`: row blocks (pairs in the two-row modes).
+//   More wide tiles than SMs: narrow ones in the forwards up to 10 K blocks.  4096 x d x 32000,
+//   us, 256 -> 128 columns: bf16, d = 256 forward 182 -> 160, keeping 245 -> 225, readout 177 ->
+//   160; d = 512 239 -> 238, 310 -> 290, 211 -> 190; d = 640 270 -> 279, 341 -> 330, 227 -> 209;
+//   d = 1000 404 -> 448; fp32, d = 320 298 -> 303, 641 -> 615, 255 -> 238.  (One row block, whose
+//   W is read from memory once: 0.98 to 1.15 of the wide tiles' time.)
+//   Otherwise each SM has one tile at most, and a narrow one is half as long, as long as these too
+//   are at most one per SM (gradient of 16 x 3072 x 30000, 118 wide or 235 narrow tiles: 44 us
+//   wide, 66 narrow; of 512 x 3072 x 4096, 64 or 128: 30 and 21).  In a forward every tile is a
+//   split and its records cost the merge time: kMergeCycles a split against half a tile's cycles
+//   (16 x 3072 x 4096 41.7 -> 34.3 us; 128 x 1024 x 16000 32.5 -> 36.0, x 3072 52.6 -> 48.7).
+//   fp32 forwards have fewer splits than narrow tiles (forward_splits), so these only cost (512 x
+//   256 x 4096: 24.2 -> 26.8 us).
 constexpr int kNarrowBlocks = 10;
 
-int loss_tile_columns(const alr_params* p, int sms, bool bwd, int64_t n_rb) {
-  if (n_rb * ((p->V + 255) / 256) <= sms) return 128;
+int loss_tile_columns(const alr_params* p, int sms, bool bwd, PlanKind kind, int64_t n_rb) {
+  const int64_t n_wide = (p->V + 255) / 256, n_narrow = (p->V + 127) / 128;
   const int n_kb = (p->d + int(k_per_row(p->dtype)) - 1) / int(k_per_row(p->dtype));
-  return !bwd && n_kb <= kNarrowBlocks ? 128 : 256;
+  if (n_rb * n_wide > sms) return !bwd && n_kb <= kNarrowBlocks ? 128 : 256;
+  if (n_rb * n_narrow > sms) return 256;
+  if (bwd) return 128;
+  if (p->dtype == ALR_F32) return 256;
+  // cycles of a merged split (4, 2 and 2 records a row) and of a wide tile's epilogue
+  constexpr int64_t kMergeCycles[] = {380, 295, 150}, kEpilogue[] = {7000, 20000, 7000};
+  return 1090 * n_kb + kEpilogue[kind] > 2 * n_wide * kMergeCycles[kind] ? 128 : 256;
 }
 
 // Vocabulary splits of a forward over `rb` row blocks (row-block pairs in the two-row modes).
@@ -210,7 +225,7 @@ int loss_tile_columns(const alr_params* p, int sms, bool bwd, int64_t n_rb) {
 // 100000 1443 -> 1150, 8320 x 1024 x 32000 857 -> 760, 1920 x 4096 x 151936 2770 -> 2677; label
 // readout of 4096 x 2048 x 32000 533 -> 431.
 constexpr int64_t kPartBytes = 48ll << 20;
-constexpr int64_t kMaxRecordBytes = 4 * int64_t(sizeof(float)) * alr::kPFields;   // per row and split
+constexpr int64_t kMaxRecordBytes = 4 * int64_t(sizeof(float)) * alr::kPFields;   // row and split
 
 int forward_splits(const alr_params* p, int sms, int rb, int bn, int n_vt, int group,
                    PlanKind kind) {
@@ -222,9 +237,12 @@ int forward_splits(const alr_params* p, int sms, int rb, int bn, int n_vt, int g
   const int most = int(std::min<int64_t>(n_vt, std::max<int64_t>(1, fit)));
   const int base = std::min(most, round);
   // cycles of one tile: two 128 x 256 products over d (about 1090 per 64 of d) and an epilogue of
-  // about 7000, or half of both, overlapped, the products 30 % slower; a unit adds its first loads and its record, about 2500, and in the readout the
-  // filling of its top-8 lists, about 25000; a split adds its records' trip through memory (at
-  // about 2800 bytes a cycle)
+  // about 7000; a 128-column tile, its epilogue hidden, 0.65 of such products.  (Alone it takes 0.78
+  // of them at d = 1000 to 0.97 at 384, but that weight, 0.87, ranks the split counts worse, taking
+  // more of them: 1088 x 640 x 60000 152 -> 159 us, 4320 x 512 x 60000 453 -> 461; 6784 x 640 x
+  // 1400 53 -> 51.)  A unit adds its first loads and its record, about 2500, and in the
+  // readout the filling of its top-8 lists, about 25000; a split adds its records' trip through
+  // memory (at about 2800 bytes a cycle).
   const double products = 1090.0 * ((p->d + 63) / 64) * (p->dtype == ALR_BF16 ? 1 : 2);
   const double tile = bn == 256 ? products + 7000.0 : std::max(0.65 * products, 4500.0);
   const double per_unit = (kind == kPlanReadout ? 27500.0 : 2500.0) / tile;
@@ -261,7 +279,7 @@ alr::LossPlan loss_plan(const alr_params* p, int sms, bool bwd, PlanKind kind = 
   // forms), in raster groups of up to two rounds of the grid at its base split (16 row blocks).
   // Recomputing backward: one vocabulary tile per unit, raster groups of 16 row blocks as well.
   const int rb = int((p->N + 127) / 128);
-  P.bn = loss_tile_columns(p, sms, bwd, two_rows ? (rb + 1) / 2 : rb);
+  P.bn = loss_tile_columns(p, sms, bwd, kind, two_rows ? (rb + 1) / 2 : rb);
   P.mc = !two_rows && P.bn == 256 && loss_multicast(p) ? 1 : 0;
   const bool pairs = P.mc || two_rows;
   P.n_rb = pairs ? (rb + 1) / 2 : rb;
@@ -443,8 +461,8 @@ uint32_t gemm_b_rows(const GemmChoice& c) {
 
 // Up to this K the accumulating products are bound by the traffic of C, which the L2 prefetch helps
 // (dW at d = 4096, V = 151936, with two pieces ahead: K = 128 1060 -> 968 us, 512 1091 -> 1079);
-// beyond, it only competes with the operands' loads (1024: 1206 -> 1226, 1920: 1691 -> 1780).  With a tile or two per CTA
-// there is nothing to run ahead of.
+// beyond, it only competes with the operands' loads (1024: 1206 -> 1226, 1920: 1691 -> 1780).
+// With a tile or two per CTA there is nothing to run ahead of.
 constexpr int kPrefetchK = 512;
 
 alr::GemmArgs gemm_plan(int M, int Nc, int K, float* C, int64_t ldc, int sms) {

@@ -481,11 +481,16 @@ def test_loss_kernel_forms_agree_bit_for_bit(N, d, V, monkeypatch):
 
 # (A, B, d, V): 256-column tiles (11 K blocks and more tiles than SMs, also counted over pairs of
 # row blocks) with edges everywhere: the last tile 8 or 248 columns wide, a K tail, a last row block
-# of 1 to 127 rows, an odd number of row blocks, anchors across row blocks
+# of 1 to 127 rows, an odd number of row blocks, anchors across row blocks.  The last three have fewer
+# tiles than SMs: more narrow ones than SMs; few enough, but the merge of their records costs more
+# than they save; fp32
 @pytest.mark.parametrize("dtype,A,B,d,V", [(torch.bfloat16, 43, 3, 648, 39176),
                                            (torch.bfloat16, 17, 15, 712, 39160),
                                            (torch.bfloat16, 257, 1, 696, 19704),
-                                           (torch.float32, 24, 16, 328, 20248)])
+                                           (torch.float32, 24, 16, 328, 20248),
+                                           (torch.bfloat16, 2, 8, 72, 30008),
+                                           (torch.bfloat16, 8, 16, 64, 16008),
+                                           (torch.float32, 16, 8, 40, 4104)])
 def test_wide_tiles_at_their_edges(dtype, A, B, d, V):
     """The fused kernels' 256-column tiles at ragged sizes, which the smaller parity shapes run on
     128 columns: forward (kept and not), both logit gradients, dH, dW, against the oracle."""
