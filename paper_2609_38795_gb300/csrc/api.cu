@@ -391,7 +391,10 @@ struct GemmChoice {
 //           B is read once per pair.  It draws more power per product, though: at
 //           the text8b size (4.1e13 flop per product, the step at the power cap throughout) dH
 //           and dW gain 1.5 ms and the forward behind them loses 5, 102.5 -> 106.1 ms per step;
-//           at 1.0e13 the step gains 1 %, at 2.4e12 4 %, at 5.4e11 5 %.  So: up to kPairFlops.
+//           at 1.0e13 the step gains 1 %, at 2.4e12 4 %, at 5.4e11 5 %.  So: up to kPairFlops,
+//           where it turns (step at d = 4096, V = 151936, ms, mcast -> pair: 8192 rows, 1.0e13 flop
+//           a product, 26.7 -> 26.4; 12288, 1.5e13, 40.1 -> 40.5; 16384 53.2 -> 54.2; 24576 80.2 ->
+//           81.9).
 //   mcast   35.5 per K block; single 42, but no cluster has to be placed and an odd row block
 //           leaves no CTA idle (128 x 32000 x 512: 9.4 against 15.4 us).
 //   split   few tiles, long K: `split` CTAs per tile fill SMs that would idle.  128 x 4096 x
