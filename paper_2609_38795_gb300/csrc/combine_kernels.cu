@@ -42,7 +42,8 @@ ALR_DEV double add_part(double acc, float f, float s, float c) {
 // The row's sums carry the factor 2^r of its maximum m (exp_residual): the sum divided by it, and
 // its natural logarithm.  With x = r ln 2, 1 - x + x^2 / 2 leaves x^3 / 6, 5e-9 at |r| = 4e-3
 // (the fp16 range of logits) and 1e-14 at 6e-5 (|logit| < 1000).
-ALR_DEV double ln_residual(float m) { return double(exp_residual(m)) * 0.6931471805599453; }
+constexpr double kLn2Double = 0.6931471805599453;
+ALR_DEV double ln_residual(float m) { return double(exp_residual(m)) * kLn2Double; }
 ALR_DEV double without_residual(double s, float m) {
   const double x = ln_residual(m);
   return s * (1.0 - x + 0.5 * x * x);
@@ -101,15 +102,16 @@ struct FullState {
     zx = quiet_nan();
     id = it = 0x7fffffff;
   }
-  // u and w are measured from their part's maxima (z_d - md, z_t - mt): moved to the row's.
+  // u and w are measured from their part's maxima ((z_d - md) log2 e, (z_t - mt) log2 e): moved to
+  // the row's.
   ALR_DEV void add(const Record& o, const float (&ref)[kRefs]) {
     if (!(o.mt > -INFINITY)) return;       // no columns
     const float dd = ref_step(o.md, -ref[0] * kLog2e), dt = ref_step(o.mt, -ref[1] * kLog2e);
     const float ft = ex2(dt);
     sd = add_part(sd, ex2(dd), o.sd, o.cd);
     st = add_part(st, ft, o.st, o.ct);
-    u = fmaf(ft, fmaf(dd * kLn2, o.st, o.u), u);
-    w = fmaf(ft, fmaf(dt * kLn2, o.st, o.w), w);
+    u = fmaf(ft, fmaf(dd, o.st, o.u), u);
+    w = fmaf(ft, fmaf(dt, o.st, o.w), w);
     merge_top2(bd, secd, id, o.md, o.secd, o.id);
     merge_top2(bt, sect, it, o.mt, o.sect, o.it);
     if (o.zx == o.zx) zx = o.zx;
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
     const FullState st = sm.get(0, sr);
     const int r = row0 + sr;
     const double ls = log(side == 0 ? st.sd : st.st);
-    const double x = double(side == 0 ? st.u : st.w);
+    const double x = double(side == 0 ? st.u : st.w) * kLn2Double;
     const float v = float(ls - x / st.st);
     const float m = side == 0 ? st.bd : st.bt;
     const float lse = m + float(ls - ln_residual(m));

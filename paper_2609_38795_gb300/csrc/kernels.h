@@ -38,8 +38,8 @@ enum PartField {
   kPSd,       // sum exp(z_d - m_d)
   kPMt,       // max of z_t
   kPSt,       // sum exp(z_t - m_t)
-  kPU,        // sum exp(z_t - m_t) * (z_d - m_d)
-  kPW,        // sum exp(z_t - m_t) * (z_t - m_t)
+  kPU,        // sum exp(z_t - m_t) * (z_d - m_d) log2 e
+  kPW,        // sum exp(z_t - m_t) * (z_t - m_t) log2 e
   kPId,       // index of the maximum of z_d (int bits)
   kPSecd,     // second-best z_d (any other index)
   kPIt,

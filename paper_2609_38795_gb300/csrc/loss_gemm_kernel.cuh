@@ -309,7 +309,7 @@ ALR_DEV void stats_sub(RowStats& st, const uint32_t (&rd)[16], const uint32_t (&
   const float nbt = fmaxf(st.best_t, ct), nbd = fmaxf(st.best_d, cd);
   const float bt = -nbt * kLog2e, bd = -nbd * kLog2e;
   // per column: T = (z_t - nbt) log2 e, D = (z_d - nbd) log2 e, E = 2^T; sums of E, 2^D,
-  // E D and E T (the last two in log2 units, converted once below)
+  // E D and E T (the last two, like u and w, in units of ln 2)
   float s0 = 0.f, s1 = 0.f, d0 = 0.f, d1 = 0.f, u0 = 0.f, u1 = 0.f, w0 = 0.f, w1 = 0.f;
   if constexpr (kFull) {
     // even / odd columns in the two lanes of packed registers
@@ -346,11 +346,11 @@ ALR_DEV void stats_sub(RowStats& st, const uint32_t (&rd)[16], const uint32_t (&
   // reference is still -inf), rescale, add this sub-chunk
   const bool any = st.s_t > 0.f;
   const float step_t = ref_step(st.best_t, bt), step_d = ref_step(st.best_d, bd);
-  const float u_sh = any ? fmaf(step_d * kLn2, st.s_t + st.c_t, st.u) : 0.f;
-  const float w_sh = any ? fmaf(step_t * kLn2, st.s_t + st.c_t, st.w) : 0.f;
+  const float u_sh = any ? fmaf(step_d, st.s_t + st.c_t, st.u) : 0.f;
+  const float w_sh = any ? fmaf(step_t, st.s_t + st.c_t, st.w) : 0.f;
   const float sct = ex2(step_t), scd = ex2(step_d);
-  st.u = fmaf(u_sh, sct, (u0 + u1) * kLn2);
-  st.w = fmaf(w_sh, sct, (w0 + w1) * kLn2);
+  st.u = fmaf(u_sh, sct, u0 + u1);
+  st.w = fmaf(w_sh, sct, w0 + w1);
   sum2_scaled(st.s_t, st.c_t, sct, s0 + s1);
   sum2_scaled(st.s_d, st.c_d, scd, d0 + d1);
   // greedy top-2 of both sides (moves best_d / best_t to the new maxima nbd / nbt)
