@@ -71,6 +71,7 @@ struct FullState {
   int id, it;
 
   static constexpr int kWords = 13, kRefs = 2;
+  static constexpr bool kLongAdd = false;
   static ALR_DEV constexpr int ref_field(int i) { return i == 0 ? kPMd : kPMt; }
 
   struct Record {
@@ -150,6 +151,7 @@ struct ReadoutState {
   int ti[kTopK];
 
   static constexpr int kWords = 3 + 2 * kTopK, kRefs = 1;
+  static constexpr bool kLongAdd = true;    // a merge of two lists
   static ALR_DEV constexpr int ref_field(int) { return kRM; }
 
   struct Record {
@@ -211,6 +213,7 @@ struct TopkState {
   float z[kTopK];               // z_d at the label tokens, NaN until their column is met
 
   static constexpr int kWords = 7 + kTopK, kRefs = 1;
+  static constexpr bool kLongAdd = false;
   static ALR_DEV constexpr int ref_field(int) { return kKM; }
 
   struct Record {
@@ -332,13 +335,28 @@ ALR_DEV void merge_rows(const LossPlan& P, const float* part, int row0, int n_ro
 
   St st;
   st.init();
-  if (any) st.add(first, ref);
-  if (rr < n_rows) {
+  if constexpr (St::kLongAdd) {
+    // one copy of the long add, the next record on its way meanwhile
+    if (any) {
+#pragma unroll 1
+      for (int k = k0;;) {
+        const typename St::Record o = first;
+        k += step;
+        const bool more = k < P.n_parts;
+        if (more) first.load(col + size_t(k) * size_t(P.N), fs);
+        st.add(o, ref);
+        if (!more) break;
+      }
+    }
+  } else {
+    if (any) st.add(first, ref);
+    if (rr < n_rows) {
 #pragma unroll 2
-    for (int k = k0 + step; k < P.n_parts; k += step) {
-      typename St::Record o;
-      o.load(col + size_t(k) * size_t(P.N), fs);
-      st.add(o, ref);
+      for (int k = k0 + step; k < P.n_parts; k += step) {
+        typename St::Record o;
+        o.load(col + size_t(k) * size_t(P.N), fs);
+        st.add(o, ref);
+      }
     }
   }
 #pragma unroll
