@@ -63,8 +63,9 @@ ALR_DEV void merge_top2(float& best, float& sec, int& id, float best2, float sec
 // ------------------------------------------------------------------ row states ---
 // A state holds sums measured from the row's maxima over all records (`ref`, kRefs of them, found
 // first), so that every record's sums are multiplied by one factor, whatever the order of the
-// merge.  kWords: its 32-bit words, without padding.  init() is a row with no columns, Record one partial record (field stride fs), add()
-// folds a record in, merge() another state of the same row.
+// merge.  kWords: its 32-bit words, without padding.  init() is a row with no columns, Record one
+// partial record (field stride fs), add() folds a record in, merge() another state of the same
+// row.
 struct FullState {
   double sd, st;
   float u, w, bd, secd, bt, sect, zx;
@@ -622,24 +623,35 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
 }
 
 // ------------------------------------------------------------------ launch shape ---
-// Enough 32-row blocks to fill the device twice over: 32 rows and 8 warps per block, whose record
-// reads are whole 128-byte lines.  Fewer: the smallest of 8, 16 or 32 rows that holds a whole
-// anchor, with 16 warps over the records (32 warps leave a thread 64 registers and spill).
-constexpr int kReadoutFewRows = 1024;
-
+// The smallest of 8, 16 or 32 rows that holds a whole anchor and 16 warps over the records (32
+// warps leave a thread 64 registers and spill), as long as every such block has an SM; else 32 rows,
+// whose record reads are whole 128-byte lines, and 8 warps.  Forward and top-8 forward, us, first ->
+// second shape: 1920 x 64 x 151936 in anchors of 16 (120 blocks) 225 -> 226 and 153 -> 155; 4096 x
+// 64 x 60000 in anchors of 16 (256) 226 -> 219 and 158 -> 152; 1600 x 64 x 20000 in anchors of 8
+// (200) 51 -> 47 and 56 -> 50; 9000 x 64 x 20000 in anchors of 8 (1125) 197 -> 156 and 209 -> 153.
 struct MergeShape {
   int rows, warps, rows_per_block, blocks;
 };
 
 MergeShape merge_shape(int N, int B, int sms) {
-  const int per32 = 32 / B * B;
-  MergeShape m{32, 8, per32, (N + per32 - 1) / per32};
-  if (m.blocks >= 2 * sms) return m;
-  m.rows = B <= 8 ? 8 : B <= 16 ? 16 : 32;
-  m.warps = 16;
+  MergeShape m{B <= 8 ? 8 : B <= 16 ? 16 : 32, 16, 0, 0};
   m.rows_per_block = m.rows / B * B;
   m.blocks = (N + m.rows_per_block - 1) / m.rows_per_block;
-  return m;
+  if (m.blocks <= sms) return m;
+  const int per32 = 32 / B * B;
+  return MergeShape{32, 8, per32, (N + per32 - 1) / per32};
+}
+
+// The readout's rows are independent, and a merge of two top-8 lists costs several times a plain
+// record's, so with more rows fewer lanes share one: 64, 16 or 8 (us, 64 -> 16 -> 8 lanes: 768 x 64
+// x 151936 129 -> 133 -> 138; 1024 x 64 x 60000 93 -> 93 -> 98; 1920 x 64 x 151936 247 -> 231 ->
+// 234; 4096 x 64 x 60000 243 -> 204 -> 203; 9000 x 64 x 20000 243 -> 178 -> 168).
+constexpr int kReadoutFewRows = 1024;
+
+MergeShape readout_shape(int N, int sms) {
+  if (N < kReadoutFewRows) return MergeShape{8, 16, 8, (N + 7) / 8};
+  if ((N + 15) / 16 <= 2 * sms) return MergeShape{16, 8, 16, (N + 15) / 16};
+  return MergeShape{32, 8, 32, (N + 31) / 32};
 }
 
 }  // namespace
@@ -666,16 +678,10 @@ cudaError_t launch_readout_combine(const LossPlan& plan, const float* part, bool
                                    int32_t* top_idx, float* top_prob, float* tail, float* lse_t,
                                    int32_t* argmax_t, float* gap_t, float* logp_x,
                                    cudaStream_t s) {
-  // a merge of two top-8 lists costs several times a plain record's, so with more rows fewer lanes
-  // share one: 64, 16 from 1024 rows, 8 (readout with 16 instead of 64: 1920 x 64 x 151936 243 ->
-  // 229 us, 9000 x 64 x 20000 231 -> 191; 768 x 64 x 151936 130 -> 131)
-  MergeShape m = merge_shape(plan.N, 1, plan.sms);
-  auto kern = readout_combine_kernel<32, 8>;
-  if (m.rows < 32) {
-    const bool few = plan.N < kReadoutFewRows;
-    kern = few ? readout_combine_kernel<8, 16> : readout_combine_kernel<16, 8>;
-    m = few ? MergeShape{8, 16, 8, (plan.N + 7) / 8} : MergeShape{16, 8, 16, (plan.N + 15) / 16};
-  }
+  const MergeShape m = readout_shape(plan.N, plan.sms);
+  auto kern = m.rows == 8    ? readout_combine_kernel<8, 16>
+              : m.rows == 16 ? readout_combine_kernel<16, 8>
+                             : readout_combine_kernel<32, 8>;
   return launch_pdl(kern, m.blocks, 32 * m.warps, 0, s, plan, part, has_corpus ? 1 : 0, top_idx,
                     top_prob, tail, lse_t, argmax_t, gap_t, logp_x);
 }

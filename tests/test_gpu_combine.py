@@ -1,7 +1,7 @@
 """The merge of the forward's partial records (combine_kernels.cu) at the edges of its block
 shapes: 8, 16 or 32 rows per block by the anchor size, whole anchors per block, the last block
-partly filled, and the large-batch shape (at least 304 blocks of 32 rows), for the
-full-vocabulary forward, the label readout and the top-k forward, against the oracle."""
+partly filled, and the large-batch shape of 32 rows, for the full-vocabulary forward, the label
+readout and the top-k forward, against the oracle."""
 
 import numpy as np
 import pytest
@@ -25,10 +25,11 @@ def _lib():
 
 
 # (A, B): one row; a partial 8-row block; anchors of 3 and 8 in 8 rows; 9 and 16 in 16; 17 and
-# 32 in 32; the last shape of the small form (303 blocks of 30 rows) and the first of the large;
-# the two sides of the readout's choice of lanes per row
+# 32 in 32; many blocks of 30 and of 32 rows; the last shapes with a block per SM on 152 SMs (15 rows
+# each, 8 rows each) and the first beyond; the two sides of the readout's choices of lanes per row
 SHAPES = [(1, 1), (13, 1), (5, 3), (3, 8), (3, 9), (7, 16), (4, 17), (3, 32), (606, 15),
-          (607, 15), (9729, 1), (1023, 1), (1024, 1)]
+          (607, 15), (9729, 1), (1023, 1), (1024, 1), (152, 15), (153, 15), (1216, 1), (1217, 1),
+          (4865, 1)]
 
 
 @pytest.mark.parametrize("mode", [alr.ALR_MODE_ERASE_SOFT, alr.ALR_MODE_ERASE_HARD])
@@ -133,6 +134,10 @@ def test_sums_keep_their_precision_at_large_logits(N, d, V):
     out = P.gpu_forward(Hd, Ht, W, 16 if N % 16 == 0 else 8).out
     lab = T.gpu_readout(Ht, W, 16 if N % 16 == 0 else 8)
     ref["top_prob"] = p.gather(1, lab["top_idx"].long())
+    # the tail is S minus the eight largest terms over S: no term of S is off by more than 2^-21 of
+    # itself (its exponent's rounding and ex2.approx), so neither is the tail by more than that of 1
+    tail = p.scatter(1, lab["top_idx"].long(), 0.0).sum(1)
+    assert float((lab["tail"].double() - tail).abs().max()) <= 2.0 ** -21
     for k, x in ref.items():
         got = (lab if k == "top_prob" else out)[k].double()
         err = float((got - x).norm() / x.norm())
