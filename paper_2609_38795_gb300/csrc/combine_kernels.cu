@@ -39,15 +39,9 @@ ALR_DEV double add_part(double acc, float f, float s, float c) {
   return fma(f64, widen(s), fma(f64, widen(c), acc));
 }
 
-// The row's sums carry the factor 2^r of its maximum m (exp_residual): the sum divided by it, and
-// its natural logarithm.  With x = r ln 2, 1 - x + x^2 / 2 leaves x^3 / 6, 5e-9 at |r| = 4e-3
-// (the fp16 range of logits) and 1e-14 at 6e-5 (|logit| < 1000).
+// The row's sums carry the factor 2^r of its maximum m (exp_residual): its natural logarithm.
 constexpr double kLn2Double = 0.6931471805599453;
 ALR_DEV double ln_residual(float m) { return double(exp_residual(m)) * kLn2Double; }
-ALR_DEV double without_residual(double s, float m) {
-  const double x = ln_residual(m);
-  return s * (1.0 - x + 0.5 * x * x);
-}
 
 // Top-2 of two disjoint column sets; equal leaders go to the lower token id.
 ALR_DEV void merge_top2(float& best, float& sec, int& id, float best2, float sec2, int id2) {
@@ -550,18 +544,18 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
           ti = st.t[j];
           id = st.ti[j];
         }
-      const double e = exp(double(ti) - double(st.t[0]));
-      const double S = without_residual(st.s, st.t[0]);
+      // with the factor that S carries
+      const double e = exp(double(ti) - double(st.t[0]) + ln_residual(st.t[0]));
       s_e[i][rr] = e;
       top_idx[size_t(row0 + rr) * kTopK + i] = id;
-      top_prob[size_t(row0 + rr) * kTopK + i] = float(e / S);
+      top_prob[size_t(row0 + rr) * kTopK + i] = float(e / st.s);
     }
   }
   __syncthreads();
   if (int(threadIdx.x) < n_rows) {
     const int rr = threadIdx.x, r = row0 + rr;
     const ReadoutState st = sm.get(0, rr);
-    const double S = without_residual(st.s, st.t[0]), ls = log(S);
+    const double S = st.s, ls = log(S) - ln_residual(st.t[0]);
     double inside = 0.0;
 #pragma unroll
     for (int i = 0; i < kTopK; ++i) inside += s_e[i][rr];
@@ -597,7 +591,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 8 ? 2 : 1)
   if (int(threadIdx.x) < n_rows) {         // n_rows <= 32: the first warp
     const int s = threadIdx.x % P.B, r = row0 + threadIdx.x;
     const TopkState st = sm.get(0, threadIdx.x);
-    const double S = without_residual(st.s, st.best), ls = log(S);
+    const double ls = log(st.s) - ln_residual(st.best);
     // log q_i = (z_i - M) - log S: the difference z_i - M is exact in fp64
     double ce = 0.0;
 #pragma unroll
