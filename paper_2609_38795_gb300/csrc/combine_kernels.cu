@@ -7,10 +7,9 @@
 // record of it, the lanes of a row are then merged by shuffles and the warps through shared
 // memory, in a fixed order.  The row's maxima over all records are found first, so every record's
 // sums are multiplied by one factor only, and all sums of exponentials are held in fp64.  Bound by
-// latency (record loads) and, in few blocks, by the fp64 rate, so the split over records is what
-// sets its time: 31 us at 128 rows and 608 records (25 with two-float sums and the maxima moved
-// record by record, whose results were further from the fp64 reference), 16 us at 2000 rows and
-// 76 records, against 1087 us at 128 rows with one warp per anchor walking all records.
+// latency (record loads, three in flight per lane: 31 us with two at 128 rows and 608 records, 25
+// with three), so the split over records is what sets its time: 25 us there, 16 us at 2000 rows
+// and 76 records, against 1087 us at 128 rows with one warp per anchor walking all records.
 #include <cfloat>
 
 #include "kernels.h"
@@ -346,7 +345,7 @@ ALR_DEV void merge_rows(const LossPlan& P, const float* part, int row0, int n_ro
   } else {
     if (any) st.add(first, ref);
     if (rr < n_rows) {
-#pragma unroll 2
+#pragma unroll 3
       for (int k = k0 + step; k < P.n_parts; k += step) {
         typename St::Record o;
         o.load(col + size_t(k) * size_t(P.N), fs);
