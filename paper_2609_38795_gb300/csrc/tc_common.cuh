@@ -41,8 +41,8 @@ ALR_DEV float ex2(float x) {
 // The exponent every column gets relative to the reference m is fma(z, log2 e, b(m)) with
 // b(m) = -m log2 e rounded, which at z = m is not 0 but the rounding residual of m log2 e (exactly
 // representable, up to ~4e-6 at |m| ~ 40): every exponential summed against m carries the factor
-// 2^r, which is divided out of the row's sums, so that log S and the log-probabilities taken
-// from it keep their precision.
+// 2^r.  It cancels between a row's sums and is taken off where log S stands alone, so that the
+// log-probabilities keep their precision.
 ALR_DEV float exp_residual(float m) { return fmaf(m, kLog2e, -m * kLog2e); }
 
 // Exponent of the step from the reference m to one with b = b(nm), nm >= m: the difference of the
